@@ -231,13 +231,14 @@ struct PrologueArgs {
 // A projection's unit stream as the device code walks it.
 struct OpDesc {
   const uint8_t* units;
-  int n_rb, upr;
+  int n_rb;
+  int upr : 27;
   // Work split.  q = 0: the unit stream is cut into one contiguous run per
   // warp of the grid.  q > 0 (whole-step kernel, gate|up): row-block rb
   // belongs to one CTA, whose q warps take its units in q contiguous K
   // ranges and reduce them in shared memory (set only when every row-block
   // of the projection finds its CTA in one round).
-  int q;
+  int q : 5;
 };
 
 // Arguments of the whole-step kernel (step_kernel.cu).
@@ -253,26 +254,28 @@ struct StepKernelArgs {
   long long* acc_gu;         // [16][gate|up rows], zero between steps
   int* cnt_kv;               // [Hkv] q|k|v units finished per kv head, zero between steps
   int* cnt_gu;               // [gate|up row-blocks], zero between steps
-  uint16_t* act_h;           // [16][Kp_H] (normalised rows, when they do not fit in shared memory)
+  uint16_t* act_h;           // [16][Kp_H] normalised rows
   uint16_t* act_attn;        // [16][Kp_dq]
   uint16_t* act_f;           // [16][Kp_F]
   uint16_t* kpool;           // [L][n_rows][Hkv][cap][d]
   uint16_t* vpool;
   size_t layer_stride;
-  int cap, n_chunks;         // items per row at kAttnChunkMin entries (the partials layout)
+  int cap;
   const uint8_t* mask;
   int mask_stride;
   int packed;                // mask row per token (one request), no implicit causal bound
-  float* attn_part;          // [B][Hkv][n_chunks][16*G][d+4]
-  int* attn_cnt;             // [16][Hkv] finished chunks per (request, kv head); zero, self-resetting
+  float* attn_part;          // [item][16*G][d+4]; rows are cut into items only while every CTA has one at most
+  int* attn_cnt;             // [16][Hkv] finished chunks per (request, kv head), zero between steps
   int* status;
   unsigned long long* barrier;         // grid-barrier counter (monotonic)
   unsigned long long barrier_base;     // its value when this launch starts
   unsigned long long* phase_clock;     // [step_barriers(L) + 1] globaltimer at each barrier
   int* status_out;           // host-mapped mirror: the last CTA to finish copies a nonzero status there
+  int* norm_cnt;             // rows normalised so far in this launch (zero between launches)
   int* exit_count;           // CTAs finished in this launch (zero between launches; the last resets it)
   int debug_skip_arrival;    // test knob: >= 0 makes CTA 1 skip that grid barrier's arrival
   unsigned wait_limit;       // polls before a cross-CTA wait gives up
+  uint32_t area_bytes;       // shared memory for attention items and normalised rows (step_area_bytes)
   int gu_part;               // 1: shared memory holds the gate|up partial sums (OpDesc::q may be used)
 };
 // One-time attribute setup of the step kernel variants for a group size and
@@ -288,11 +291,13 @@ int step_gu_split(int n_rb, int upr, int grid, int group, int L);
 int step_gu_cta_tokens();
 // Whether the kernel's shared memory for L layers has room for the partial sums.
 bool step_gu_part_fits(int group, int L);
+// Shared memory of the attention / normalised-row area for steps of M tokens.
+size_t step_area_bytes(int group, int H, int L, bool part, int M);
 int step_barriers(int n_layers);
 cudaError_t launch_step(const StepKernelArgs& a, int nt, int group, int grid, cudaStream_t s);
-size_t step_attention_part_floats(int B, int Hkv, int n_chunks, int G, int d);
-constexpr int kAttnChunk = 64;     // most cache entries per attention item
-constexpr int kAttnChunkMin = 32;  // fewest (partials are laid out for this many per item)
+// Size of the attention partials for a grid of that many CTAs.
+size_t step_attention_part_floats(int grid, int G, int d);
+constexpr int kAttnChunkMin = 64;  // fewest cache entries per attention item
 
 // Weight repacking (one fused op; all source pointers device).
 // Source matrices of a fused op (q, k, v for OP_QKV; gate, up for OP_GU; one

@@ -104,6 +104,9 @@ struct shard_s {
   int* status = nullptr;           // device status word
   int* status_host = nullptr;      // host-mapped mirror the step kernel writes a nonzero status to
   int* status_host_dev = nullptr;  // its device address
+  int* norm_cnt = nullptr;         // step kernel: rows normalised (zero between launches)
+  bool gu_part = false;            // step kernel: gate|up partial sums in shared memory
+  uint32_t area_bytes[kMaxTokens + 1] = {};  // step kernel: shared-memory area per token count
   int* exit_count = nullptr;       // step kernel: CTAs finished (zero between launches)
   int grid[3] = {0, 0, 0};         // standalone GEMV grid per token bucket
   OpDesc* ops_dev = nullptr;       // [4L] op descriptors for the step kernel
@@ -131,7 +134,6 @@ struct kvstate_s {
   std::vector<int> cursor, len_host;
   bool shared = false;    // rows may share entries (a beam gather ran)
   bool poisoned = false;  // a step aborted on the device
-  int n_chunks = 0;       // attention items per row at the smallest item size (kAttnChunkMin)
   float* attn_part = nullptr;
 };
 
@@ -207,6 +209,7 @@ cudaError_t reset_work_buffers(shard_s* sh) {
   if (e == cudaSuccess) e = cudaMemset(sh->cnt_gu, 0, sizeof(int) * sh->n_rb_gu);
   if (e == cudaSuccess) e = cudaMemset(sh->cnt_store, 0, sizeof(int) * sh->max_rb);
   if (e == cudaSuccess) e = cudaMemset(sh->attn_cnt, 0, sizeof(int) * kMaxRequests * sh->Hkv);
+  if (e == cudaSuccess) e = cudaMemset(sh->norm_cnt, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(sh->exit_count, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(sh->barrier, 0, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -243,6 +246,7 @@ void release_shard(shard_s* sh) {
   cudaFree(sh->act_attn);
   cudaFree(sh->act_f);
   cudaFree(sh->status);
+  cudaFree(sh->norm_cnt);
   cudaFree(sh->exit_count);
   cudaFree(sh->dstage);
   if (sh->pin) cudaFreeHost(sh->pin);
@@ -454,6 +458,7 @@ int shard_create(const shard_config* cfg, const shard_weights_host* w, shard_t* 
   CUDA_TRY(cudaHostAlloc(&sh->status_host, sizeof(int), cudaHostAllocMapped));
   *sh->status_host = 0;
   CUDA_TRY(cudaHostGetDevicePointer(reinterpret_cast<void**>(&sh->status_host_dev), sh->status_host, 0));
+  CUDA_TRY(cudaMalloc(&sh->norm_cnt, sizeof(int)));
   CUDA_TRY(cudaMalloc(&sh->exit_count, sizeof(int)));
   CUDA_TRY(cudaMemset(sh->exit_count, 0, sizeof(int)));
   {
@@ -467,6 +472,9 @@ int shard_create(const shard_config* cfg, const shard_weights_host* w, shard_t* 
     CUDA_TRY(cudaMalloc(&sh->ops_dev, sizeof(OpDesc) * od.size()));
     CUDA_TRY(cudaMemcpy(sh->ops_dev, od.data(), sizeof(OpDesc) * od.size(), cudaMemcpyHostToDevice));
   }
+  sh->gu_part = step_gu_part_fits(sh->cfg.group, sh->L);
+  for (int m = 1; m <= kMaxTokens; ++m)
+    sh->area_bytes[m] = (uint32_t)step_area_bytes(sh->cfg.group, sh->H, sh->L, sh->gu_part, m);
   sh->n_barriers = step_barriers(sh->L);
   CUDA_TRY(cudaMalloc(&sh->barrier, sizeof(unsigned long long)));
   CUDA_TRY(cudaMalloc(&sh->phase_clock, sizeof(unsigned long long) * (sh->n_barriers + 1)));
@@ -496,7 +504,6 @@ int kv_state_alloc(shard_t sh, int n_rows, int capacity, kvstate_t* out) {
   const size_t pool = st->layer_stride * sh->L;
   st->cursor.assign(n_rows, 0);
   st->len_host.assign(n_rows, 0);
-  st->n_chunks = (capacity + kAttnChunkMin - 1) / kAttnChunkMin;
   int rc = SHARD_OK;
   auto chk = [&](cudaError_t e) {
     if (e != cudaSuccess && rc == SHARD_OK)
@@ -508,7 +515,7 @@ int kv_state_alloc(shard_t sh, int n_rows, int capacity, kvstate_t* out) {
   chk(cudaMalloc(&st->bt[1], sizeof(int) * (size_t)n_rows * capacity));
   chk(cudaMalloc(&st->lens, sizeof(int) * n_rows));
   const int G = sh->Hq / sh->Hkv;
-  chk(cudaMalloc(&st->attn_part, sizeof(float) * step_attention_part_floats(n_rows, sh->Hkv, st->n_chunks, G, sh->d)));
+  chk(cudaMalloc(&st->attn_part, sizeof(float) * step_attention_part_floats(sh->num_sms, G, sh->d)));
   if (rc == SHARD_OK) {
     chk(cudaMemset(st->lens, 0, sizeof(int) * n_rows));
     chk(cudaMemset(st->k, 0, sizeof(uint16_t) * pool));
@@ -810,13 +817,14 @@ static int step_impl(shard_t sh, kvstate_t st, const uint16_t* hidden_in, const 
   ka.vpool = st->v;
   ka.layer_stride = st->layer_stride;
   ka.cap = st->cap;
-  ka.n_chunks = st->n_chunks;
   ka.attn_part = st->attn_part;
   ka.attn_cnt = sh->attn_cnt;
   ka.status = sh->status;
   ka.debug_skip_arrival = sh->debug_skip_arrival;
   ka.wait_limit = sh->wait_limit;
-  ka.gu_part = step_gu_part_fits(sh->cfg.group, sh->L) ? 1 : 0;
+  ka.gu_part = sh->gu_part ? 1 : 0;
+  ka.area_bytes = sh->area_bytes[M];
+  ka.norm_cnt = sh->norm_cnt;
   ka.barrier = sh->barrier;
   ka.barrier_base = sh->barrier_base;
   ka.phase_clock = sh->phase_clock;

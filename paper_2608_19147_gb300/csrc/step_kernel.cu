@@ -17,8 +17,8 @@
 // The residual stream and the projections' sums are 64-bit fixed point
 // (kernels.h): contributors add with integer atomics and nobody waits for a
 // merge; results do not depend on the order of arrival.
-// Each RMSNorm is computed by every CTA at the start of the projection that
-// consumes it, from the whole residual (the same bits in every CTA).
+// Each RMSNorm runs at the start of the projection that consumes it: one row by
+// every CTA for itself, several by one CTA each.
 //
 // Every cross-CTA wait is bounded: a wait that runs out sets a status bit and
 // proceeds (the step's results are then reported invalid) instead of hanging.
@@ -34,33 +34,48 @@ namespace {
 constexpr int kWarps = kCtaWarps;           // consumer warps
 constexpr int kThreads = kWarps * 32;       // consumer threads
 constexpr int kBlockThreads = kThreads + (kSelfRefill ? 0 : 32);  // + the producer warp, if any
-constexpr int kChunk = kAttnChunk;  // most cache entries per attention item (kChunk / 32 per lane)
-constexpr bool kNormInSmem = true;   // normalised activations in shared memory when they fit
 // Polls of a busy slot before the producer gives up: a slot may legitimately
 // stay busy while its consumer works through a whole attention phase, so this
 // bound is fixed and far above any step's length.
 constexpr uint32_t kProducerLimit = 1u << 22;
 
-// The attention area: one item's tiles at kChunk entries and head_dim 128
-// (AttnSmem), rounded up to 1 KB; it also holds the normalised rows when they fit.
-constexpr size_t kAttnArea =
-    ((size_t)kChunk * (128 + 8) * 2 + (size_t)kChunk * 128 * 2 + 16 * 128 * 4 + 16 * kChunk * 4 + 2 * kChunk * 4 +
-     (size_t)kMaxTokens * kChunk + 1023) / 1024 * 1024;
+// Dynamic shared memory: weight rings, their barriers, the op table (4L
+// entries), gate|up partial sums (when they fit), and the area: an attention
+// item's (AttnSmem), which between attentions holds the normalised rows when
+// they fit.  The host sizes the area for the step's token count.
+constexpr size_t kAttnArea = 51 * 1024;  // at least: AttnSmem at head_dim 128, checked in the kernel
 
 template <int GPU>
 struct StepSmem {
   static constexpr int kSlots = Geom<GPU>::kStepSlots;
   static constexpr size_t kRing = (size_t)kWarps * kSlots * Geom<GPU>::kUnitBytes;
   static constexpr size_t kBars = (size_t)2 * kWarps * kSlots * sizeof(uint64_t);
-  // attention item area (AttnSmem), also the normalised rows
-  static constexpr size_t kQ = kAttnArea;
-  static constexpr size_t kFixed = kRing + kBars + kQ;  // + the op table (4L entries)
+  static constexpr size_t kOps = kRing + kBars;
   // gate|up partial sums of the shared-memory reduction (swiglu_cta_write)
   static constexpr size_t kPart = (size_t)kWarps * kGuCtaTokens * kRowsPerBlock * sizeof(float);
-  __host__ __device__ static size_t ops_bytes(int n_layers) { return ((size_t)4 * n_layers * sizeof(OpDesc) + 15) / 16 * 16; }
-  static size_t total(int n_layers) { return kFixed + ops_bytes(n_layers); }
-  static size_t total_with_part(int n_layers) { return total(n_layers) + kPart; }
+  // offset of the area
+  __host__ __device__ static size_t area(int n_layers, bool part) {
+    return (kOps + (size_t)4 * n_layers * sizeof(OpDesc) + (part ? kPart : 0) + 127) / 128 * 128;
+  }
+  static size_t total(int n_layers, bool part) { return area(n_layers, part) + kAttnArea; }
 };
+
+// Row stride (halves) of the normalised rows in shared memory: padded so that
+// the two token rows a fragment load touches in one phase fall on different
+// banks.
+__host__ __device__ constexpr int xn_stride(int H) { return H + 32; }
+// Bytes of M such rows, and of the one residual row staged behind them when M = 1.
+__host__ __device__ constexpr size_t xn_bytes(int H, int M) { return ((size_t)M * xn_stride(H) * 2 + 127) / 128 * 128; }
+__host__ __device__ constexpr size_t xn_stage_bytes(int H, int M) { return M == 1 ? (size_t)H * 8 : 0; }
+
+// The same value, which the compiler may not trace to where it came from.  The
+// phases of the layer loop start from such values: it would otherwise compute
+// their address parts before the loop and hold them in registers (or spill
+// them) through all the other phases.
+__device__ __forceinline__ int opaque(int v) {
+  asm volatile("" : "+r"(v));
+  return v;
+}
 
 // Barrier among the consumer warps of a CTA (the producer warp runs on its own).
 __device__ __forceinline__ void cbar() { named_bar_sync(1, kThreads); }
@@ -95,7 +110,8 @@ __device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned 
 // Grid-wide barrier on a monotonically increasing counter, in two halves so
 // that work may sit between arriving and waiting.  `target` is this CTA's
 // running count of expected arrivals.  Called by the consumer warps; the
-// caller has synchronised them (cbar) before grid_arrive.
+// caller has synchronised them (cbar) before grid_arrive.  Lives in shared
+// memory (only thread 0 uses it), so that it takes no registers of the phases.
 struct GridBarrier {
   unsigned long long* ctr;
   unsigned long long target;
@@ -108,8 +124,8 @@ struct GridBarrier {
   __device__ __forceinline__ void arrive() {
     if (threadIdx.x == 0) {
       if (!(blockIdx.x == 1 && n_arrive == skip_arrival)) red_release_add(ctr, 1ULL);
+      ++n_arrive;
     }
-    ++n_arrive;
   }
   __device__ __forceinline__ void wait() {
     if (threadIdx.x == 0) {
@@ -124,9 +140,8 @@ struct GridBarrier {
         if ((it & 1023) == 0 && (*reinterpret_cast<volatile int*>(status) & ST_WAIT_TIMEOUT)) break;
         __nanosleep(16);
       }
-      if (blockIdx.x == 0) clock[n_wait + 1] = globaltimer();
+      if (blockIdx.x == 0) clock[++n_wait] = globaltimer();
     }
-    ++n_wait;
     cbar();
   }
   __device__ __forceinline__ void sync() {
@@ -241,12 +256,18 @@ __device__ __noinline__ void prologue_work(const PrologueArgs& a, const StepPara
 }
 
 // ---------------------------------------------------------------------------
-// RMSNorm, run by every CTA at the start of the projection that consumes it:
+// RMSNorm at the start of the projection that consumes it:
 // r[m] = 1 / sqrt(mean(x[m]^2) + eps), act = fp16(x * r * w).  x is the
 // residual stream (fixed point) or, before the first layer, the step's fp16
-// input rows (the same values).  Two passes: the sums of squares (added in a
-// fixed order, so every CTA gets the same r), then the scaled rows; the first
-// row's pieces stay in registers between the passes.  H is a multiple of 4.
+// input rows (the same values).  H is a multiple of 4.
+//
+// A single row that fits is normalised by every CTA for itself
+// (rmsnorm_staged): one memory round trip and no hand-over.  Otherwise row m
+// is normalised by CTA m alone, and the others wait for the count of finished
+// rows and read the fp16 result: every CTA reading all M rows of 64-bit sums
+// (H * 8 bytes each, 39 MB over the chip for 8 rows of 4096) costs more than
+// that hand-over (8B width, norm + gate|up: 5 rows 26.6 -> 21.5 us, 8 rows
+// 40 -> 26, 16 rows 80 -> 39).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float4 norm_load(bool from_x, const long long* X, const uint16_t* const* rowp, int H, int m,
                                             int k) {
@@ -261,87 +282,53 @@ __device__ __forceinline__ float4 norm_load(bool from_x, const long long* X, con
   }
 }
 
-// kP pieces (float4) per row and thread are held in registers (the rest of a
-// longer row is streamed).  Rows go kR at a time, every piece of the kR rows
-// requested at once (one memory round trip per batch; the norm weights come
-// with the first).  When all M rows fit in one batch they stay in registers
-// for the second pass, so X is read once.
-template <int kP, int kR>
-__device__ __forceinline__ void rmsnorm_rows(bool from_x, const long long* X, const uint16_t* const* rowp, int H,
-                                             const uint16_t* w, float eps, uint16_t* out, int out_ld, int M) {
-  __shared__ float s_part[kWarps][kMaxTokens];
-  __shared__ float s_r[kMaxTokens];
+// Row m to `out` (fp16), counted in *done (release) if given.  kP pieces
+// (float4) per thread stay in registers between the sum of squares and the
+// scaling; the rest of a longer row is read twice.
+__device__ __forceinline__ void rmsnorm_row(bool from_x, const long long* X, const uint16_t* const* rowp, int H, int m,
+                                            const uint16_t* w, float eps, uint16_t* out, int* done) {
+  constexpr int kP = 6;
+  __shared__ float s_part[kWarps];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H4 = H / 4;
   uint2 wv[kP];
-  float4 v[kR][kP];
+  float4 v[kP];
 #pragma unroll
   for (int i = 0; i < kP; ++i) {
     const int c = tid + i * kThreads;
     wv[i] = c < H4 ? *reinterpret_cast<const uint2*>(w + 4 * c) : make_uint2(0, 0);
+    v[i] = c < H4 ? norm_load(from_x, X, rowp, H, m, 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  auto load_batch = [&](int m0) {
+  float t = 0.f;
 #pragma unroll
-    for (int h = 0; h < kR; ++h)
+  for (int i = 0; i < kP; ++i) t += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+  for (int c = tid + kP * kThreads; c < H4; c += kThreads) {
+    const float4 u = norm_load(from_x, X, rowp, H, m, 4 * c);
+    t += u.x * u.x + u.y * u.y + u.z * u.z + u.w * u.w;
+  }
 #pragma unroll
-      for (int i = 0; i < kP; ++i) {
-        const int c = tid + i * kThreads;
-        v[h][i] = c < H4 && m0 + h < M ? norm_load(from_x, X, rowp, H, m0 + h, 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) s_part[warp] = t;
+  cbar();
+  float u = 0.f;
+  for (int w8 = 0; w8 < kWarps; ++w8) u += s_part[w8];
+  const float r = rsqrtf(u / H + eps);
+  auto emit = [&](int c, float4 x, uint2 wq) {
+    const float2 w01 = h2f2(wq.x), w23 = h2f2(wq.y);
+    uint2 o;
+    o.x = pack_h2(x.x * r * w01.x, x.y * r * w01.y);
+    o.y = pack_h2(x.z * r * w23.x, x.w * r * w23.y);
+    *reinterpret_cast<uint2*>(out + 4 * c) = o;
   };
-  for (int m0 = 0; m0 < M; m0 += kR) {
-    load_batch(m0);
-    float t[kR];
 #pragma unroll
-    for (int h = 0; h < kR; ++h) {
-      t[h] = 0.f;
-#pragma unroll
-      for (int i = 0; i < kP; ++i)
-        t[h] += v[h][i].x * v[h][i].x + v[h][i].y * v[h][i].y + v[h][i].z * v[h][i].z + v[h][i].w * v[h][i].w;
-      if (m0 + h < M)
-        for (int c = tid + kP * kThreads; c < H4; c += kThreads) {
-          const float4 u = norm_load(from_x, X, rowp, H, m0 + h, 4 * c);
-          t[h] += u.x * u.x + u.y * u.y + u.z * u.z + u.w * u.w;
-        }
-    }
-#pragma unroll
-    for (int h = 0; h < kR; ++h) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t[h] += __shfl_xor_sync(0xffffffffu, t[h], o);
-      if (lane == 0 && m0 + h < M) s_part[warp][m0 + h] = t[h];
-    }
+  for (int i = 0; i < kP; ++i) {
+    const int c = tid + i * kThreads;
+    if (c < H4) emit(c, v[i], wv[i]);
   }
+  for (int c = tid + kP * kThreads; c < H4; c += kThreads)
+    emit(c, norm_load(from_x, X, rowp, H, m, 4 * c), *reinterpret_cast<const uint2*>(w + 4 * c));
   cbar();
-  if (tid < M) {
-    float t = 0.f;
-    for (int w8 = 0; w8 < kWarps; ++w8) t += s_part[w8][tid];
-    s_r[tid] = rsqrtf(t / H + eps);
-  }
-  cbar();
-  for (int m0 = 0; m0 < M; m0 += kR) {
-    if (M > kR) load_batch(m0);  // else the one batch is still in registers
-#pragma unroll
-    for (int h = 0; h < kR; ++h) {
-      const int m = m0 + h;
-      if (m >= M) break;
-      const float r = s_r[m];
-      auto emit = [&](int c, float4 x, uint2 wq) {
-        const float2 w01 = h2f2(wq.x), w23 = h2f2(wq.y);
-        uint2 o;
-        o.x = pack_h2(x.x * r * w01.x, x.y * r * w01.y);
-        o.y = pack_h2(x.z * r * w23.x, x.w * r * w23.y);
-        *reinterpret_cast<uint2*>(out + (size_t)m * out_ld + 4 * c) = o;
-      };
-#pragma unroll
-      for (int i = 0; i < kP; ++i) {
-        const int c = tid + i * kThreads;
-        if (c < H4) emit(c, v[h][i], wv[i]);
-      }
-      for (int c = tid + kP * kThreads; c < H4; c += kThreads)
-        emit(c, norm_load(from_x, X, rowp, H, m, 4 * c), *reinterpret_cast<const uint2*>(w + 4 * c));
-    }
-  }
-  cbar();
+  if (done && tid == 0) red_release_add_s32(done, 1);
 }
 
 // One row from the residual stream (M = 1, H <= 24 * kThreads) through
@@ -349,7 +336,7 @@ __device__ __forceinline__ void rmsnorm_rows(bool from_x, const long long* X, co
 // (`stage`, 16-byte aligned, H * 8 bytes; completion on `bar`, whose phase
 // the caller tracks), so the read runs at copy-engine bandwidth instead of
 // being bounded by each thread's loads in flight; both passes then read
-// shared memory.  The values and the arithmetic are those of rmsnorm_rows.
+// shared memory.  The values and the arithmetic are those of rmsnorm_row.
 __device__ __forceinline__ void rmsnorm_staged(const long long* X, int H, const uint16_t* w, float eps, uint16_t* out,
                                                long long* stage, uint64_t* bar, uint32_t& phase, int* status) {
   constexpr int kP = 6;
@@ -414,32 +401,50 @@ __device__ __forceinline__ void rmsnorm_staged(const long long* X, int H, const 
   cbar();
 }
 
-// Rows of up to 3 pieces per thread (H <= 4608) go three at a time; longer
-// rows two at a time with 6 pieces in registers.  from_x: the residual
-// stream, else the step's fp16 input rows (before the first layer).
-__device__ __forceinline__ void rmsnorm_cta(bool from_x, const long long* X, const uint16_t* const* rowp, int H,
-                                            const uint16_t* w, float eps, uint16_t* out, int out_ld, int M) {
-  if (H / 4 <= 3 * kThreads)
-    rmsnorm_rows<3, 3>(from_x, X, rowp, H, w, eps, out, out_ld, M);
-  else
-    rmsnorm_rows<6, 2>(from_x, X, rowp, H, w, eps, out, out_ld, M);
-}
-
 // ---------------------------------------------------------------------------
 // Attention.  Item = (request b, kv head hk, chunk c of cs entries); one CTA
-// per item, items dealt round-robin.  cs is the smallest of 32, 64, 128 that
-// gives no more items than CTAs (short caches: more parallel items), else 128
-// (long caches: fewer rounds and merges).  Each item writes (max, sum of exp,
-// unnormalised output) per query (the request's new tokens x the kv head's
-// query heads).  With several items per CTA, after its items the CTA that
-// took the last chunk of (b, hk) waits for the chunk count and combines the
-// chunks in order, so the merges are spread over CTAs and never delay
-// anyone's items; with one item per CTA at most, the CTA that finishes the
-// last chunk merges at once.
+// per item.  cs is the smallest multiple of 16, from kAttnChunkMin up, that
+// gives no more items than CTAs; when there are more (request, kv head) pairs
+// than CTAs, an item is a whole row and CTAs take several.
+//
+// The bound is the K/V stream (32 KB per 64 entries of a head at d = 128, each
+// byte read once) and, for short caches, the chain of dependent L2 round
+// trips.  Both products run on mma.sync straight from registers:
+//   - a warp takes blocks of 16 entries; a lane's K fragment is 16 consecutive
+//     bytes of an entry's row (the head dimension is summed in that order on
+//     both sides), its V fragment the same 16 bytes of four entries,
+//     interleaved by byte permutes, so K and V go from global memory to the
+//     tensor cores without passing through shared memory, and every warp
+//     keeps its next block's rows in flight while it works on the last;
+//   - queries go in tiles of 8: a tile's 16 MMA rows are the 8 queries' fp16
+//     values and what that rounding left out (after scaling each query by a
+//     power of two to a largest value in [1, 2)), so the scores carry an fp32
+//     query at one MMA per tile; probabilities (times 2^12) are split the
+//     same way for the value sum.  Sums are fp32, the softmax is online per
+//     warp.
+// A warp holds one query tile; kWarps / tiles warps side by side take different
+// blocks (a tile's blocks meet the other tiles' reads of them in L1), and the
+// CTA adds their pieces in shared memory in a fixed order.  Two tiles per warp
+// would halve the L1 reads, but their accumulators and the rows in flight do
+// not fit 168 registers.  Chunks of one
+// (request, kv head) meet in `part`: the CTA that finishes the last one merges
+// when that is little to read, else every chunk's CTA waits for the others
+// and merges its share of the queries.
+//
+// First layer's attention phase, against the CUDA-core version before it (a warp
+// per query over 64-entry tiles in shared memory, a CTA's items one after
+// another): 70B width, 4096 entries, 1 token 38 -> 18 us, 5 tokens 113 -> 32;
+// 8B width, 8 requests of 128..2048 entries 69 -> 23, 16 packed tokens over
+// 1024 entries 73 -> 28, 5 tokens over 512 entries 20 -> 15, 1 token over 72..327
+// entries 9 -> 9 (there it is the latency of the waits).
 // ---------------------------------------------------------------------------
 // A partial is (max, sum of exp, 2 unused, unnormalised output[d]): the
 // output starts 16-byte aligned.
 __host__ __device__ constexpr int part_stride(int d) { return d + 4; }
+
+constexpr int kAttnQ = 64;        // queries per pass over an item's entries
+constexpr int kAttnWin = 1024;    // entries whose slots and visibility are staged at a time
+constexpr float kProbScale = 4096.f;
 
 struct AttnView {
   const long long* acc;     // q|k|v sums [16][acc_ld] (fixed point), GPU row order
@@ -448,8 +453,8 @@ struct AttnView {
   uint16_t* kpool;          // layer 0; layer l at + l * layer_stride
   uint16_t* vpool;
   size_t layer_stride;
-  int cap, Hq, Hkv, d, n_chunks, qmax;
-  float* part;
+  int cap, Hq, Hkv, d, qmax;
+  float* part;              // [item][16 * G queries][d + 4]
   int* cnt;                 // finished chunks per (request, kv head)
   const int* cnt_kv;        // q|k|v units finished per kv head
   int kv_units;             // units per kv head when its q|k|v rows are complete
@@ -457,8 +462,8 @@ struct AttnView {
   const uint8_t* mask;
   int mask_stride;
   int packed;               // a mask row per token of request 0 instead of one per request
-  int cs;                   // entries per item this step: 32, 64 or 128 (kChunk)
-  int last_merges;          // at most one item per CTA: the CTA finishing the last chunk merges at once
+  int cs;                   // entries per item this step
+  int total;                // items this step
   uint32_t limit;
   uint16_t* out;
   int out_ld;
@@ -466,93 +471,51 @@ struct AttnView {
 
 __device__ __forceinline__ int n_chunks_of(int L, int cs) { return (L + cs - 1) / cs; }
 
-// Finds the item's (b, hk, c) from a flat index; false if past the end.
-__device__ __forceinline__ bool decode_item(const StepParams* sp, int Hkv, int cs, int item, int& b, int& hk, int& c) {
-  for (b = 0; b < sp->B; ++b) {
+// The step's item size and count (one warp; lane b takes request b).
+__device__ __forceinline__ void attn_plan(const StepParams* sp, int Hkv, int grid, int lane, int& cs, int& total) {
+  const int L = lane < sp->B ? sp->req_len[lane] : 0;
+  const unsigned all = 0xffffffffu;
+  const int longest = __reduce_max_sync(all, L), sum = __reduce_add_sync(all, L);
+  cs = max(kAttnChunkMin, (int)(((long long)sum * Hkv + grid - 1) / grid + 15) / 16 * 16);
+  // rounding up per row can need a little more than the even share
+  while (cs < longest) {
+    total = Hkv * __reduce_add_sync(all, n_chunks_of(L, cs));
+    if (total <= grid) return;
+    cs += 16 * max(1, cs / 256);
+  }
+  cs = longest;
+  total = Hkv * sp->B;
+}
+
+// Finds the item's (b, hk, c) from a flat index.
+__device__ __forceinline__ void decode_item(const StepParams* sp, int Hkv, int cs, int item, int& b, int& hk, int& c) {
+  hk = c = 0;
+  for (b = 0; b < sp->B - 1; ++b) {
     const int per = Hkv * n_chunks_of(sp->req_len[b], cs);
-    if (item < per) {
-      hk = item / n_chunks_of(sp->req_len[b], cs);
-      c = item % n_chunks_of(sp->req_len[b], cs);
-      return true;
-    }
+    if (item < per) break;
     item -= per;
   }
-  return false;
+  const int nc = n_chunks_of(sp->req_len[b], cs);
+  hk = item / nc;
+  c = item - hk * nc;
 }
 
-// q (fp32, shared) . K row (fp16, shared) over KP 8-element pieces; the
-// two-row form scores rows k0 and k1 with one pass over q.
-__device__ __forceinline__ float dot_q_k(const float* qq, const uint16_t* k0r, int KP) {
-  float s0 = 0.f;
-#pragma unroll 4
-  for (int t = 0; t < KP; ++t) {
-    const uint4 k0 = *reinterpret_cast<const uint4*>(k0r + t * 8);
-    const float4 qa = *reinterpret_cast<const float4*>(qq + t * 8);
-    const float4 qb = *reinterpret_cast<const float4*>(qq + t * 8 + 4);
-    float2 f = h2f2(k0.x);
-    s0 = fmaf(qa.x, f.x, s0);
-    s0 = fmaf(qa.y, f.y, s0);
-    f = h2f2(k0.y);
-    s0 = fmaf(qa.z, f.x, s0);
-    s0 = fmaf(qa.w, f.y, s0);
-    f = h2f2(k0.z);
-    s0 = fmaf(qb.x, f.x, s0);
-    s0 = fmaf(qb.y, f.y, s0);
-    f = h2f2(k0.w);
-    s0 = fmaf(qb.z, f.x, s0);
-    s0 = fmaf(qb.w, f.y, s0);
-  }
-  return s0;
-}
-__device__ __forceinline__ float dot_q_k2(const float* qq, const uint16_t* k0r, const uint16_t* k1r, float& s1,
-                                          int KP) {
-  float s0 = 0.f;
-  s1 = 0.f;
-#pragma unroll 4
-  for (int t = 0; t < KP; ++t) {
-    const uint4 k0 = *reinterpret_cast<const uint4*>(k0r + t * 8);
-    const uint4 k1 = *reinterpret_cast<const uint4*>(k1r + t * 8);
-    const float4 qa = *reinterpret_cast<const float4*>(qq + t * 8);
-    const float4 qb = *reinterpret_cast<const float4*>(qq + t * 8 + 4);
-    float2 f = h2f2(k0.x), g = h2f2(k1.x);
-    s0 = fmaf(qa.x, f.x, s0);
-    s0 = fmaf(qa.y, f.y, s0);
-    s1 = fmaf(qa.x, g.x, s1);
-    s1 = fmaf(qa.y, g.y, s1);
-    f = h2f2(k0.y);
-    g = h2f2(k1.y);
-    s0 = fmaf(qa.z, f.x, s0);
-    s0 = fmaf(qa.w, f.y, s0);
-    s1 = fmaf(qa.z, g.x, s1);
-    s1 = fmaf(qa.w, g.y, s1);
-    f = h2f2(k0.z);
-    g = h2f2(k1.z);
-    s0 = fmaf(qb.x, f.x, s0);
-    s0 = fmaf(qb.y, f.y, s0);
-    s1 = fmaf(qb.x, g.x, s1);
-    s1 = fmaf(qb.y, g.y, s1);
-    f = h2f2(k0.w);
-    g = h2f2(k1.w);
-    s0 = fmaf(qb.z, f.x, s0);
-    s0 = fmaf(qb.w, f.y, s0);
-    s1 = fmaf(qb.z, g.x, s1);
-    s1 = fmaf(qb.w, g.y, s1);
-  }
-  return s0;
-}
-
-// Shared-memory layout of one attention item.
+// Shared-memory layout of one attention item.  Query rows are padded so that
+// the two rows of a quarter-warp's 16-byte loads fall on different banks.
 template <int DPL>
 struct AttnSmem {
   static constexpr int d = 32 * DPL;
-  static constexpr int kKld = d + 8;  // padded K row (halves): consecutive rows start on different banks
-  static constexpr int kQg = 16;      // queries per group
-  static constexpr size_t kK = (size_t)kChunk * kKld * 2;
-  static constexpr size_t kV = (size_t)kChunk * d * 2;
-  static constexpr size_t kQ = (size_t)kQg * d * 4;
-  static constexpr size_t kP = (size_t)kQg * kChunk * 4;
-  static constexpr size_t kVisT = (size_t)kMaxTokens * kChunk;  // packed mode: [token][entry] mask bytes
-  static constexpr size_t kBytes = kK + kV + kQ + kP + 2 * kChunk * sizeof(int) + kVisT;
+  static constexpr int kQld = d + 32;                             // halves
+  static constexpr size_t kQ = (size_t)kAttnQ * kQld * 2;         // fp16 queries, and the same for their remainders
+  static constexpr size_t kRows = (size_t)kAttnWin * 4;           // pool row of each entry
+  static constexpr size_t kVis = (size_t)kAttnWin * 2;            // bit t: token t sees the entry
+  static constexpr size_t kScale = (size_t)kAttnQ * 4;            // score scale of each query
+  static constexpr size_t kLoop = 2 * kQ + kRows + kVis + kScale;
+  // the same space, once the entries are done: a tile's pieces of every warp
+  static constexpr int kOld = part_stride(d);                     // floats per query of a piece
+  static constexpr size_t kPieces = (size_t)kWarps * 8 * kOld * 4;
+  static constexpr size_t kMl = (size_t)kWarps * 8 * 8;           // (max, sum) per piece and query
+  static constexpr size_t kBytes = kLoop > kPieces + kMl ? kLoop : kPieces + kMl;
 };
 
 // Row of the q|k|v projection holding dimension i (< d/2) of q head h, or of
@@ -562,41 +525,72 @@ __device__ __forceinline__ int rot_row(int first, int h, int i, int d) {
   return first + 16 * (h * (d >> 4) + (i >> 3)) + (i & 7);
 }
 
-// Queries q0 .. q0 + qn of an item into shared memory: the fixed-point q sums
-// of the query's head and token, rotated by the token's position (RoPE,
-// pairs (i, i + d/2)), fp32.
+// Queries q0 .. q0 + qn of an item into shared memory: a warp per query reads
+// the fixed-point q sums of the query's head and token, rotates them by the
+// token's position (RoPE, pairs (i, i + d/2)), scales the row by a power of
+// two and splits it into fp16 and the fp16 of what that left out.
 template <int DPL>
 __device__ __forceinline__ void attn_load_queries(const AttnView& a, const StepParams* sp, int hk, int tok0, int q0,
-                                                  int qn, float* qsm) {
-  constexpr int d = 32 * DPL, half = d / 2;
-  const int G = a.Hq / a.Hkv;
-  for (int e = threadIdx.x; e < qn * half; e += kThreads) {
-    const int qi = e / half, i = e % half, q = q0 + qi;
-    const int m = tok0 + q / G, h = hk * G + q % G;
-    const long long* row = a.acc + (size_t)m * a.acc_ld;
-    const int R = rot_row(0, h, i, d);
-    const float lo = fixed_to_f32(__ldcg(row + R)), hi = fixed_to_f32(__ldcg(row + R + 8));
-    const float2 cs = a.rope[(size_t)sp->tok_pos[m] * half + i];
-    qsm[qi * d + i] = lo * cs.x - hi * cs.y;
-    qsm[qi * d + half + i] = hi * cs.x + lo * cs.y;
+                                                  int qn, uint16_t* qhi, uint16_t* qlo, float* qscale) {
+  constexpr int d = 32 * DPL, half = d / 2, kPair = half / 32, kRowsAtOnce = 4;
+  const int G = a.Hq / a.Hkv, tid = opaque(threadIdx.x), warp = tid >> 5, lane = tid & 31;
+  const float sm = rsqrtf(static_cast<float>(d));
+  for (int b0 = warp; b0 < qn; b0 += kWarps * kRowsAtOnce) {
+    long long lo[kRowsAtOnce][kPair], hi[kRowsAtOnce][kPair];
+    float2 cs[kRowsAtOnce][kPair];
+#pragma unroll
+    for (int r = 0; r < kRowsAtOnce; ++r) {
+      const int q = q0 + min(b0 + r * kWarps, qn - 1);
+      const int m = tok0 + q / G, h = hk * G + q % G;
+      const long long* row = a.acc + (size_t)m * a.acc_ld;
+#pragma unroll
+      for (int p = 0; p < kPair; ++p) {
+        const int i = lane + 32 * p, R = rot_row(0, h, i, d);
+        lo[r][p] = __ldcg(row + R);
+        hi[r][p] = __ldcg(row + R + 8);
+        cs[r][p] = a.rope[(size_t)sp->tok_pos[m] * half + i];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRowsAtOnce; ++r) {
+      const int qi = b0 + r * kWarps;
+      if (qi >= qn) break;
+      float x[2 * kPair];
+      uint32_t big = 0;
+#pragma unroll
+      for (int p = 0; p < kPair; ++p) {
+        const float l = fixed_to_f32(lo[r][p]), h = fixed_to_f32(hi[r][p]);
+        x[2 * p] = l * cs[r][p].x - h * cs[r][p].y;
+        x[2 * p + 1] = h * cs[r][p].x + l * cs[r][p].y;
+        big = max(big, max(__float_as_uint(fabsf(x[2 * p])), __float_as_uint(fabsf(x[2 * p + 1]))));
+      }
+      // 2^-e for the largest value's exponent e (the sums are below 2^32)
+      const int e = max((int)(__reduce_max_sync(0xffffffffu, big) >> 23), 64);
+      const float down = __uint_as_float((uint32_t)(254 - e) << 23);
+      if (lane == 0) qscale[qi] = sm * __uint_as_float((uint32_t)e << 23);
+      uint16_t* oh = qhi + (size_t)qi * AttnSmem<DPL>::kQld;
+      uint16_t* ol = qlo + (size_t)qi * AttnSmem<DPL>::kQld;
+#pragma unroll
+      for (int p = 0; p < 2 * kPair; ++p) {
+        const int i = lane + 32 * (p >> 1) + (p & 1) * half;
+        const float v = x[p] * down;
+        const uint16_t hv = f2h(v);
+        oh[i] = hv;
+        ol[i] = f2h(v - h2f(hv));
+      }
+    }
   }
 }
 
 // Merge of one (request, kv head, query): chunks in order, kMergeBatch at a
 // time with all their loads in flight; lane c of a batch holds chunk c's max
 // and sum, each lane DPL output dims.  The running result is rescaled when a
-// batch raises the maximum (online softmax).
+// batch raises the maximum (online softmax).  `base`: chunk 0's partial of
+// this query; cstride floats between chunks.
 template <int DPL>
-__device__ __forceinline__ void attn_merge_warp(const AttnView* ap, const StepParams* sp, int b, int hk, int qi, int lane) {
-  const AttnView& a = *ap;
-  constexpr int d = 32 * DPL;
+__device__ __forceinline__ void attn_merge_warp(const float* base, size_t cstride, int nc, uint16_t* out, int lane) {
   constexpr int kMergeBatch = 16;
   using VecT = typename std::conditional<DPL == 4, float4, float2>::type;
-  const int L = sp->req_len[b], tok0 = sp->req_tok0[b];
-  const int G = a.Hq / a.Hkv;
-  const int nc = n_chunks_of(L, a.cs);
-  const size_t cstride = (size_t)a.qmax * part_stride(d);
-  const float* base = a.part + (((size_t)b * a.Hkv + hk) * a.n_chunks) * cstride + (size_t)qi * part_stride(d);
   float M = -INFINITY, den = 0.f, num[DPL];
 #pragma unroll
   for (int u = 0; u < DPL; ++u) num[u] = 0.f;
@@ -638,220 +632,287 @@ __device__ __forceinline__ void attn_merge_warp(const AttnView* ap, const StepPa
     }
     M = Mn;
   }
-  uint16_t* out = a.out + (size_t)(tok0 + qi / G) * a.out_ld + (hk * G + qi % G) * d + DPL * lane;
 #pragma unroll
-  for (int u = 0; u < DPL; ++u) out[u] = f2h(num[u] / den);
+  for (int u = 0; u < DPL; ++u) out[DPL * lane + u] = f2h(num[u] / den);
 }
 
-// One item, processed by the CTA's consumer warps:
-//   1. the chunk's slots (beam table) and mask bits;
-//   2. the K and V rows of earlier steps, in flight while the item waits
-//      (bounded) for its kv head's q|k|v units;
-//   3. the rows this step appends, from the fixed-point k and v sums (k
-//      rotated by its token's position, both rounded to fp16) -- written to
-//      the shared tile and, by the one item whose chunk holds them, to the
-//      KV pool -- and the first query group;
-//   4. scores: warp w takes queries w, w + kWarps, ...; lane = entry; the
-//      softmax pieces (max, sum of exp) per query across the lanes;
-//   5. values: thread = (query, pair of head dims), sum over the entries;
-//   6. a release count of the finished chunk for its (request, kv head); when
-//      every CTA has at most one item, the CTA that counts the last chunk
-//      merges at once.
+// Partials (queries x chunks) up to which the last chunk's CTA merges alone: it
+// saves the other CTAs' polls, but reads them all through one SM (528 bytes each
+// at d = 128; 64 of them are one batch of loads per warp).
+constexpr int kMergeAlone = 64;
+
+// One item, processed by the CTA's consumer warps.
 template <int DPL>
-__device__ __forceinline__ void attn_item_cta(const AttnView* ap, int layer, const StepParams* sp, int b, int hk, int c,
-                                           uint8_t* area, int* status) {
+__device__ __forceinline__ void attn_item_cta(const AttnView* ap, int layer, const StepParams* sp, int item,
+                                              uint8_t* area, int* status) {
   const AttnView& a = *ap;
+  using S = AttnSmem<DPL>;
+  constexpr int d = S::d, half = d / 2;
+  constexpr int KJ = d / 32;   // 16-byte pieces of a lane's K row share
+  constexpr int VJ = d / 64;   // 16-byte pieces of a lane's V row share
+  int b, hk, c;
+  decode_item(sp, a.Hkv, a.cs, item, b, hk, c);
   uint16_t* kpool = a.kpool + (size_t)layer * a.layer_stride;
   uint16_t* vpool = a.vpool + (size_t)layer * a.layer_stride;
-  using S = AttnSmem<DPL>;
-  constexpr int d = S::d, KP = d / 8, half = d / 2;  // 16-byte pieces per row
-  uint16_t* Ks = reinterpret_cast<uint16_t*>(area);
-  uint16_t* Vs = reinterpret_cast<uint16_t*>(area + S::kK);
-  float* qsm = reinterpret_cast<float*>(area + S::kK + S::kV);
-  float* ps = reinterpret_cast<float*>(area + S::kK + S::kV + S::kQ);
-  int* slot_s = reinterpret_cast<int*>(area + S::kK + S::kV + S::kQ + S::kP);
-  int* vis_s = slot_s + kChunk;
-  uint8_t* vis_t = reinterpret_cast<uint8_t*>(vis_s + kChunk);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint16_t* qhi = reinterpret_cast<uint16_t*>(area);
+  uint16_t* qlo = reinterpret_cast<uint16_t*>(area + S::kQ);
+  uint32_t* rows_s = reinterpret_cast<uint32_t*>(area + 2 * S::kQ);
+  uint16_t* vis_s = reinterpret_cast<uint16_t*>(area + 2 * S::kQ + S::kRows);
+  float* qscale = reinterpret_cast<float*>(area + 2 * S::kQ + S::kRows + S::kVis);
+  float* pieces = reinterpret_cast<float*>(area);
+  float2* ml_s = reinterpret_cast<float2*>(area + S::kPieces);
+  const int tid = opaque(threadIdx.x), warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
   const int L = sp->req_len[b], P = sp->req_P[b];
   const int tok0 = sp->req_tok0[b], nb = sp->req_tok0[b + 1] - tok0;
   const int G = a.Hq / a.Hkv, Q = nb * G;
-  const int j0 = c * a.cs, nj = min(a.cs, L - j0);
-  const float scale = rsqrtf(static_cast<float>(d));
-  float* part = a.part + ((((size_t)b * a.Hkv + hk) * a.n_chunks + c) * a.qmax) * part_stride(d);
+  const int j0 = c * a.cs, nj = min(a.cs, L - j0), nc = n_chunks_of(L, a.cs);
 
-  // 1. the chunk's slots and mask bits (independent of this step's projections);
-  //    packed mode (Section 8.6): one mask row per token, each query reads its
-  //    token's row and no implicit causal bound applies
-  if (tid < kChunk) {
-    int slot = 0, vis = 0;
-    if (tid < nj) {
-      slot = __ldcg(a.bt + (size_t)b * a.cap + j0 + tid);
-      vis = a.packed ? 1 : __ldcg(a.mask + (size_t)b * a.mask_stride + j0 + tid) != 0;
-    }
-    slot_s[tid] = slot;
-    vis_s[tid] = vis;
-  }
-  if (a.packed)
-    for (int e = tid; e < nb * nj; e += kThreads)
-      vis_t[(e / nj) * kChunk + e % nj] = __ldcg(a.mask + (size_t)(tok0 + e / nj) * a.mask_stride + j0 + e % nj) != 0;
-  cbar();
-  {
-    constexpr int kRowPieces = kChunk * KP;
-    constexpr int kPer = (2 * kRowPieces + kThreads - 1) / kThreads;
-    uint4 v[kPer];
-    auto row_of = [&](int r) {
-      const int sl = slot_s[r];
-      return (((size_t)(sl / a.cap) * a.Hkv + hk) * a.cap + sl % a.cap) * d;
-    };
-    // 2. K/V rows of entries from earlier steps: in flight during the wait
+  uint4 kf[2][KJ], vf[4][VJ];
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      const int pi = tid + i * kThreads, r = (pi % kRowPieces) / KP;
-      v[i] = make_uint4(0, 0, 0, 0);
-      if (pi < 2 * kRowPieces && r < nj && j0 + r < P)
-        v[i] = __ldcg(reinterpret_cast<const uint4*>((pi >= kRowPieces ? vpool : kpool) + row_of(r)) + pi % KP);
+  for (int j = 0; j < KJ; ++j) kf[0][j] = kf[1][j] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+  for (int j = 0; j < VJ; ++j) vf[0][j] = vf[1][j] = vf[2][j] = vf[3][j] = make_uint4(0, 0, 0, 0);
+  // K rows: entries gid and gid + 8 of the block; V rows: entries 2 tig, + 1, + 8, + 9
+  auto load_k = [&](int blk) {
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+      const uint4* p = reinterpret_cast<const uint4*>(kpool + (size_t)rows_s[16 * blk + 8 * n + gid] * d) + tig;
+#pragma unroll
+      for (int j = 0; j < KJ; ++j) kf[n][j] = p[4 * j];
     }
-    if (tid == 0) wait_count(a.cnt_kv + hk, a.kv_units, status, a.limit);
+  };
+  auto load_v = [&](int blk) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const uint4* p =
+          reinterpret_cast<const uint4*>(vpool + (size_t)rows_s[16 * blk + 8 * (r >> 1) + 2 * tig + (r & 1)] * d) + gid;
+#pragma unroll
+      for (int j = 0; j < VJ; ++j) vf[r][j] = p[8 * j];
+    }
+  };
+  // the window's pool rows and visibility; entries that fill up the last
+  // block repeat the window's last one and are seen by nobody
+  auto stage = [&](int w0, int nw) {
+    for (int e = tid; e < (nw + 15) / 16 * 16; e += kThreads) {
+      const int j = j0 + w0 + min(e, nw - 1);
+      const int slot = __ldcg(a.bt + (size_t)b * a.cap + j);
+      uint32_t bits = 0;
+      if (e < nw) {
+        if (a.packed) {  // a mask row per token, and no causal bound of its own
+          const uint8_t* mp = a.mask + (size_t)tok0 * a.mask_stride + j;
+#pragma unroll 4
+          for (int t = 0; t < nb; ++t) bits |= (__ldcg(mp + (size_t)t * a.mask_stride) != 0 ? 1u : 0u) << t;
+        } else if (__ldcg(a.mask + (size_t)b * a.mask_stride + j) != 0) {
+          bits = 0xFFFFu << max(j - P, 0);  // token t sees entries up to P + t
+        }
+      }
+      const uint32_t pr = (uint32_t)slot / (uint32_t)a.cap;
+      rows_s[e] = (pr * a.Hkv + hk) * (uint32_t)a.cap + ((uint32_t)slot - pr * (uint32_t)a.cap);
+      vis_s[e] = (uint16_t)bits;
+    }
+  };
+
+  for (int q0 = 0; q0 < Q; q0 += kAttnQ) {
+    const int qn = min(kAttnQ, Q - q0), nqt = (qn + 7) >> 3;
+    const int eg = kWarps / nqt;             // warps side by side over the entries
+    const int qt = warp / eg, g = warp - qt * eg;
+    const bool active = qt < nqt;
+    const int tk = (q0 + min(8 * qt + gid, qn - 1)) / G;  // the token of query gid
+    float o[4 * VJ][4], mx = -INFINITY, den = 0.f, qs = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4 * VJ; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+    for (int w0 = 0; w0 < nj; w0 += kAttnWin) {
+      const int nw = min(kAttnWin, nj - w0), nblk = (nw + 15) >> 4;
+      const bool first = q0 == 0 && w0 == 0;
+      bool have = false;
+      if (w0 > 0) cbar();  // the previous window's entries are done
+      if (first || nj > kAttnWin || q0 > 0) stage(w0, nw);  // (the pieces overwrote it between passes)
+      if (first) {
+        cbar();
+        // a block of entries from earlier steps loads during the wait for q|k|v
+        have = active && g < nblk && j0 + 16 * g + 16 <= P;
+        if (have) {
+          load_k(g);
+          load_v(g);
+        }
+        if (tid == 0) wait_count(a.cnt_kv + hk, a.kv_units, status, a.limit);
+        cbar();
+        // the entries this step appends (they lie in the request's last
+        // chunks): k rotated by its token's position, both rounded to fp16
+        const int r0 = max(P - j0, 0), nnew = nj - r0;
+        if (nnew > 0) {
+          const int k_first = a.Hq * d, v_first = (a.Hq + a.Hkv) * d;
+          for (int e = tid; e < nnew * d; e += kThreads) {
+            const int r = e / d, i = e - r * d;
+            const int m = tok0 + (j0 + r0 + r - P);
+            const long long* row = a.acc + (size_t)m * a.acc_ld;
+            const int sl = sp->tok_slot[m];
+            const size_t at = (((size_t)(sl / a.cap) * a.Hkv + hk) * a.cap + sl % a.cap) * d;
+            if (i < half) {
+              const int R = rot_row(k_first, hk, i, d);
+              const float lo = fixed_to_f32(__ldcg(row + R)), hi = fixed_to_f32(__ldcg(row + R + 8));
+              const float2 cs = a.rope[(size_t)sp->tok_pos[m] * half + i];
+              kpool[at + i] = f2h(lo * cs.x - hi * cs.y);
+              kpool[at + half + i] = f2h(hi * cs.x + lo * cs.y);
+            } else {
+              const int i2 = 2 * (i - half);
+              const long long* vr = row + v_first + hk * d + i2;
+              *reinterpret_cast<uint32_t*>(vpool + at + i2) =
+                  pack_h2(fixed_to_f32(__ldcg(vr)), fixed_to_f32(__ldcg(vr + 1)));
+            }
+          }
+        }
+      }
+      if (w0 == 0) attn_load_queries<DPL>(a, sp, hk, tok0, q0, qn, qhi, qlo, qscale);
+      cbar();
+      if (!active) continue;
+      if (w0 == 0) qs = qscale[min(8 * qt + gid, qn - 1)];
+      if (!have && g < nblk) {
+        load_k(g);
+        load_v(g);
+      }
+      const uint16_t* qh = qhi + (8 * qt + gid) * S::kQld + 8 * tig;
+      const uint16_t* ql = qlo + (8 * qt + gid) * S::kQld + 8 * tig;
+      for (int blk = g; blk < nblk; blk += eg) {
+        const bool more = blk + eg < nblk;
+        const uint32_t va = *reinterpret_cast<const uint32_t*>(vis_s + 16 * blk + 2 * tig) >> tk;
+        const uint32_t vb = *reinterpret_cast<const uint32_t*>(vis_s + 16 * blk + 8 + 2 * tig) >> tk;
+        float s[2][2][4];  // two chains per 8 entries
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) s[n][e][0] = s[n][e][1] = s[n][e][2] = s[n][e][3] = 0.f;
+#pragma unroll
+        for (int j = 0; j < KJ; ++j) {
+          const uint4 h = *reinterpret_cast<const uint4*>(qh + 32 * j);
+          const uint4 l = *reinterpret_cast<const uint4*>(ql + 32 * j);
+#pragma unroll
+          for (int n = 0; n < 2; ++n) {
+            mma_16816(s[n][0], h.x, l.x, h.y, l.y, kf[n][j].x, kf[n][j].y);
+            mma_16816(s[n][1], h.z, l.z, h.w, l.w, kf[n][j].z, kf[n][j].w);
+          }
+        }
+        if (more) load_k(blk + eg);
+        // scores of query gid and entries 2 tig, + 1, + 8, + 9
+        float x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float (&u)[2][4] = s[i >> 1];
+          const int e = i & 1;
+          const bool see = ((i < 2 ? va : vb) >> (16 * e)) & 1u;
+          x[i] = see ? ((u[0][e] + u[1][e]) + (u[0][2 + e] + u[1][2 + e])) * qs : -INFINITY;
+        }
+        float mn = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+        mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
+        mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
+        mn = fmaxf(mn, mx);
+        if (__any_sync(0xffffffffu, mn > mx)) {
+          const float alpha = mx == -INFINITY ? 0.f : expf(mx - mn);
+          den *= alpha;
+          const float a0 = __shfl_sync(0xffffffffu, alpha, 8 * tig), a1 = __shfl_sync(0xffffffffu, alpha, 8 * tig + 4);
+#pragma unroll
+          for (int i = 0; i < 4 * VJ; ++i) {
+            o[i][0] *= a0;
+            o[i][1] *= a1;
+            o[i][2] *= a0;
+            o[i][3] *= a1;
+          }
+          mx = mn;
+        }
+        uint32_t ph[2], pl[2];  // the probabilities as the value sum's B fragments
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float p0 = x[2 * i] == -INFINITY ? 0.f : expf(x[2 * i] - mn) * kProbScale;
+          const float p1 = x[2 * i + 1] == -INFINITY ? 0.f : expf(x[2 * i + 1] - mn) * kProbScale;
+          den += p0 + p1;
+          const uint16_t u = f2h(p0), w = f2h(p1);
+          ph[i] = (uint32_t)u | ((uint32_t)w << 16);
+          pl[i] = pack_h2(p0 - h2f(u), p1 - h2f(w));
+        }
+        // O^T += V^T P^T: a lane's 32-bit word u of the four entries' rows
+        // holds dims 2 u and 2 u + 1 of its 8: rows gid and gid + 8 of a tile
+#pragma unroll
+        for (int i = 0; i < 4 * VJ; ++i) {
+          const int j = i >> 2, u = i & 3;
+          auto word = [&](const uint4& v) { return u == 0 ? v.x : u == 1 ? v.y : u == 2 ? v.z : v.w; };
+          const uint32_t r0 = word(vf[0][j]), r1 = word(vf[1][j]), r2 = word(vf[2][j]), r3 = word(vf[3][j]);
+          const uint32_t f0 = prmt_u32(r0, r1, 0x5410u), f1 = prmt_u32(r0, r1, 0x7632u);
+          const uint32_t f2 = prmt_u32(r2, r3, 0x5410u), f3 = prmt_u32(r2, r3, 0x7632u);
+          mma_16816(o[i], f0, f1, f2, f3, ph[0], ph[1]);
+          mma_16816(o[i], f0, f1, f2, f3, pl[0], pl[1]);
+        }
+        if (more) load_v(blk + eg);
+      }
+    }
+    // the CTA's pieces through shared memory
+    const int ngr = min(eg, (min(nj, kAttnWin) + 15) >> 4);  // warps of a tile that had entries
     cbar();
+    if (active && g < ngr) {
+      den += __shfl_xor_sync(0xffffffffu, den, 1);
+      den += __shfl_xor_sync(0xffffffffu, den, 2);
+      if (tig == 0) ml_s[warp * 8 + gid] = make_float2(mx, den);
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-      const int pi = tid + i * kThreads, r = (pi % kRowPieces) / KP;
-      if (pi < 2 * kRowPieces && r < nj && j0 + r < P) {
-        uint4* dst = pi >= kRowPieces ? reinterpret_cast<uint4*>(Vs + r * d) : reinterpret_cast<uint4*>(Ks + r * S::kKld);
-        dst[pi % KP] = v[i];
+      for (int e = 0; e < 2; ++e) {  // query 2 tig + e
+        float* w = pieces + (size_t)(warp * 8 + 2 * tig + e) * S::kOld + 8 * gid;
+#pragma unroll
+        for (int j = 0; j < VJ; ++j) {
+          *reinterpret_cast<float4*>(w + 64 * j) =
+              make_float4(o[4 * j][e], o[4 * j][2 + e], o[4 * j + 1][e], o[4 * j + 1][2 + e]);
+          *reinterpret_cast<float4*>(w + 64 * j + 4) =
+              make_float4(o[4 * j + 2][e], o[4 * j + 2][2 + e], o[4 * j + 3][e], o[4 * j + 3][2 + e]);
+        }
       }
     }
-  }
-  // 3. the entries this step appends (they lie in the request's last chunks)
-  {
-    const int r0 = max(P - j0, 0), nnew = nj - r0;
-    if (nnew > 0) {
-      const int k_first = a.Hq * d, v_first = (a.Hq + a.Hkv) * d;
-      for (int e = tid; e < nnew * half; e += kThreads) {
-        const int r = r0 + e / half, i = e % half;
-        const int m = tok0 + (j0 + r - P);
-        const long long* row = a.acc + (size_t)m * a.acc_ld;
-        const int R = rot_row(k_first, hk, i, d);
-        const float lo = fixed_to_f32(__ldcg(row + R)), hi = fixed_to_f32(__ldcg(row + R + 8));
-        const float2 cs = a.rope[(size_t)sp->tok_pos[m] * half + i];
-        const uint16_t klo = f2h(lo * cs.x - hi * cs.y), khi = f2h(hi * cs.x + lo * cs.y);
-        Ks[r * S::kKld + i] = klo;
-        Ks[r * S::kKld + half + i] = khi;
-        const int sl = sp->tok_slot[m];
-        uint16_t* kp = kpool + (((size_t)(sl / a.cap) * a.Hkv + hk) * a.cap + sl % a.cap) * d;
-        kp[i] = klo;
-        kp[half + i] = khi;
-      }
-      for (int e = tid; e < nnew * d; e += kThreads) {
-        const int r = r0 + e / d, i = e % d;
-        const int m = tok0 + (j0 + r - P);
-        const uint16_t vv = f2h(fixed_to_f32(__ldcg(a.acc + (size_t)m * a.acc_ld + v_first + hk * d + i)));
-        Vs[r * d + i] = vv;
-        const int sl = sp->tok_slot[m];
-        vpool[(((size_t)(sl / a.cap) * a.Hkv + hk) * a.cap + sl % a.cap) * d + i] = vv;
-      }
-    }
-    // rows past the chunk's end take part with weight zero: keep them finite
-    for (int e = tid; e < (kChunk - nj) * KP; e += kThreads) {
-      const int r = nj + e / KP;
-      if (r < a.cs) {
-        reinterpret_cast<uint4*>(Ks + r * S::kKld)[e % KP] = make_uint4(0, 0, 0, 0);
-        reinterpret_cast<uint4*>(Vs + r * d)[e % KP] = make_uint4(0, 0, 0, 0);
-      }
-    }
-  }
-  for (int q0 = 0; q0 < Q; q0 += S::kQg) {
-    const int qn = min(S::kQg, Q - q0);
-    if (q0 > 0) cbar();
-    attn_load_queries<DPL>(a, sp, hk, tok0, q0, qn, qsm);
     cbar();
-    for (int qi = warp; qi < qn; qi += kWarps) {
-      const float* qq = qsm + qi * d;
-      // lane scores entries lane, lane + 32, ... (cs / 32 of them)
-      float sc[kChunk / 32];
-#pragma unroll
-      for (int k = 0; k < kChunk / 32; ++k) sc[k] = 0.f;
-      if (a.cs == 32) {
-        sc[0] = dot_q_k(qq, Ks + lane * S::kKld, KP);
-      } else {
-#pragma unroll
-        for (int k = 0; k < kChunk / 32; k += 2)
-          if (32 * k < a.cs) sc[k] = dot_q_k2(qq, Ks + (lane + 32 * k) * S::kKld, Ks + (lane + 32 * k + 32) * S::kKld, sc[k + 1], KP);
+    for (int i = tid; i < qn * (d / 4); i += kThreads) {
+      const int f = i % (d / 4), qi = i / (d / 4), r = qi & 7, wa = (qi >> 3) * eg;
+      float M = -INFINITY, D = 0.f;
+      float4 num = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int w = wa; w < wa + ngr; ++w) M = fmaxf(M, ml_s[w * 8 + r].x);
+      for (int w = wa; w < wa + ngr; ++w) {
+        const float2 ml = ml_s[w * 8 + r];
+        const float k = ml.x == -INFINITY ? 0.f : expf(ml.x - M);
+        const float4 v = *reinterpret_cast<const float4*>(pieces + (size_t)(w * 8 + r) * S::kOld + 4 * f);
+        D = fmaf(ml.y, k, D);
+        num.x = fmaf(v.x, k, num.x);
+        num.y = fmaf(v.y, k, num.y);
+        num.z = fmaf(v.z, k, num.z);
+        num.w = fmaf(v.w, k, num.w);
       }
       const int q = q0 + qi;
-      const int lim = P + q / G;  // causal limit of this query's token
-      float mx = -INFINITY;
-      bool vis[kChunk / 32];
-#pragma unroll
-      for (int k = 0; k < kChunk / 32; ++k) {
-        const int e = lane + 32 * k;
-        vis[k] = e < nj && vis_s[e] && (a.packed ? vis_t[(q / G) * kChunk + e] != 0 : j0 + e <= lim);
-        sc[k] = vis[k] ? sc[k] * scale : -INFINITY;
-        mx = fmaxf(mx, sc[k]);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      float l = 0.f;
-#pragma unroll
-      for (int k = 0; k < kChunk / 32; ++k) {
-        const float e = vis[k] ? expf(sc[k] - mx) : 0.f;
-        l += e;
-        if (32 * k < a.cs) ps[qi * kChunk + lane + 32 * k] = e;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-      if (lane == 0) {
-        part[(size_t)q * part_stride(d)] = mx;
-        part[(size_t)q * part_stride(d) + 1] = l;
+      if (nc == 1) {
+        uint2 h;
+        h.x = pack_h2(num.x / D, num.y / D);
+        h.y = pack_h2(num.z / D, num.w / D);
+        *reinterpret_cast<uint2*>(a.out + (size_t)(tok0 + q / G) * a.out_ld + (hk * G + q % G) * d + 4 * f) = h;
+      } else {
+        float* p = a.part + ((size_t)item * a.qmax + q) * part_stride(d);
+        if (f == 0) *reinterpret_cast<float2*>(p) = make_float2(M, D);
+        *reinterpret_cast<float4*>(p + 4 + 4 * f) = num;
       }
     }
-    cbar();
-    for (int w = tid; w < qn * (d / 2); w += kThreads) {
-      const int qi = w / (d / 2), dp = w % (d / 2);
-      const float* pq = ps + qi * kChunk;
-      float o0 = 0.f, o1 = 0.f;
-#pragma unroll 8
-      for (int e = 0; e < a.cs; ++e) {  // rows past nj are zero with weight zero
-        const float pe = pq[e];
-        const float2 vf = h2f2(*reinterpret_cast<const uint32_t*>(Vs + e * d + 2 * dp));
-        o0 = fmaf(pe, vf.x, o0);
-        o1 = fmaf(pe, vf.y, o1);
-      }
-      *reinterpret_cast<float2*>(part + (size_t)(q0 + qi) * part_stride(d) + 4 + 2 * dp) = make_float2(o0, o1);
-    }
+    cbar();  // the partials are written, and the area is free
   }
-  // the item's partials are written (and the area is free for the next item);
-  // the release orders them before the count the merging CTA acquires
-  cbar();
-  if (!a.last_merges) {
-    if (tid == 0) red_release_add_s32(&a.cnt[b * a.Hkv + hk], 1);
-    return;
-  }
+  if (nc == 1) return;
+  // chunks of (b, hk) are items item - c .. item - c + nc - 1
+  int* cnt = &a.cnt[b * a.Hkv + hk];
   __shared__ int s_last;
-  if (tid == 0) s_last = atom_add_acq_rel(&a.cnt[b * a.Hkv + hk], 1) == n_chunks_of(L, a.cs) - 1;
-  cbar();
-  if (s_last) {
-    for (int qi = warp; qi < Q; qi += kWarps) attn_merge_warp<DPL>(ap, sp, b, hk, qi, lane);
-    cbar();
-    if (tid == 0) a.cnt[b * a.Hkv + hk] = 0;
+  const bool alone = Q * nc <= kMergeAlone;
+  if (tid == 0) {
+    if (alone) {
+      s_last = atom_add_acq_rel(cnt, 1) == nc - 1;
+    } else {
+      red_release_add_s32(cnt, 1);
+      wait_count(cnt, nc, status, a.limit);
+      s_last = 1;
+    }
   }
-}
-
-// Merge of (request b, kv head hk) by its designated CTA, after that CTA's
-// own items: wait until every chunk is counted (bounded), merge the queries
-// (one warp each), reset the count.
-template <int DPL>
-__device__ __forceinline__ void attn_merge_cta(const AttnView* ap, const StepParams* sp, int b, int hk, int* status) {
-  const AttnView& a = *ap;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int L = sp->req_len[b], nb = sp->req_tok0[b + 1] - sp->req_tok0[b];
-  const int Q = nb * (a.Hq / a.Hkv);
-  if (tid == 0) wait_count(&a.cnt[b * a.Hkv + hk], n_chunks_of(L, a.cs), status, a.limit);
   cbar();
-  for (int qi = warp; qi < Q; qi += kWarps) attn_merge_warp<DPL>(ap, sp, b, hk, qi, lane);
-  cbar();
-  if (tid == 0) a.cnt[b * a.Hkv + hk] = 0;
+  if (!s_last) return;
+  const float* base = a.part + (size_t)(item - c) * a.qmax * part_stride(d);
+  for (int q = alone ? warp : c + nc * warp; q < Q; q += alone ? kWarps : nc * kWarps)
+    attn_merge_warp<DPL>(base + (size_t)q * part_stride(d), (size_t)a.qmax * part_stride(d), nc,
+                         a.out + (size_t)(tok0 + q / G) * a.out_ld + (hk * G + q % G) * d, lane);
 }
 
 template <int NT, int GPU, int DPL>
@@ -860,6 +921,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   __shared__ GemvPhase s_gp[4];            // per projection kind: q|k|v, o, gate|up, down
   constexpr int kSlots = Geom<GPU>::kStepSlots;
   __shared__ AttnView s_av;
+  __shared__ int2 s_plan;                  // attention items: entries per item, number
   __shared__ uint64_t s_nbar;              // the staged RMSNorm's bulk copies
   __shared__ StepParams s_sp;
   __shared__ const uint16_t* s_rowp[kMaxTokens];  // the step's fp16 input rows
@@ -868,9 +930,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   uint8_t* rings = smem;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + SS::kRing);
   uint64_t* empty = full + kWarps * kSlots;
-  uint8_t* att_area = smem + SS::kRing + SS::kBars;
-  static_assert(AttnSmem<DPL>::kBytes <= SS::kQ, "attention area too small");
-  OpDesc* s_ops = reinterpret_cast<OpDesc*>(smem + SS::kFixed);
+  uint8_t* att_area = smem + SS::area(a.L, a.gu_part);
+  static_assert(AttnSmem<DPL>::kBytes <= kAttnArea, "attention area too small");
+  OpDesc* s_ops = reinterpret_cast<OpDesc*>(smem + SS::kOps);
   for (int i = threadIdx.x; i < 4 * a.L; i += kBlockThreads) s_ops[i] = a.ops[i];
   if (threadIdx.x == 0) {
     mbar_init(&s_nbar, 1);
@@ -899,8 +961,12 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   // ---- consumer warps from here on: CTA barriers are cbar() ----
   const StepParams* sp = &s_sp;
   const int M = sp->M;
-  GridBarrier gb{a.barrier, a.barrier_base, a.status, a.phase_clock, 0, 0, a.debug_skip_arrival, a.wait_limit};
-  // this warp's ring (its state stays in registers for the whole step)
+  __shared__ GridBarrier gb;
+  if (threadIdx.x == 0)
+    gb = GridBarrier{a.barrier, a.barrier_base, a.status, a.phase_clock, 0, 0, a.debug_skip_arrival, a.wait_limit};
+  // this warp's ring: its state stays in registers, except during attention,
+  // which needs them all (s_ring holds it meanwhile)
+  __shared__ WarpRing<GPU, kSlots> s_ring[kWarps];
   WarpRing<GPU, kSlots> ring;
   ring.ring = rings + (size_t)warp * kSlots * Geom<GPU>::kUnitBytes;
   ring.full = full + warp * kSlots;
@@ -908,20 +974,17 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   ring.n_used = 0;
   ring.timed_out = false;
   if (kSelfRefill) ring.start(s_ops, 4 * a.L, blockIdx.x * kWarps + warp, gridDim.x * kWarps, lane);
-  // Each CTA normalises the whole hidden state for itself; when the M rows
-  // fit, it keeps them in the attention area (idle during the q|k|v and
-  // gate|up projections) and the projections read them from there.  Rows are
-  // padded by 32 halves so that the two token rows a fragment load touches in
-  // one phase fall on different banks.
-  const int xn_ld = a.H + 32;
-  const bool xn_smem = kNormInSmem && a.Kp_H == a.H && (size_t)M * xn_ld * 2 <= SS::kQ;
-  uint16_t* xn = xn_smem ? reinterpret_cast<uint16_t*>(att_area) : a.act_h;
-  const int xn_out_ld = xn_smem ? xn_ld : a.Kp_H;
+  // The normalised rows: in the area (idle during the q|k|v and gate|up
+  // projections) when they fit, else read from act_h.
+  const int xn_ld = xn_stride(a.H);
+  const bool xn_smem = a.Kp_H == a.H && xn_bytes(a.H, M) <= a.area_bytes;
+  uint16_t* xn = reinterpret_cast<uint16_t*>(att_area);
   // one row from the residual stream: staged through shared memory behind
   // the normalised row (rmsnorm_staged)
-  const size_t stage_off = ((size_t)M * xn_ld * 2 + 127) / 128 * 128;
-  const bool norm_staged = M == 1 && xn_smem && a.H <= 24 * kThreads && stage_off + (size_t)a.H * 8 <= SS::kQ;
+  const size_t stage_off = xn_bytes(a.H, 1);
+  const bool norm_staged = M == 1 && xn_smem && a.H <= 24 * kThreads && stage_off + xn_stage_bytes(a.H, 1) <= a.area_bytes;
   long long* stage = reinterpret_cast<long long*>(att_area + stage_off);
+  int norms_done = 0;
   uint32_t nphase = 0;
   const int G = a.Hq / a.Hkv;
   if (threadIdx.x < 4) {
@@ -944,7 +1007,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
     gp.kv_rb_per_head = a.d / kRowsPerBlock;
     gp.kv_rb_k = a.Hq * a.d / kRowsPerBlock;
     gp.kv_rb_v = (a.Hq + a.Hkv) * a.d / kRowsPerBlock;
-    gp.part = reinterpret_cast<float*>(smem + SS::kFixed + SS::ops_bytes(a.L));
+    gp.part = reinterpret_cast<float*>(smem + SS::kOps + (size_t)4 * a.L * sizeof(OpDesc));
     s_gp[k] = gp;
   }
   if (threadIdx.x == 32) {
@@ -959,7 +1022,6 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
     av.Hq = a.Hq;
     av.Hkv = a.Hkv;
     av.d = a.d;
-    av.n_chunks = a.n_chunks;
     av.qmax = kMaxTokens * G;
     av.part = a.attn_part;
     av.cnt = a.attn_cnt;
@@ -970,21 +1032,20 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
     av.mask_stride = a.mask_stride;
     av.packed = a.packed;
     av.limit = a.wait_limit;
-    int items = 0;
-    for (int b = 0; b < sp->B; ++b) items += a.Hkv * n_chunks_of(sp->req_len[b], kAttnChunkMin);
-    // the smallest item size that needs one round of CTAs, else the largest
-    av.cs = kAttnChunkMin;
-    while (av.cs < kChunk && items > (int)gridDim.x) {
-      av.cs *= 2;
-      items = 0;
-      for (int b = 0; b < sp->B; ++b) items += a.Hkv * n_chunks_of(sp->req_len[b], av.cs);
-    }
-    av.last_merges = items <= (int)gridDim.x;
     av.out = a.act_attn;
     av.out_ld = a.Kp_dq;
     s_av = av;
   }
+  if (warp == 2) {
+    int cs, total;
+    attn_plan(sp, a.Hkv, gridDim.x, lane, cs, total);
+    if (lane == 0) s_plan = make_int2(cs, total);
+  }
   cbar();
+  if (threadIdx.x == 32) {
+    s_av.cs = s_plan.x;
+    s_av.total = s_plan.y;
+  }
   prologue_work(a.pro, sp, s_rowp, a.X);
   cbar();
   gb.arrive();  // split barrier: waited for before the first attention
@@ -1001,33 +1062,52 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
       // RMSNorm of the attention (k = 0) or MLP block; before the first
       // layer from the step's input rows
       const uint16_t* nw_ = a.norms + (size_t)l * 2 * a.H + (k == 2 ? a.H : 0);
-      if (norm_staged && ph != 0)
+      if (norm_staged && ph != 0) {
         rmsnorm_staged(a.X, a.H, nw_, a.eps, xn, stage, &s_nbar, nphase, a.status);
-      else
-        rmsnorm_cta(ph != 0, a.X, s_rowp, a.H, nw_, a.eps, xn, xn_out_ld, M);
+      } else {
+        // the one row of a staged step is fp16 here (8 KB): each CTA's own
+        for (int m = norm_staged ? 0 : blockIdx.x; m < M; m += gridDim.x)
+          rmsnorm_row(ph != 0, a.X, s_rowp, a.H, m, nw_, a.eps, norm_staged ? xn : a.act_h + (size_t)m * a.Kp_H,
+                      norm_staged ? nullptr : a.norm_cnt);
+      }
+      if (!norm_staged) {
+        norms_done += M;
+        if (threadIdx.x == 0) {
+          wait_count(a.norm_cnt, norms_done, a.status, a.wait_limit);
+          if (xn_smem) {
+            // the rows were written through the generic proxy; the area was
+            // last used by generic accesses of this CTA
+            asm volatile("fence.proxy.async;" ::: "memory");
+            mbar_arrive_expect_tx(&s_nbar, (uint32_t)M * a.H * 2u);
+            for (int m = 0; m < M; ++m)
+              bulk_g2s(xn + (size_t)m * xn_ld, a.act_h + (size_t)m * a.Kp_H, (uint32_t)a.H * 2u, &s_nbar);
+          }
+        }
+        if (xn_smem) {
+          if (!mbar_wait(&s_nbar, nphase) && threadIdx.x == 0) atomicOr(a.status, ST_WAIT_TIMEOUT);
+          nphase ^= 1u;
+        }
+        cbar();
+      }
     } else if (k == 1) {
       // the q|k|v sums and counts are consumed: clear them for the next layer
       for (int e = gt; e < M * qkv_rows; e += gs) __stcg(a.acc_qkv + e, 0LL);
-      if (blockIdx.x == 0 && threadIdx.x < a.Hkv) __stcg(a.cnt_kv + threadIdx.x, 0);
+      if (blockIdx.x == 0) {
+        if (threadIdx.x < a.Hkv) __stcg(a.cnt_kv + threadIdx.x, 0);
+        for (int e = threadIdx.x; e < sp->B * a.Hkv; e += kThreads) __stcg(a.attn_cnt + e, 0);
+      }
     }
     gemv_run<NT, GPU, kSlots>(ring, &s_ops[ph], &s_gp[k], g, nw, lane);
     if (k == 0) {
+      if (lane == 0) s_ring[warp] = ring;
+      __syncwarp();
       if (l == 0) gb.wait();        // the prologue's tables and residual are complete
       else if (xn_smem) cbar();     // the attention items reuse the normalised rows' space
-      int total = 0;
-      for (int b = 0; b < sp->B; ++b) total += a.Hkv * n_chunks_of(sp->req_len[b], s_av.cs);
-      for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        int b, hk, c;
-        if (decode_item(sp, a.Hkv, s_av.cs, item, b, hk, c)) attn_item_cta<DPL>(&s_av, l, sp, b, hk, c, att_area, a.status);
-      }
-      // merges, when CTAs take several items: (b, hk) goes to the CTA that
-      // took its last chunk
-      for (int b = 0, base = 0; !s_av.last_merges && b < sp->B; ++b) {
-        const int nc = n_chunks_of(sp->req_len[b], s_av.cs);
-        for (int hk = 0; hk < a.Hkv; ++hk)
-          if ((base + hk * nc + nc - 1) % gridDim.x == blockIdx.x) attn_merge_cta<DPL>(&s_av, sp, b, hk, a.status);
-        base += a.Hkv * nc;
-      }
+      for (int item = blockIdx.x; item < s_av.total; item += gridDim.x)
+        attn_item_cta<DPL>(&s_av, l, sp, item, att_area, a.status);
+      __syncwarp();
+      asm volatile("" ::: "memory");
+      ring = s_ring[warp];
     }
     gb.sync();
   }
@@ -1043,6 +1123,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   cbar();
   if (threadIdx.x == 0 && atom_add_acq_rel(a.exit_count, 1) == (int)gridDim.x - 1) {
     *a.exit_count = 0;
+    *a.norm_cnt = 0;
     const int st = ld_acquire_s32(a.status);
     if (st) *reinterpret_cast<volatile int*>(a.status_out) = st;
   }
@@ -1054,7 +1135,7 @@ cudaError_t launch_t(const StepKernelArgs& a, int grid, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kBlockThreads);
-  cfg.dynamicSmemBytes = a.gu_part ? StepSmem<GPU>::total_with_part(a.L) : StepSmem<GPU>::total(a.L);
+  cfg.dynamicSmemBytes = StepSmem<GPU>::area(a.L, a.gu_part) + a.area_bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -1092,7 +1173,16 @@ size_t dyn_limit_group() {
 
 template <int GPU>
 bool part_fits(int L) {
-  return StepSmem<GPU>::total_with_part(L) <= dyn_limit_group<GPU>();
+  return StepSmem<GPU>::total(L, true) <= dyn_limit_group<GPU>();
+}
+
+// Bytes of the shared-memory area for steps of M tokens: room for the
+// normalised rows where the kernel's limit allows it.
+template <int GPU>
+size_t area_bytes_t(int H, int L, bool part, int M) {
+  const size_t want = xn_bytes(H, M) + xn_stage_bytes(H, M);
+  if (want <= kAttnArea || StepSmem<GPU>::area(L, part) + want > dyn_limit_group<GPU>()) return kAttnArea;
+  return want;
 }
 
 }  // namespace
@@ -1108,6 +1198,12 @@ bool step_gu_part_fits(int group, int L) {
   return false;
 }
 
+size_t step_area_bytes(int group, int H, int L, bool part, int M) {
+  if (group == 128) return area_bytes_t<1>(H, L, part, M);
+  if (group == 64) return area_bytes_t<2>(H, L, part, M);
+  return area_bytes_t<4>(H, L, part, M);
+}
+
 int step_gu_split(int n_rb, int upr, int grid, int group, int L) {
   if (n_rb < 1 || upr < 1 || grid < 1 || !step_gu_part_fits(group, L)) return 0;
   const long long nw = (long long)grid * kWarps;
@@ -1121,8 +1217,8 @@ int step_gu_split(int n_rb, int upr, int grid, int group, int L) {
   return best;
 }
 
-size_t step_attention_part_floats(int B, int Hkv, int n_chunks, int G, int d) {
-  return (size_t)B * Hkv * n_chunks * (kMaxTokens * G) * part_stride(d);
+size_t step_attention_part_floats(int grid, int G, int d) {
+  return (size_t)grid * (kMaxTokens * G) * part_stride(d);
 }
 
 cudaError_t step_setup(int group, int head_dim) {
