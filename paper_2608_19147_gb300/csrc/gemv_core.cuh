@@ -336,9 +336,94 @@ __device__ __noinline__ void ring_producer(const OpDesc* ops, int n_ops, int cta
 constexpr float kTotScaleLo = 72057594037927936.0f;  // 2^56 = 2^32 (fixed point) * 2^24
 constexpr float kTotScaleHi = 4503599627370496.0f;   // 2^52 = 2^32 * 2^20
 
+// Group end of one 16-row tile: zero-point correction and scale.  zw: the
+// zero bytes of tiles 2 i and 2 i + 1 (z_lo, 16 z_hi of each), scw: the
+// tile's two scales.
+template <int NT>
+__device__ __forceinline__ void group_end(float (&tot)[NT][4], const float (&acc)[NT][4], const float (&sa)[NT][4],
+                                          uint32_t zw, uint32_t scw, int rt) {
+  const uint32_t p = 2u * (rt & 1);
+  // fp16 bits 0x8000 | z and 0x8000 | 16 z: -z * 2^-24 and -16 z * 2^-24
+  const uint32_t zp = prmt_u32(zw, 0x80u, p | (4u << 4) | ((p + 1u) << 8) | (4u << 12));
+  const float zlo = h2f(static_cast<uint16_t>(zp & 0xFFFFu));
+  const float zhi = h2f(static_cast<uint16_t>(zp >> 16));
+  const float slo = h2f(static_cast<uint16_t>(scw & 0xFFFFu));
+  const float shi = h2f(static_cast<uint16_t>(scw >> 16));
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    tot[nt][0] = fmaf(slo, fmaf(zlo, sa[nt][0], acc[nt][0]), tot[nt][0]);
+    tot[nt][1] = fmaf(slo, fmaf(zlo, sa[nt][1], acc[nt][1]), tot[nt][1]);
+    tot[nt][2] = fmaf(shi, fmaf(zhi, sa[nt][0], acc[nt][2]), tot[nt][2]);
+    tot[nt][3] = fmaf(shi, fmaf(zhi, sa[nt][1], acc[nt][3]), tot[nt][3]);
+  }
+}
+
+// Two token tiles (M > 8): two 16-row tiles at a time.  With all four, their
+// sums beside two units' activations do not fit the registers (1448 bytes of
+// spills in the step kernel, now 272; 16 packed tokens at 8B width, 4 layers:
+// 470 -> 427 us).
+template <int GPU>
+__device__ __forceinline__ void mma_unit2(const uint8_t* __restrict__ U, const uint4 (&act)[2][2][2],
+                                          float (&tot)[4][2][4], int lane) {
+  constexpr int BPG = Geom<GPU>::kBlocksPerGroup;
+  constexpr uint32_t kOnes = 0x3C003C00u;  // fp16x2 (1, 1)
+  const int gid = lane >> 2;
+#pragma unroll
+  for (int gi = 0; gi < GPU; ++gi) {
+    const uint8_t* meta = U + kCodeBytes + gi * kMetaBytesPerGroup;
+    float sa[2][4];
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) sa[nt][0] = sa[nt][1] = sa[nt][2] = sa[nt][3] = 0.f;
+#pragma unroll
+    for (int r0 = 0; r0 < 4; r0 += 2) {
+      float acc[2][2][4];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) acc[r][nt][0] = acc[r][nt][1] = acc[r][nt][2] = acc[r][nt][3] = 0.f;
+      uint4 A[2];
+#pragma unroll
+      for (int blk = gi * BPG; blk < (gi + 1) * BPG; ++blk) {
+        const int j = blk & 3;
+        if (blk == gi * BPG || j == 0)
+#pragma unroll
+          for (int r = 0; r < 2; ++r)
+            A[r] = *reinterpret_cast<const uint4*>(U + ((blk >> 2) * 4 + r0 + r) * 512 + lane * 16);
+        uint32_t b0[2], b1[2];
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          const uint4 v = act[nt][blk >> 2][(blk >> 1) & 1];
+          b0[nt] = (blk & 1) ? v.z : v.x;
+          b1[nt] = (blk & 1) ? v.w : v.y;
+          if (r0 == 0) mma_16816(sa[nt], kOnes, kOnes, kOnes, kOnes, b0[nt], b1[nt]);
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const uint32_t w = (j == 0) ? A[r].x : (j == 1) ? A[r].y : (j == 2) ? A[r].z : A[r].w;
+          const uint32_t w2 = w >> 8;
+          const uint32_t a0 = w & 0x000F000Fu, a1 = w & 0x00F000F0u;
+          const uint32_t a2 = w2 & 0x000F000Fu, a3 = w2 & 0x00F000F0u;
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) mma_16816(acc[r][nt], a0, a1, a2, a3, b0[nt], b1[nt]);
+        }
+      }
+      const uint2 zz = *reinterpret_cast<const uint2*>(meta + 128 + gid * 8);
+      const uint4 sc = *reinterpret_cast<const uint4*>(meta + gid * 16);
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        group_end<2>(tot[r0 + r], acc[r], sa, r0 == 0 ? zz.x : zz.y, r0 == 0 ? (r ? sc.y : sc.x) : (r ? sc.w : sc.z), r);
+    }
+  }
+}
+
+// NT token tiles of 8.
 template <int NT, int GPU>
 __device__ __forceinline__ void mma_unit(const uint8_t* __restrict__ U, const uint4 (&act)[NT][2][2],
                                          float (&tot)[4][NT][4], int lane) {
+  if constexpr (NT == 2) {
+    mma_unit2<GPU>(U, act, tot, lane);
+    return;
+  }
   constexpr int BPG = Geom<GPU>::kBlocksPerGroup;
   constexpr uint32_t kOnes = 0x3C003C00u;  // fp16x2 (1, 1)
   const int gid = lane >> 2;
@@ -388,23 +473,7 @@ __device__ __forceinline__ void mma_unit(const uint8_t* __restrict__ U, const ui
         const uint4 sc = *reinterpret_cast<const uint4*>(meta + gid * 16);
         const uint32_t scw[4] = {sc.x, sc.y, sc.z, sc.w};
 #pragma unroll
-        for (int rt = 0; rt < 4; ++rt) {
-          const uint32_t zw = rt < 2 ? zz.x : zz.y;  // bytes: z_lo, 16 z_hi of tiles 2i, then 2i + 1
-          const uint32_t p = 2u * (rt & 1);
-          // fp16 bits 0x8000 | z and 0x8000 | 16 z: -z * 2^-24 and -16 z * 2^-24
-          const uint32_t zp = prmt_u32(zw, 0x80u, p | (4u << 4) | ((p + 1u) << 8) | (4u << 12));
-          const float zlo = h2f(static_cast<uint16_t>(zp & 0xFFFFu));
-          const float zhi = h2f(static_cast<uint16_t>(zp >> 16));
-          const float slo = h2f(static_cast<uint16_t>(scw[rt] & 0xFFFFu));
-          const float shi = h2f(static_cast<uint16_t>(scw[rt] >> 16));
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            tot[rt][nt][0] = fmaf(slo, fmaf(zlo, sa[nt][0], accg[rt][nt][0]), tot[rt][nt][0]);
-            tot[rt][nt][1] = fmaf(slo, fmaf(zlo, sa[nt][1], accg[rt][nt][1]), tot[rt][nt][1]);
-            tot[rt][nt][2] = fmaf(shi, fmaf(zhi, sa[nt][0], accg[rt][nt][2]), tot[rt][nt][2]);
-            tot[rt][nt][3] = fmaf(shi, fmaf(zhi, sa[nt][1], accg[rt][nt][3]), tot[rt][nt][3]);
-          }
-        }
+        for (int rt = 0; rt < 4; ++rt) group_end<NT>(tot[rt], accg[rt], sa, rt < 2 ? zz.x : zz.y, scw[rt], rt);
       }
     }
   }
