@@ -566,17 +566,18 @@ static __device__ __noinline__ void finish_store(const GemvPhase* pp, int rb, in
 // ---------------------------------------------------------------------------
 // Gate|up with OpDesc::q > 0: row-block rb is reduced inside its CTA.  Each
 // of its q warps writes its sums, in natural scale, to its own slot of the
-// CTA's partial area (fp32 [kCtaWarps][kGuCtaTokens][64]); after a named
-// barrier of the q warps (id 2 + group) they add the q slots in a fixed order
-// and write h = silu(gate) * up as fp16.  No global atomics; the result does
-// not depend on arrival order.
+// CTA's partial area (fp32 [kCtaWarps][M][64]); after a named barrier of the q
+// warps (id 2 + group) they add the q slots in a fixed order and write
+// h = silu(gate) * up as fp16.  No global atomics (64 M per warp and
+// row-block otherwise, and a second pass over the sums: norm + gate|up of 8
+// tokens at 8B width 25.8 -> 21.2 us); the result does not depend on arrival
+// order.
 // ---------------------------------------------------------------------------
-constexpr int kGuCtaTokens = 5;  // tokens up to which the whole-step kernel reduces gate|up this way
 
 template <int NT>
 __device__ __forceinline__ void swiglu_cta_write(const GemvPhase& p, const float (&tot)[4][NT][4], int w, int lane) {
   const int gid = lane >> 2, tig = lane & 3;
-  float* slot = p.part + (size_t)w * kGuCtaTokens * kRowsPerBlock;
+  float* slot = p.part + (size_t)w * p.M * kRowsPerBlock;
 #pragma unroll
   for (int rt = 0; rt < 4; ++rt)
 #pragma unroll
@@ -596,7 +597,7 @@ __device__ __forceinline__ void swiglu_cta_write(const GemvPhase& p, const float
 static __device__ __forceinline__ void swiglu_cta_finish(const GemvPhase* pp, int rb, int q, int w, int lane) {
   const GemvPhase& p = *pp;
   const int grp0 = w - w % q;
-  const float* base = p.part + (size_t)grp0 * kGuCtaTokens * kRowsPerBlock;
+  const float* base = p.part + (size_t)grp0 * p.M * kRowsPerBlock;
   for (int it = (w - grp0) * 32 + lane; it < 32 * p.M; it += q * 32) {
     const int m = it >> 5, jl = it & 31;
     const int Rg = 16 * (jl >> 3) + (jl & 7);
@@ -604,7 +605,7 @@ static __device__ __forceinline__ void swiglu_cta_finish(const GemvPhase* pp, in
     // sums): the same bits for any token count
     long long gs = 0, us = 0;
     for (int i = 0; i < q; ++i) {
-      const float* sl = base + (size_t)i * kGuCtaTokens * kRowsPerBlock + m * kRowsPerBlock;
+      const float* sl = base + (size_t)(i * p.M + m) * kRowsPerBlock;
       gs += f2fix(sl[Rg] * kFixOne);
       us += f2fix(sl[Rg + 8] * kFixOne);
     }
@@ -683,7 +684,7 @@ __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* o
   int wb, we;
   run_range(*op, g, nw, wb, we);
   if (wb >= we) {
-    if (op->q > 0 && p.M <= kGuCtaTokens) {  // a group member without units still adds (zero) sums
+    if (op->q > 0) {  // a group member without units still adds (zero) sums
       float zero[4][NT][4];
 #pragma unroll
       for (int rt = 0; rt < 4; ++rt)
@@ -727,7 +728,7 @@ __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* o
       if (!ring.timed_out) mma_unit<NT, GPU>(U, cur, tot, lane);
       ring.release(lane);
     }
-    if (op->q > 0 && p.M <= kGuCtaTokens)
+    if (op->q > 0)
       swiglu_cta_end<NT>(pp, op, tot, g, lane);  // the run is one whole segment
     else
       segment_end<NT>(pp, tot, rb, seg_end - seg_begin, upr, lane);

@@ -287,9 +287,8 @@ cudaError_t step_setup(int group, int head_dim);
 // grid-wide split), when the kernel's shared memory for L layers leaves room
 // for the partial sums.
 int step_gu_split(int n_rb, int upr, int grid, int group, int L);
-// Token count up to which the whole-step kernel uses that reduction.
-int step_gu_cta_tokens();
-// Whether the kernel's shared memory for L layers has room for the partial sums.
+// Whether the kernel's shared memory for L layers has room for the partial
+// sums of the largest step.
 bool step_gu_part_fits(int group, int L);
 // Shared memory of the attention / normalised-row area for steps of M tokens.
 size_t step_area_bytes(int group, int H, int L, bool part, int M);

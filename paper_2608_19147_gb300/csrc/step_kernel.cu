@@ -51,13 +51,12 @@ struct StepSmem {
   static constexpr size_t kRing = (size_t)kWarps * kSlots * Geom<GPU>::kUnitBytes;
   static constexpr size_t kBars = (size_t)2 * kWarps * kSlots * sizeof(uint64_t);
   static constexpr size_t kOps = kRing + kBars;
-  // gate|up partial sums of the shared-memory reduction (swiglu_cta_write)
-  static constexpr size_t kPart = (size_t)kWarps * kGuCtaTokens * kRowsPerBlock * sizeof(float);
+  // gate|up partial sums of the shared-memory reduction (swiglu_cta_write) for M tokens
+  __host__ __device__ static size_t part(int M) { return (size_t)kWarps * M * kRowsPerBlock * sizeof(float); }
   // offset of the area
-  __host__ __device__ static size_t area(int n_layers, bool part) {
-    return (kOps + (size_t)4 * n_layers * sizeof(OpDesc) + (part ? kPart : 0) + 127) / 128 * 128;
+  __host__ __device__ static size_t area(int n_layers, bool with_part, int M) {
+    return (kOps + (size_t)4 * n_layers * sizeof(OpDesc) + (with_part ? part(M) : 0) + 127) / 128 * 128;
   }
-  static size_t total(int n_layers, bool part) { return area(n_layers, part) + kAttnArea; }
 };
 
 // Row stride (halves) of the normalised rows in shared memory: padded so that
@@ -930,7 +929,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   uint8_t* rings = smem;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + SS::kRing);
   uint64_t* empty = full + kWarps * kSlots;
-  uint8_t* att_area = smem + SS::area(a.L, a.gu_part);
+  uint8_t* att_area = smem + SS::area(a.L, a.gu_part, a.pro.M);
   static_assert(AttnSmem<DPL>::kBytes <= kAttnArea, "attention area too small");
   OpDesc* s_ops = reinterpret_cast<OpDesc*>(smem + SS::kOps);
   for (int i = threadIdx.x; i < 4 * a.L; i += kBlockThreads) s_ops[i] = a.ops[i];
@@ -1135,7 +1134,7 @@ cudaError_t launch_t(const StepKernelArgs& a, int grid, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kBlockThreads);
-  cfg.dynamicSmemBytes = StepSmem<GPU>::area(a.L, a.gu_part) + a.area_bytes;
+  cfg.dynamicSmemBytes = StepSmem<GPU>::area(a.L, a.gu_part, a.pro.M) + a.area_bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -1173,7 +1172,7 @@ size_t dyn_limit_group() {
 
 template <int GPU>
 bool part_fits(int L) {
-  return StepSmem<GPU>::total(L, true) <= dyn_limit_group<GPU>();
+  return StepSmem<GPU>::area(L, true, kMaxTokens) + kAttnArea <= dyn_limit_group<GPU>();
 }
 
 // Bytes of the shared-memory area for steps of M tokens: room for the
@@ -1181,15 +1180,13 @@ bool part_fits(int L) {
 template <int GPU>
 size_t area_bytes_t(int H, int L, bool part, int M) {
   const size_t want = xn_bytes(H, M) + xn_stage_bytes(H, M);
-  if (want <= kAttnArea || StepSmem<GPU>::area(L, part) + want > dyn_limit_group<GPU>()) return kAttnArea;
+  if (want <= kAttnArea || StepSmem<GPU>::area(L, part, M) + want > dyn_limit_group<GPU>()) return kAttnArea;
   return want;
 }
 
 }  // namespace
 
 int step_barriers(int n_layers) { return 4 * n_layers + 1; }
-
-int step_gu_cta_tokens() { return kGuCtaTokens; }
 
 bool step_gu_part_fits(int group, int L) {
   if (group == 128) return part_fits<1>(L);
