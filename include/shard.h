@@ -216,7 +216,7 @@ int shard_step_packed(shard_t shard, kvstate_t state, const uint16_t* hidden_in,
  * is the one shard_step gives for S tokens of one request -- the same
  * rounding points, causal attention among the new tokens and over the row's
  * entries with mask != 0 -- computed with the projections as dense
- * contractions on the tensor cores, in chunks of up to 256 tokens.
+ * contractions on the tensor cores, in chunks of up to 512 tokens.
  *   hidden_in / token_ids  as shard_step (exactly one), [S] rows
  *   position_ids           dev int32 [S]
  *   attention_mask         dev uint8 [mask_len], the row's mask, mask_len >=

@@ -5,26 +5,40 @@
 // is filled by running the prompt through the stage) -- where the per-token
 // GEMV of the decode step would stream every weight once per 16 tokens.
 //
-// One CTA computes a tile of 128 weight rows (two 64-row blocks) by N tokens,
-// walking K one 128-input unit per step, with warp roles joined by mbarriers:
+// One CTA computes a tile of 128 weight rows (two row-blocks) by N tokens over
+// all of K or a part of it, walking K one 128-input unit per step, with warp
+// roles joined by mbarriers:
 //   - warp 0 (producer): bulk-copies the step's two units (codes, scales,
 //     zero points) and loads the token tile with two 2-D tensor copies (64
-//     inputs x N tokens each, 128-byte swizzle); 3 stages ahead;
-//   - warps 10..17 (dequantise): turn the codes into exact fp16 (q - z) in the
-//     A tile; 2 stages;
-//   - warp 1 (MMA): issues tcgen05.mma (kind::f16, M = 128, N tokens, K = 16
-//     per instruction) into a TMEM accumulator per quantisation group and
-//     commits to the stages' mbarriers; 2 accumulator stages;
-//   - warps 2..9 (epilogue): read the step's accumulators (tcgen05.ld; warp w
-//     owns TMEM lanes 32 (w % 4) .. + 31 = tile rows, half the token columns
-//     each), multiply by the row's fp32 group scale and add into registers;
-//     at the end they write their rows' outputs.
-// Both operands sit in shared memory in the canonical K-major layout with the
-// 128-byte swizzle: per 64-input half of the step, row r's 128 bytes at r *
-// 128, its 16-byte chunk c at chunk c ^ (r % 8) -- what the tensor copy writes
-// with that swizzle, whole 32-byte sectors from L2, and a layout in which the
-// dequantise warps' 16-byte stores of 8 consecutive rows hit distinct banks.
-// The
+//     inputs x N tokens each, 128-byte swizzle), several stages ahead;
+//   - warps 20..27 (dequantise): turn the codes into exact fp16 (q - z) and
+//     store them to tensor memory, the A operand; two sets of four warps take
+//     the steps in turn, 2 stages;
+//   - warps 1, 2 (MMA): a thread each, steps in turn, issues tcgen05.mma
+//     (kind::f16, M = 128, N tokens, K = 16 per instruction, A in tensor memory,
+//     B in shared memory) into a ring of accumulators, one per quantisation
+//     group and step, and commits to the step's mbarrier;
+//   - warps 4..19 (epilogue): read the accumulators (tcgen05.ld; warp w owns
+//     lanes 32 (w % 4) .. + 31 = tile rows, a quarter of the token columns),
+//     multiply by the row's fp32 group scale and add into registers; at the
+//     end they write their rows' outputs.
+// A in tensor memory: with A in shared memory too, a step of 128 x 128 x 128 moved
+// 64 KB of operands through it beside 40 KB of arriving copies and 40 KB of
+// dequantisation. The code words' fragment order (kernels.h) is the lane order
+// of tcgen05.st's 16x256b shape, so a warp reads its words with conflict-free
+// 16-byte loads and stores each word's four fp16 pairs as they are. The price is
+// the order of the inputs: a lane's word holds inputs 8 t + 4 j .. + 3 of a
+// 32-input block (t = lane % 4), so activations are kept with each block's
+// 4-input chunks in the order 0 2 4 6 1 3 5 7 (act_pos).
+// What bounds it is the roles' own chains of barrier polls and short dependent
+// work, ~1150 cycles a step against 512 of tensor time: leaving out, one at a
+// time, the MMAs, the dequantisation's arithmetic, the epilogue's loads or the
+// copies changes a step by 2-6 %. Against the first version (A in shared memory,
+// three commits a step by one thread, suspending waits), 512 tokens at 8B width,
+// 4 layers: gate|up 225 -> 159 us per layer, o and down 73 -> 48, q|k|v 61 -> 46;
+// 604 -> 850 TFLOP/s for gate|up alone.
+// The token tile sits in the canonical K-major layout with the 128-byte
+// swizzle, as the tensor copy writes it. The
 // arithmetic is the decode projection's: exact (q - z), fp32 sums per group,
 // the fp16 scale applied in fp32.  Every wait is bounded; a wait that runs out
 // sets the status word.  The TMEM columns are freed before the CTA exits.
@@ -38,24 +52,32 @@ namespace shard {
 namespace {
 
 constexpr int kTcRows = 128;        // weight rows per CTA tile (two row-blocks)
-constexpr int kTcWarps = 18;        // producer, MMA, 8 epilogue, 8 dequantise
-constexpr int kDqWarps = 8;
+constexpr int kTcWarps = 20;
 constexpr int kTcThreads = kTcWarps * 32;
-constexpr int kEpiWarp0 = 2, kDqWarp0 = 10;
-constexpr int kUStages = 4, kBStages = 3, kAStages = 2, kDStages = 2;
+constexpr int kMmaWarp0 = 1, kMmaWarps = 2, kEpiWarp0 = 4, kEpiWarps = 8, kDqWarp0 = 12, kDqSets = 2;
+constexpr int kUStages = 6, kBStages = 4, kAStages = 2;
 
 template <int N, int GPU>
 struct TcSmem {
   static constexpr size_t kUnit = Geom<GPU>::kUnitBytes;
   static constexpr size_t kUnits = 2 * kUnit;                          // the tile's two units
-  static constexpr size_t kA = (size_t)kTcRows * 256;                  // 16 K chunks x 128 rows x 16 B
-  static constexpr size_t kB = (size_t)N * 256;                        // 16 K chunks x N tokens x 16 B
-  static constexpr size_t kAOff = 0;                                   // [kAStages][kA]
-  static constexpr size_t kBOff = kAOff + kAStages * kA;               // [kBStages][kB]
+  static constexpr size_t kB = (size_t)N * 256;                        // 128 inputs x N tokens
+  static constexpr size_t kBOff = 0;                                   // [kBStages][kB]
   static constexpr size_t kUOff = kBOff + kBStages * kB;               // [kUStages][kUnits]
-  static constexpr size_t kSc = (size_t)GPU * kTcRows * sizeof(float);  // a step's scales [group][row]
-  static constexpr size_t kScOff = kUOff + kUStages * kUnits;          // [kAStages][kSc]
-  static constexpr size_t kTotal = kScOff + kAStages * kSc + 1024;     // + alignment slack
+  static constexpr int kHLd = 72;                                      // halves per token of the staged SwiGLU rows
+  static constexpr size_t kTotal = kUOff + kUStages * kUnits + 1024;   // + alignment slack
+  static_assert((size_t)N * kHLd * 2 <= kBStages * kB, "SwiGLU staging");
+  // tensor memory: two A stages of 64 columns behind the accumulator ring
+  static constexpr int kDStages = N == 128 ? 3 : N == 64 ? 6 : 8;
+  static constexpr uint32_t kACol = kDStages * N;
+  static constexpr uint32_t kCols = 512;
+  static_assert(kACol + kAStages * 64 <= kCols, "tensor memory");
+  // Two threads issue steps in turn and may be a step apart: an accumulator's
+  // barrier must not be two phases behind the one that is waited for (parity
+  // waits could not tell). A thread that issues accumulator q has issued q - G
+  // - 1 or later before, so q - G - 1 - kDStages has been read; q - 2 kDStages
+  // must be no later.
+  static_assert(kDStages >= GPU + 1, "accumulator ring");
 };
 
 // Shared-memory matrix descriptor, K-major with the 128-byte swizzle: 8-row
@@ -82,11 +104,30 @@ __device__ __forceinline__ uint32_t instr_desc() {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, bool acc) {
+// One lane of the converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
+// A in tensor memory, B in shared memory.
+__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, bool acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)acc)
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"((uint32_t)acc)
+      : "memory");
+}
+
+// 16 lanes x 32 columns: register 4 i + 2 h + e of a lane goes to row
+// lane / 4 + 8 h, column 8 i + 2 (lane % 4) + e.
+__device__ __forceinline__ void tc_st16x256x4(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+      "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
 
@@ -96,9 +137,9 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                : "memory");
 }
 
-// 16 consecutive fp32 columns of this thread's tensor-memory lane (into v[0..15]).
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[16];
+// W (8 or 16) consecutive fp32 columns of this thread's tensor-memory lane; the
+// registers are not to be read before tc_ld_wait.
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
       "[%16];"
@@ -106,9 +147,18 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[32]) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
+}
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+template <int W>
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[W]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < W; ++i) asm volatile("" : "+r"(r[i]));  // not read before the wait
 }
 
 // 2-D tensor copy of one box into shared memory, completion on `bar`.
@@ -120,15 +170,8 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// Offset of element (row, k) of an operand tile of `rows` rows x 128 inputs,
-// 128-byte swizzled K-major: [64-input half][row][128 B], chunk c at c ^ (row % 8).
-__device__ __forceinline__ uint32_t op_off(int rows, int row, int k) {
-  return (uint32_t)(k >> 6) * (uint32_t)(rows * 128) + (uint32_t)row * 128u +
-         (uint32_t)((((k >> 3) & 7) ^ (row & 7)) << 4) + (uint32_t)(k & 7) * 2u;
-}
-
 // Kernel arguments: the projection and the tensor map of its activations
-// (fp16 [S][act_ld], box 8 inputs x N tokens).
+// (fp16 [S][act_ld] in act_pos order).
 struct TcParams {
   GemmArgs a;
   CUtensorMap act_map;  // {K inputs, S tokens}, box 64 x N, 128-byte swizzle
@@ -141,49 +184,37 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
   constexpr int UB = Geom<GPU>::kUnitBytes;
   constexpr int G = GPU;                        // quantisation groups per unit
   constexpr int kMmaPerGroup = 8 / GPU;         // K = 16 per instruction
-  constexpr int kHalf = N / 2;                  // token columns per epilogue thread
-  constexpr uint32_t kHalfA = kTcRows * 128, kHalfB = N * 128;  // bytes per 64-input half
-  constexpr uint32_t kColsNeed = (uint32_t)kDStages * G * N;
-  constexpr uint32_t kCols = kColsNeed <= 32 ? 32u : kColsNeed <= 64 ? 64u : kColsNeed <= 128 ? 128u
-                             : kColsNeed <= 256 ? 256u : 512u;
-  static_assert(kColsNeed <= 512, "accumulators exceed tensor memory");
-  static_assert(kHalf % 16 == 0, "columns per epilogue thread");
-  static_assert(kAStages == kDStages, "the epilogue reads the scales of its accumulator stage");
+  constexpr int kPer = N / (kEpiWarps / 4);     // token columns per epilogue thread
+  constexpr int kLd = kPer < 16 ? kPer : 16;    // of them, columns per load
+  constexpr int kDStages = L::kDStages;
+  constexpr uint32_t kHalfB = N * 128;          // bytes per 64-input half
+  static_assert(kPer % kLd == 0, "columns per epilogue thread");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t u_full[kUStages], u_empty[kUStages], b_full[kBStages], b_empty[kBStages];
-  __shared__ uint64_t a_full[kAStages], a_empty[kAStages], d_full[kDStages], d_empty[kDStages];
+  // u_*: a step's units; full: a step's A and B are in place; done: the MMAs up
+  // to a step's group are; d_empty: an accumulator has been read
+  __shared__ uint64_t u_full[kUStages], u_empty[kUStages], full[kBStages], done[kBStages * G], d_empty[kDStages];
   __shared__ uint32_t s_tmem;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // warp: known uniform
   const int rb0 = 2 * blockIdx.x;   // the tile's first row-block
   const int n0 = blockIdx.y * N;    // the tile's first token
-  const int steps = a.upr;
-  auto A_of = [&](int s) { return smem + L::kAOff + (size_t)s * L::kA; };
+  const int k_begin = part_start(a.upr, blockIdx.z, gridDim.z);
+  const int steps = part_start(a.upr, blockIdx.z + 1, gridDim.z) - k_begin;
   auto B_of = [&](int s) { return smem + L::kBOff + (size_t)s * L::kB; };
   auto U_of = [&](int s) { return smem + L::kUOff + (size_t)s * L::kUnits; };
-  auto Sc_of = [&](int s) { return reinterpret_cast<float*>(smem + L::kScOff + (size_t)s * L::kSc); };
   if (tid == 0) {
     for (int i = 0; i < kUStages; ++i) {
       mbar_init(&u_full[i], 1);
-      mbar_init(&u_empty[i], kDqWarps);
+      mbar_init(&u_empty[i], 4 + kEpiWarps);  // the step's dequantise set; the epilogue takes the scales from the unit
     }
-    for (int i = 0; i < kBStages; ++i) {
-      mbar_init(&b_full[i], 1);
-      mbar_init(&b_empty[i], 1);
-    }
-    for (int i = 0; i < kAStages; ++i) {
-      mbar_init(&a_full[i], kDqWarps);
-      mbar_init(&a_empty[i], 1);
-    }
-    for (int i = 0; i < kDStages; ++i) {
-      mbar_init(&d_full[i], 1);
-      mbar_init(&d_empty[i], 8);
-    }
+    for (int i = 0; i < kBStages; ++i) mbar_init(&full[i], 4 + 1);
+    for (int i = 0; i < kBStages * G; ++i) mbar_init(&done[i], 1);
+    for (int i = 0; i < kDStages; ++i) mbar_init(&d_empty[i], kEpiWarps);
     mbar_fence_init();
   }
-  if (warp == 1) {
+  if (warp == kMmaWarp0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&s_tmem)),
-                 "r"(kCols)
+                 "r"(L::kCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -192,9 +223,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
   tc_fence_after();
   const uint32_t tmem = s_tmem;
   bool ok = true;  // false once a wait gave up: the role skips the rest of its waits
+  // spinning: the suspending try_wait measured 8 % slower over the whole kernel
   auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (ok && !mbar_wait(bar, parity)) ok = false;
+    if (!ok) return;
+    uint32_t it = 0;
+    while (!mbar_test_wait(bar, parity))
+      if (++it > (1u << 26)) {
+        ok = false;
+        break;
+      }
   };
+  // the MMAs of step k, up to group gq
+  auto wait_done = [&](int k, int gq) { wait(&done[(k % kBStages) * G + gq], (k / kBStages) & 1); };
 
   if (warp == 0) {
     // ---- producer: units and token tiles, kUStages / kBStages steps ahead ----
@@ -205,148 +245,179 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
         mbar_arrive_expect_tx(&u_full[su], 2 * UB);
         for (int u = 0; u < 2; ++u) {
           const int rb = rb0 + u < a.n_rb ? rb0 + u : rb0;  // a missing second block repeats the first (unused)
-          bulk_g2s(U_of(su) + (size_t)u * UB, a.units + ((size_t)rb * a.upr + k) * UB, UB, &u_full[su]);
+          bulk_g2s(U_of(su) + (size_t)u * UB, a.units + ((size_t)rb * a.upr + k_begin + k) * UB, UB, &u_full[su]);
         }
-        wait(&b_empty[sb], ((k / kBStages) & 1) ^ 1);
-        mbar_arrive_expect_tx(&b_full[sb], N * 256);
+        if (k >= kBStages) wait_done(k - kBStages, G - 1);
+        mbar_arrive_expect_tx(&full[sb], N * 256);
         for (int h = 0; h < 2; ++h)  // tokens past S read as zero
-          tma_load_2d(B_of(sb) + (size_t)h * kHalfB, &P.act_map, k * kUnitK + h * 64, n0, &b_full[sb]);
+          tma_load_2d(B_of(sb) + (size_t)h * kHalfB, &P.act_map, (k_begin + k) * kUnitK + h * 64, n0, &full[sb]);
       }
     }
-  } else if (warp == 1) {
-    // ---- MMA issue: one thread ----
-    if (lane == 0) {
-      for (int k = 0; k < steps; ++k) {
-        const int sa = k % kAStages, sb = k % kBStages, sd = k % kDStages;
-        wait(&a_full[sa], (k / kAStages) & 1);
-        wait(&b_full[sb], (k / kBStages) & 1);
-        wait(&d_empty[sd], ((k / kDStages) & 1) ^ 1);
-        tc_fence_after();
-        if (ok) {
-          const uint32_t aBase = smem_addr(A_of(sa)), bBase = smem_addr(B_of(sb));
+  } else if (warp >= kMmaWarp0 && warp < kMmaWarp0 + kMmaWarps) {
+    // ---- MMA issue: one thread per warp, steps in turn ----
+    // A step's issue is a chain of two barrier polls, 8 MMAs and a commit per
+    // group, ~1150 cycles for a thread alone (more with a commit each for A, B
+    // and the accumulator): two threads overlap it. Steps need no order among
+    // themselves: each group starts a fresh accumulator.
+    {
+      const bool leader = elect_one();
+      for (int k = warp - kMmaWarp0; k < steps; k += kMmaWarps) {
+        const int sa = k % kAStages, sb = k % kBStages;
+        const uint32_t aBase = tmem + L::kACol + (uint32_t)sa * 64u;
+        const uint64_t bDesc = smem_desc_sw128(smem_addr(B_of(sb)));  // advanced by 16-byte units
+        wait(&full[sb], (k / kBStages) & 1);
 #pragma unroll
-          for (int gq = 0; gq < G; ++gq)
+        for (int gq = 0; gq < G; ++gq) {
+          const int q = k * G + gq, sd = q % kDStages;
+          if (q >= kDStages) wait(&d_empty[sd], ((q / kDStages) & 1) ^ 1);
+          tc_fence_after();
+          if (ok && leader) {
 #pragma unroll
             for (int i = 0; i < kMmaPerGroup; ++i) {
-              const int kk = gq * kMmaPerGroup + i;  // K = 16: inputs 16 kk .. + 15
-              const uint32_t ko = (uint32_t)(kk & 3) * 32u;  // inside the 64-input half
-              tc_mma(tmem + (uint32_t)((sd * G + gq) * N), smem_desc_sw128(aBase + (kk >> 2) * kHalfA + ko),
-                     smem_desc_sw128(bBase + (kk >> 2) * kHalfB + ko), instr_desc<N>(), i > 0);
+              const int kk = gq * kMmaPerGroup + i;          // K = 16: 8 columns of A, 32 bytes of a 64-input half of B
+              tc_mma(tmem + (uint32_t)(sd * N), aBase + 8u * kk, bDesc + (((kk >> 2) * kHalfB + (kk & 3) * 32u) >> 4),
+                     instr_desc<N>(), i > 0);
             }
+          }
+          if (leader) tc_commit(&done[sb * G + gq]);
+          __syncwarp();
         }
-        tc_commit(&a_empty[sa]);
-        tc_commit(&b_empty[sb]);
-        tc_commit(&d_full[sd]);
       }
     }
   } else if (warp >= kDqWarp0) {
-    // ---- dequantise: exact fp16 (q - z) into the A tile ----
-    const int dt = (warp - kDqWarp0) * 32 + lane;
-    const int gid = dt & 7, tig = (dt >> 3) & 3;  // 8 consecutive threads: rows gid 0..7 of one K chunk
-    const int l = gid * 4 + tig;                  // the fragment lane whose words this thread takes
-    for (int k = 0; k < steps; ++k) {
+    // ---- dequantise: exact fp16 (q - z) into the A stage ----
+    // the warp's tensor-memory lanes are 32 (warp % 4) .. + 31: two 16-row
+    // tiles of one unit
+    const int quad = warp & 3, u = quad >> 1, gid = lane >> 2;
+    for (int k = (warp - kDqWarp0) >> 2; k < steps; k += kDqSets) {
       const int su = k % kUStages, sa = k % kAStages;
+      const uint8_t* U = U_of(su) + (size_t)u * UB;
       wait(&u_full[su], (k / kUStages) & 1);
-      wait(&a_empty[sa], ((k / kAStages) & 1) ^ 1);
-      wait(&d_empty[sa], ((k / kAStages) & 1) ^ 1);  // the epilogue is done with this stage's scales
-      const uint8_t* Us = U_of(su);
-      uint8_t* As = A_of(sa);
-      // the step's fp32 scales [group][tile row], for the epilogue
-      for (int e = dt; e < G * kTcRows; e += kDqWarps * 32) {
-        const int gq = e / kTcRows, r = e % kTcRows, R = r & 63;
-        const int sidx = (R & 7) * 8 + ((R >> 4) & 3) * 2 + ((R >> 3) & 1);
-        Sc_of(sa)[e] = h2f(reinterpret_cast<const uint16_t*>(Us + (size_t)(r >> 6) * UB + kCodeBytes +
-                                                            gq * kMetaBytesPerGroup)[sidx]);
-      }
 #pragma unroll
-      for (int i = 0; i < 16 / kDqWarps; ++i) {
-        const int uf = (warp - kDqWarp0) + kDqWarps * i;  // (unit, code tile) 0..15
-        const int u = uf >> 3, ft = uf & 7, rt = ft & 3, kh = ft >> 2;
-        const uint8_t* U = Us + (size_t)u * UB;
-        const uint4 w4 = *reinterpret_cast<const uint4*>(U + ft * 512 + l * 16);
-        const uint32_t wv[4] = {w4.x, w4.y, w4.z, w4.w};
-        const int row = 64 * u + 16 * rt + gid;
-        uint32_t lo[2][4], hi[2][4];  // [K chunk: j / 2][4 fp16 pairs]
-        uint32_t zsub[2], zfma[2];     // per K chunk (its 8 inputs lie in one group)
+      for (int kh = 0; kh < 2; ++kh) {  // 64 inputs at a time
+        uint32_t r[2][16];
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const uint8_t* meta = U + kCodeBytes + ((64 * kh + 32 * c + 8 * tig) / (kUnitK / G)) * kMetaBytesPerGroup;
-          const uint16_t zz = *reinterpret_cast<const uint16_t*>(meta + 128 + gid * 8 + rt * 2);
-          zsub[c] = (0x6400u | (zz & 0xFFu)) * 0x00010001u;  // fp16x2 (1024 + z)
-          zfma[c] = (0xD400u | (zz >> 8)) * 0x00010001u;     // fp16x2 -(64 + z)
+        for (int i = 0; i < 2; ++i) {
+          const int rt = 2 * (quad & 1) + i;
+          const uint4 w4 = *reinterpret_cast<const uint4*>(U + (kh * 4 + rt) * 512 + lane * 16);
+          const uint32_t wv[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            // word j: rows gid and gid + 8 at inputs 64 kh + 32 (j / 2) + 8 (lane % 4) + 4 (j % 2) .. + 3
+            const uint32_t zz = *reinterpret_cast<const uint16_t*>(  // z of row gid, 16 z of row gid + 8
+                U + kCodeBytes + ((64 * kh + 32 * (j >> 1)) / (kUnitK / G)) * kMetaBytesPerGroup + 128 + gid * 8 + rt * 2);
+            const uint32_t zs = (0x6400u | (zz & 0xFFu)) * 0x00010001u;  // fp16x2 (1024 + z)
+            const uint32_t zf = (0xD400u | (zz >> 8)) * 0x00010001u;     // fp16x2 -(64 + z)
+            const uint32_t w = wv[j], w2 = w >> 8;
+            r[i][4 * j] = hsub2_u32(lop3_and_or(w, 0x000F000Fu, 0x64006400u), zs);
+            r[i][4 * j + 1] = hsub2_u32(lop3_and_or(w2, 0x000F000Fu, 0x64006400u), zs);
+            r[i][4 * j + 2] = hfma2_u32(lop3_and_or(w, 0x00F000F0u, 0x64006400u), 0x2C002C00u, zf);
+            r[i][4 * j + 3] = hfma2_u32(lop3_and_or(w2, 0x00F000F0u, 0x64006400u), 0x2C002C00u, zf);
+          }
         }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          // word j: rows gid and gid + 8 at inputs 64 kh + 32 (j / 2) + 8 tig + 4 (j % 2) .. + 3
-          const uint32_t w = wv[j], w2 = w >> 8;
-          const uint32_t zs = zsub[j >> 1], zf = zfma[j >> 1];
-          lo[j >> 1][2 * (j & 1)] = hsub2_u32(lop3_and_or(w, 0x000F000Fu, 0x64006400u), zs);
-          lo[j >> 1][2 * (j & 1) + 1] = hsub2_u32(lop3_and_or(w2, 0x000F000Fu, 0x64006400u), zs);
-          hi[j >> 1][2 * (j & 1)] = hfma2_u32(lop3_and_or(w, 0x00F000F0u, 0x64006400u), 0x2C002C00u, zf);
-          hi[j >> 1][2 * (j & 1) + 1] = hfma2_u32(lop3_and_or(w2, 0x00F000F0u, 0x64006400u), 0x2C002C00u, zf);
-        }
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const int kb = 64 * kh + 32 * c + 8 * tig;  // the 8-input chunk's first input
-          *reinterpret_cast<uint4*>(As + op_off(kTcRows, row, kb)) = make_uint4(lo[c][0], lo[c][1], lo[c][2], lo[c][3]);
-          *reinterpret_cast<uint4*>(As + op_off(kTcRows, row + 8, kb)) =
-              make_uint4(hi[c][0], hi[c][1], hi[c][2], hi[c][3]);
-        }
+        if (kh == 0 && k >= kAStages) wait_done(k - kAStages, G - 1);
+        __syncwarp();
+        if (kh == 0) tc_fence_after();
+        const uint32_t at = tmem + ((uint32_t)(32 * quad) << 16) + L::kACol + (uint32_t)sa * 64u + 32u * kh;
+        tc_st16x256x4(at, r[0]);
+        tc_st16x256x4(at + (16u << 16), r[1]);
       }
-      // the generic-proxy stores become visible to the tensor cores
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&a_full[sa]);
-        mbar_arrive(&u_empty[su]);
-      }
-    }
-  } else {
-    // ---- epilogue: scale and add each step's group sums ----
-    const int quad = warp & 3, half = (warp - kEpiWarp0) >> 2;
-    const int row = 32 * quad + lane;  // tile row = TMEM lane
-    const int c0 = half * kHalf;
-    const int R = row & 63;
-    float tot[kHalf];
-#pragma unroll
-    for (int c = 0; c < kHalf; ++c) tot[c] = 0.f;
-    for (int k = 0; k < steps; ++k) {
-      const int sd = k % kDStages;  // = the A stage: kAStages == kDStages
-      wait(&d_full[sd], (k / kDStages) & 1);
-      wait(&a_full[sd], (k / kAStages) & 1);  // the stage's scales (written before its A tile was released)
-      tc_fence_after();
-      const float* sc = Sc_of(sd);
-#pragma unroll
-      for (int gq = 0; gq < G; ++gq) {
-        const float sv = sc[gq * kTcRows + row];
-#pragma unroll
-        for (int cc = 0; cc < kHalf; cc += 16) {
-          float v[32];
-          tc_ld16(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)((sd * G + gq) * N + c0 + cc), v);
-#pragma unroll
-          for (int c = 0; c < 16; ++c) tot[cc + c] = fmaf(sv, v[c], tot[cc + c]);
-        }
-      }
+      if (lane == 0) mbar_arrive(&u_empty[su]);
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&d_empty[sd]);
+      if (lane == 0) mbar_arrive(&full[k % kBStages]);
     }
-    // outputs: natural row order, [token][row]
+  } else if (warp >= kEpiWarp0) {
+    // ---- epilogue: scale and add each step's group sums ----
+    const int quad = warp & 3;
+    const int row = 32 * quad + lane;  // tile row = TMEM lane
+    const int c0 = ((warp - kEpiWarp0) >> 2) * kPer;
+    const int R = row & 63;
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)c0;
+    const int sidx = (R & 7) * 8 + ((R >> 4) & 3) * 2 + ((R >> 3) & 1);
+    float tot[kPer];
+#pragma unroll
+    for (int c = 0; c < kPer; ++c) tot[c] = 0.f;
+    float sc[G];  // the step's scales; the next step's load behind its sums
+    auto load = [&](int k) {
+      const int su = k % kUStages;
+      wait(&u_full[su], (k / kUStages) & 1);
+#pragma unroll
+      for (int gq = 0; gq < G; ++gq)
+        sc[gq] = h2f(reinterpret_cast<const uint16_t*>(U_of(su) + (size_t)(row >> 6) * UB + kCodeBytes +
+                                                      gq * kMetaBytesPerGroup)[sidx]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&u_empty[su]);
+    };
+    load(0);
+    int q = 0;
+    for (int k = 0; k < steps; ++k) {
+#pragma unroll
+      for (int gq = 0; gq < G; ++gq, ++q) {
+        const int sd = q % kDStages;
+        wait_done(k, gq);
+        __syncwarp();
+        tc_fence_after();
+        const uint32_t at = lane_base + (uint32_t)(sd * N);
+        uint32_t v[2][kLd];
+        tc_ld(at, v[0]);
+#pragma unroll
+        for (int i = 0; i < kPer / kLd; ++i) {
+          tc_ld_wait(v[i & 1]);
+          if (i + 1 < kPer / kLd) tc_ld(at + (i + 1) * kLd, v[(i & 1) ^ 1]);
+#pragma unroll
+          for (int c = 0; c < kLd; ++c) tot[i * kLd + c] = fmaf(sc[gq], __uint_as_float(v[i & 1][c]), tot[i * kLd + c]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&d_empty[sd]);
+      }
+      if (k + 1 < steps) load(k + 1);
+    }
     const int rbr = rb0 + (row >> 6);
-    if (rbr < a.n_rb) {
+    if (a.h) {
+      // SwiGLU: gate row 16 t + r and up row 16 t + r + 8 of a block (8 lanes
+      // apart) give h index 32 rb + 8 t + r. Through shared memory (every copy
+      // into it is done: the last accumulator is), then whole 16-byte pieces.
+      uint16_t* hs = reinterpret_cast<uint16_t*>(smem);
+      const int t = R >> 4, pos = 32 * (row >> 6) + act_pos(8 * t + (R & 7));
+#pragma unroll
+      for (int c = 0; c < kPer; ++c) {
+        const float up = __shfl_down_sync(0xffffffffu, tot[c], 8);
+        if (!(R & 8)) hs[(c0 + c) * L::kHLd + pos] = f2h(silu(tot[c]) * up);
+      }
+      named_bar_sync(1, kEpiWarps * 32);
+      // positions past F (of the last, ragged block) stay as they are: zero
+      for (int e = tid - kEpiWarp0 * 32; e < N * 8; e += kEpiWarps * 32) {
+        const int c = e >> 3, j = 8 * (e & 7);
+        const int blk = rb0 + (j >> 5);
+        if (blk >= a.n_rb || n0 + c >= a.S) continue;
+        const uint16_t* src = hs + c * L::kHLd + j;
+        uint16_t* dst = a.h + (size_t)(n0 + c) * a.h_ld + 32 * blk + (j & 31);
+        if (32 * blk + 32 <= a.F) {
+          *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(src);
+        } else {
+          for (int i = 0; i < 8; ++i)
+            if (32 * blk + act_unpos((j & 31) + i) < a.F) dst[i] = src[i];
+        }
+      }
+    } else if (rbr < a.n_rb) {
+      // natural row order, [part of K][token][row]
       const int nat = natural_row(a.dims, rbr * kRowsPerBlock + R);
+      float* y = a.y + (size_t)blockIdx.z * a.y_part;
       if (nat >= 0)
 #pragma unroll
-        for (int c = 0; c < kHalf; ++c)
-          if (n0 + c0 + c < a.S) a.y[(size_t)(n0 + c0 + c) * a.y_ld + nat] = tot[c];
+        for (int c = 0; c < kPer; ++c)
+          if (n0 + c0 + c < a.S) y[(size_t)(n0 + c0 + c) * a.y_ld + nat] = tot[c];
     }
   }
   if (!ok) atomicOr(a.status, ST_WAIT_TIMEOUT);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+  if (warp == kMmaWarp0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(L::kCols) : "memory");
 }
 
 // cuTensorMapEncodeTiled, from the driver through the runtime (no link
@@ -373,8 +444,8 @@ cudaError_t launch_tc(const GemmArgs& a, cudaStream_t s) {
   using L = TcSmem<N, GPU>;
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return cudaErrorNotSupported;
-  // the activations: fp16 [S][act_ld] (16-byte aligned rows); box = 8
-  // inputs (16 bytes) x N tokens; tokens past S read as zero
+  // the activations: fp16 [S][act_ld] (16-byte aligned rows); box = 64
+  // inputs (128 bytes) x N tokens; tokens past S read as zero
   if ((reinterpret_cast<uintptr_t>(a.act) & 15) || a.act_ld % 8 || a.upr * kUnitK > a.act_ld || a.S < 1)
     return cudaErrorInvalidValue;
   TcParams p;
@@ -387,7 +458,7 @@ cudaError_t launch_tc(const GemmArgs& a, cudaStream_t s) {
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  const dim3 grid((a.n_rb + 1) / 2, (a.S + N - 1) / N);
+  const dim3 grid((a.n_rb + 1) / 2, (a.S + N - 1) / N, a.parts);
   gemm_tc_kernel<N, GPU><<<grid, kTcThreads, L::kTotal, s>>>(p);
   return cudaGetLastError();
 }
@@ -415,8 +486,23 @@ cudaError_t gemm_tc_setup() {
 
 // Token tile: 128 for long prompts, smaller for short ones; at group 32 (four
 // accumulators per step) at most 64.
-int gemm_tc_tile(int S) { return S > 64 ? 128 : S > 32 ? 64 : 32; }
-int gemm_tc_tile(int S, int group) { return group == 32 ? (S > 32 ? 64 : 32) : gemm_tc_tile(S); }
+int gemm_tc_tile(int S, int group) { return S > 64 && group != 32 ? 128 : S > 32 ? 64 : 32; }
+
+// Parts of K for a projection of n_rb row-blocks and upr units on `sms` SMs:
+// the split whose last CTA finishes first, counting whole rounds of CTAs and,
+// per CTA, about 6 steps' worth of filling the pipeline and writing the tile
+// (o projection of 8B, 77 tokens: 32 CTAs of 32 steps -> 128 of 8).
+int gemm_tc_parts(int n_rb, int upr, int S, int group, int sms) {
+  const int N = gemm_tc_tile(S, group);
+  const long long tiles = (long long)((n_rb + 1) / 2) * ((S + N - 1) / N);
+  int best = 1;
+  long long cost = 0;
+  for (int ks = 1; ks <= kGemmMaxParts && 4 * ks <= upr; ++ks) {
+    const long long c = (tiles * ks + sms - 1) / sms * ((upr + ks - 1) / ks + 6);
+    if (ks == 1 || c < cost) best = ks, cost = c;
+  }
+  return best;
+}
 
 cudaError_t launch_gemm_tc(const GemmArgs& a, int group, cudaStream_t s) {
   const int N = gemm_tc_tile(a.S, group);

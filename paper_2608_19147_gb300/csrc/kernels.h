@@ -163,26 +163,43 @@ cudaError_t launch_gemv(const GemvArgs& a, int nt, int group, int grid, cudaStre
 cudaError_t gemv_setup();
 int gemv_warps_per_cta();
 
-// Many-token projection on the tensor cores (gemm_tc.cu): y[n][natural
-// row] = sum_k W[r][k] act[n][k] for n < S.
+// Order of the many-token projection's activations: within each block of 32
+// inputs, input k is kept at act_pos(k) (chunks of 4 inputs in the order 0 2 4
+// 6 1 3 5 7; see gemm_tc.cu), and position p holds input act_unpos(p).
+__host__ __device__ constexpr int act_pos(int k) { return 16 * ((k >> 2) & 1) + 4 * ((k >> 3) & 3) + (k & 3); }
+__host__ __device__ constexpr int act_unpos(int p) { return 8 * ((p >> 2) & 3) + 4 * (p >> 4) + (p & 3); }
+
+// Many-token projection on the tensor cores (gemm_tc.cu), K in `parts` parts:
+// y[p][n][natural row] = the part's sum_k W[r][k] act[n][k] for n < S, or for
+// gate|up (h given; one part) h[n][act_pos(j)] = fp16(silu(gate) * up).
 struct GemmArgs {
   const uint8_t* units;
   int n_rb, upr;
-  const uint16_t* act;  // fp16 [S][act_ld], act_ld a multiple of 128, zero padded past K
-  int act_ld, S;
-  float* y;             // fp32 [S][y_ld]
+  const uint16_t* act;  // fp16 [S][act_ld] in act_pos order, act_ld a multiple of 128, zero padded past K
+  int act_ld, S, parts;
+  float* y;             // fp32 [parts][S][y_ld], parts y_part values apart
   int y_ld;
+  size_t y_part;
+  uint16_t* h;          // or fp16 [S][h_ld], zero past F
+  int h_ld, F;
   OpDims dims;
   int* status;
 };
 cudaError_t gemm_tc_setup();
-int gemm_tc_tile(int S);
+int gemm_tc_tile(int S, int group);
+// Parts of K for a projection of S tokens on `sms` SMs, at most kGemmMaxParts.
+constexpr int kGemmMaxParts = 4;
+int gemm_tc_parts(int n_rb, int upr, int S, int group, int sms);
 cudaError_t launch_gemm_tc(const GemmArgs& a, int group, cudaStream_t s);
+// out[t][act_pos order] = x[t][k], k < Kp (a multiple of 128).
+cudaError_t launch_act_order(const uint16_t* x, int x_ld, int S, int Kp, uint16_t* out, int out_ld, cudaStream_t s);
 
 // Prefill (prefill.cu): per-token kernels around the tensor-core projections.
 struct PrefillLayerArgs {
-  const float* y;        // q|k|v projection outputs [S][y_ld], natural rows
-  int y_ld, S, Hq, Hkv, d;
+  const float* y;        // q|k|v projection outputs [parts][S][y_ld], natural rows
+  int y_ld, parts;
+  size_t y_part;
+  int S, Hq, Hkv, d;
   const int* pos;        // [S] RoPE positions
   int max_position;
   const float2* rope;    // [max_position][d/2]
@@ -193,19 +210,31 @@ struct PrefillLayerArgs {
   const int* bt_row;     // the row's beam table
   const uint8_t* mask;   // the row's attention mask
   int P;                 // entries before the first token of this chunk
-  uint16_t* attn;        // [S][attn_ld] fp16 attention output
+  uint16_t* attn;        // [S][attn_ld] fp16 attention output, act_pos order
   int attn_ld;
+};
+// The residual stream x [S][H] and the norm that follows it.
+struct PrefillNormArgs {
+  const uint16_t* hidden_in;  // first call of a chunk: the input rows, or
+  const int* token_ids;       // the token ids (with embedding), both null later:
+  const uint16_t* embedding;
+  int vocab;
+  const float* y;             // x += sum of the projection's parts [parts][S][H]
+  int parts;
+  size_t y_part;
+  float* x;
+  int H, S;
+  const uint16_t* w;          // norm weight: act = fp16(norm(x) * w), act_pos order
+  float eps;
+  uint16_t* act;
+  int act_ld;
+  uint16_t* out;              // or, after the last layer (w null): out = fp16(x)
 };
 cudaError_t launch_prefill_check(const int* token_ids, int vocab, const int* pos, int max_position, const uint8_t* mask,
                                  int P, int S, int* status, cudaStream_t s);
-cudaError_t launch_prefill_embed(const uint16_t* hidden_in, const int* token_ids, const uint16_t* embedding, int H,
-                                 int S, int vocab, float* x, cudaStream_t s);
-cudaError_t launch_prefill_norm(const float* x, int H, const uint16_t* w, float eps, uint16_t* act, int act_ld, int S,
-                                cudaStream_t s);
+cudaError_t launch_prefill_norm(const PrefillNormArgs& a, cudaStream_t s);
 cudaError_t launch_prefill_rope_append(const PrefillLayerArgs& a, cudaStream_t s);
 cudaError_t launch_prefill_attention(const PrefillLayerArgs& a, cudaStream_t s);
-cudaError_t launch_prefill_swiglu(const float* y, int y_ld, int S, int F, uint16_t* h, int h_ld, cudaStream_t s);
-cudaError_t launch_prefill_residual(float* x, const float* y, int y_ld, int S, int H, uint16_t* out, cudaStream_t s);
 cudaError_t launch_set_int(int* p, int v, cudaStream_t s);
 
 struct PrologueArgs {

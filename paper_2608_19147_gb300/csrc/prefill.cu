@@ -7,6 +7,8 @@
 // contractions here and run on the tensor cores (gemm_tc.cu), the attention on
 // mma.sync over blocks of tokens (prefill_flash_kernel); the rest are small
 // per-token kernels, launched layer by layer on the caller's stream.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace shard {
@@ -34,95 +36,160 @@ __global__ void prefill_check_kernel(const int* token_ids, int vocab, const int*
 
 __global__ void set_int_kernel(int* p, int v) { *p = v; }
 
-// x[t][k] = fp32 of the step's fp16 input rows (hidden_in, or embedding rows).
-__global__ void prefill_embed_kernel(const uint16_t* hidden_in, const int* token_ids, const uint16_t* embedding,
-                                     int H, int S, int vocab, float* x) {
-  const size_t n = (size_t)S * H;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int t = (int)(e / H), k = (int)(e % H);
-    int tok = 0;
-    if (!hidden_in) {
-      tok = __ldg(token_ids + t);
-      tok = tok < 0 || tok >= vocab ? 0 : tok;  // out-of-range ids were flagged by the check; read a valid row
+// One CTA per token: the residual x[t] (first the input row, later x[t] plus the
+// parts of the projection before it), then act[t] = fp16(x r w) with
+// r = 1 / sqrt(mean(x^2) + eps), or after the last layer out[t] = fp16(x).
+// One pass over the row: kP pieces (float4) per thread stay in registers
+// between the sum of squares and the scaling, the rest of a longer row is read
+// back.  Bound by its L2 traffic (20 bytes per value with one part); residual
+// add and norm apart moved 28 and took two launches.
+constexpr int kNormThreads = 256;
+__global__ void __launch_bounds__(kNormThreads) prefill_norm_kernel(const __grid_constant__ PrefillNormArgs a) {
+  constexpr int kP = 8;
+  __shared__ float s_part[kNormThreads / 32];
+  const int t = blockIdx.x, tid = threadIdx.x, H4 = a.H / 4;
+  float4* xr = reinterpret_cast<float4*>(a.x + (size_t)t * a.H);
+  const uint16_t* in = nullptr;
+  if (a.hidden_in) {
+    in = a.hidden_in + (size_t)t * a.H;
+  } else if (a.token_ids) {
+    const int tok = __ldg(a.token_ids + t);  // out-of-range ids were flagged by the check; read a valid row
+    in = a.embedding + (size_t)(tok < 0 || tok >= a.vocab ? 0 : tok) * a.H;
+  }
+  // the caller's buffers may be aligned to their values only
+  const bool in8 = reinterpret_cast<uintptr_t>(in) % 8 == 0, out8 = reinterpret_cast<uintptr_t>(a.out) % 8 == 0;
+  auto get = [&](int c) {
+    if (in && !in8) return make_float4(h2f(in[4 * c]), h2f(in[4 * c + 1]), h2f(in[4 * c + 2]), h2f(in[4 * c + 3]));
+    if (in) {
+      const uint2 u = *reinterpret_cast<const uint2*>(in + 4 * c);
+      return make_float4(h2f(u.x & 0xFFFFu), h2f(u.x >> 16), h2f(u.y & 0xFFFFu), h2f(u.y >> 16));
     }
-    const uint16_t v = hidden_in ? hidden_in[e] : embedding[(size_t)tok * H + k];
-    x[e] = h2f(v);
+    float4 v = xr[c];
+    for (int p = 0; p < a.parts; ++p) {
+      const float4 y = *(reinterpret_cast<const float4*>(a.y + p * a.y_part + (size_t)t * a.H) + c);
+      v.x += y.x;
+      v.y += y.y;
+      v.z += y.z;
+      v.w += y.w;
+    }
+    return v;
+  };
+  auto halves = [](float4 v) {
+    return make_uint2((uint32_t)f2h(v.x) | ((uint32_t)f2h(v.y) << 16), (uint32_t)f2h(v.z) | ((uint32_t)f2h(v.w) << 16));
+  };
+  if (!a.w) {
+    for (int c = tid; c < H4; c += kNormThreads) {
+      const uint2 u = halves(get(c));
+      uint16_t* o = a.out + (size_t)t * a.H + 4 * c;
+      if (out8) {
+        *reinterpret_cast<uint2*>(o) = u;
+      } else {
+        o[0] = (uint16_t)u.x;
+        o[1] = (uint16_t)(u.x >> 16);
+        o[2] = (uint16_t)u.y;
+        o[3] = (uint16_t)(u.y >> 16);
+      }
+    }
+    return;
   }
-}
-
-// act[t][k] = fp16(x[t][k] * r[t] * w[k]), r = 1 / sqrt(mean(x[t]^2) + eps);
-// one CTA per token.
-__global__ void prefill_norm_kernel(const float* x, int H, const uint16_t* w, float eps, uint16_t* act, int act_ld) {
-  __shared__ float s_part[32];
-  const int t = blockIdx.x;
-  const float* xr = x + (size_t)t * H;
+  float4 v[kP];
   float ss = 0.f;
-  for (int k = threadIdx.x; k < H; k += blockDim.x) ss = fmaf(xr[k], xr[k], ss);
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float tsum = 0.f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) tsum += s_part[i];
-    s_part[0] = rsqrtf(tsum / H + eps);
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    const int c = tid + i * kNormThreads;
+    v[i] = c < H4 ? get(c) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    const int c = tid + i * kNormThreads;
+    if (c < H4) xr[c] = v[i];
+    ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+  }
+  for (int c = tid + kP * kNormThreads; c < H4; c += kNormThreads) {
+    const float4 u = get(c);
+    xr[c] = u;
+    ss += u.x * u.x + u.y * u.y + u.z * u.z + u.w * u.w;
+  }
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if ((tid & 31) == 0) s_part[tid >> 5] = ss;
   __syncthreads();
-  const float r = s_part[0];
-  for (int k = threadIdx.x; k < H; k += blockDim.x) act[(size_t)t * act_ld + k] = f2h(xr[k] * r * h2f(w[k]));
+  float tsum = 0.f;
+  for (int i = 0; i < kNormThreads / 32; ++i) tsum += s_part[i];
+  const float r = rsqrtf(tsum / a.H + a.eps);
+  auto emit = [&](int c, float4 x) {
+    const uint2 u = *reinterpret_cast<const uint2*>(a.w + 4 * c);
+    const int k = 4 * c;
+    *reinterpret_cast<uint2*>(a.act + (size_t)t * a.act_ld + (k & ~31) + act_pos(k & 31)) =
+        halves(make_float4(x.x * r * h2f(u.x & 0xFFFFu), x.y * r * h2f(u.x >> 16), x.z * r * h2f(u.y & 0xFFFFu),
+                           x.w * r * h2f(u.y >> 16)));
+  };
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    const int c = tid + i * kNormThreads;
+    if (c < H4) emit(c, v[i]);
+  }
+  for (int c = tid + kP * kNormThreads; c < H4; c += kNormThreads) emit(c, xr[c]);
 }
 
 // RoPE (pairs (i, i + d/2), the token's position) on q (kept in fp32) and k;
 // k and v rounded to fp16 and appended to the pool at the row's next slots.
-__global__ void prefill_rope_append_kernel(const float* y, int y_ld, int S, int Hq, int Hkv, int d,
-                                           const int* pos, int max_position, const float2* rope, float* q, uint16_t* kpool,
-                                           uint16_t* vpool, int row, int cap, int slot0) {
-  const int half = d / 2;
-  const int per_tok = (Hq + Hkv) * half + Hkv * d;
-  const size_t n = (size_t)S * per_tok;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int t = (int)(e / per_tok), r = (int)(e % per_tok);
-    const float* yr = y + (size_t)t * y_ld;
-    const size_t kv = (((size_t)row * Hkv) * cap + (size_t)(slot0 + t)) * d;  // head 0's entry of this token
-    if (r < (Hq + Hkv) * half) {
-      const int h = r / half, i = r % half;
-      const int p = __ldg(pos + t);
-      const float2 cs = rope[(size_t)(p < 0 || p >= max_position ? 0 : p) * half + i];  // out-of-range positions were flagged
-      const float lo = yr[h * d + i], hi = yr[h * d + half + i];
-      const float olo = lo * cs.x - hi * cs.y, ohi = hi * cs.x + lo * cs.y;
-      if (h < Hq) {
-        q[(size_t)t * Hq * d + h * d + i] = olo;
-        q[(size_t)t * Hq * d + h * d + half + i] = ohi;
+// Four dims per thread, the projection's parts added in order.
+__global__ void __launch_bounds__(256) prefill_rope_append_kernel(const __grid_constant__ PrefillLayerArgs a) {
+  const int d = a.d, half = d / 2, h4 = half / 4;
+  const int rot = (a.Hq + a.Hkv) * h4, per_tok = rot + a.Hkv * d / 4;
+  const int n = a.S * per_tok;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int t = e / per_tok, r = e % per_tok;
+    const float* yr = a.y + (size_t)t * a.y_ld;
+    auto get = [&](int row) {
+      float4 v = *reinterpret_cast<const float4*>(yr + row);
+      for (int p = 1; p < a.parts; ++p) {
+        const float4 u = *reinterpret_cast<const float4*>(yr + p * a.y_part + row);
+        v.x += u.x;
+        v.y += u.y;
+        v.z += u.z;
+        v.w += u.w;
+      }
+      return v;
+    };
+    auto halves = [](float4 v) {
+      return make_uint2((uint32_t)f2h(v.x) | ((uint32_t)f2h(v.y) << 16), (uint32_t)f2h(v.z) | ((uint32_t)f2h(v.w) << 16));
+    };
+    const size_t kv = (((size_t)a.row * a.Hkv) * a.cap + (size_t)(a.slot0 + t)) * d;  // head 0's entry of this token
+    if (r < rot) {
+      const int h = r / h4, i = 4 * (r % h4);
+      const int p = __ldg(a.pos + t);
+      const float4* cs = reinterpret_cast<const float4*>(
+          a.rope + (size_t)(p < 0 || p >= a.max_position ? 0 : p) * half + i);  // out-of-range positions were flagged
+      const float4 c0 = cs[0], c1 = cs[1];
+      const float4 lo = get(h * d + i), hi = get(h * d + half + i);
+      const float4 olo = make_float4(lo.x * c0.x - hi.x * c0.y, lo.y * c0.z - hi.y * c0.w, lo.z * c1.x - hi.z * c1.y,
+                                     lo.w * c1.z - hi.w * c1.w);
+      const float4 ohi = make_float4(hi.x * c0.x + lo.x * c0.y, hi.y * c0.z + lo.y * c0.w, hi.z * c1.x + lo.z * c1.y,
+                                     hi.w * c1.z + lo.w * c1.w);
+      if (h < a.Hq) {
+        float* q = a.q + (size_t)t * a.Hq * d + h * d + i;
+        *reinterpret_cast<float4*>(q) = olo;
+        *reinterpret_cast<float4*>(q + half) = ohi;
       } else {
-        uint16_t* kp = kpool + kv + (size_t)(h - Hq) * cap * d;
-        kp[i] = f2h(olo);
-        kp[half + i] = f2h(ohi);
+        uint16_t* kp = a.kpool + kv + (size_t)(h - a.Hq) * a.cap * d + i;
+        *reinterpret_cast<uint2*>(kp) = halves(olo);
+        *reinterpret_cast<uint2*>(kp + half) = halves(ohi);
       }
     } else {
-      const int rv = r - (Hq + Hkv) * half, h = rv / d, i = rv % d;
-      vpool[kv + (size_t)h * cap * d + i] = f2h(yr[(Hq + Hkv) * d + h * d + i]);
+      const int rv = 4 * (r - rot), h = rv / d, i = rv % d;
+      *reinterpret_cast<uint2*>(a.vpool + kv + (size_t)h * a.cap * d + i) = halves(get((a.Hq + a.Hkv) * d + rv));
     }
   }
 }
 
-
-// h[t][j] = fp16(silu(gate) * up); y holds gate (0..F) then up (F..2F).
-__global__ void prefill_swiglu_kernel(const float* y, int y_ld, int S, int F, uint16_t* h, int h_ld) {
-  const size_t n = (size_t)S * F;
+// Activations in natural order to act_pos order (the test export's input).
+__global__ void act_order_kernel(const uint16_t* x, int x_ld, int S, int Kp, uint16_t* out, int out_ld) {
+  const size_t n = (size_t)S * Kp / 4;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int t = (int)(e / F), j = (int)(e % F);
-    const float g = y[(size_t)t * y_ld + j], u = y[(size_t)t * y_ld + F + j];
-    h[(size_t)t * h_ld + j] = f2h(g / (1.f + expf(-g)) * u);
-  }
-}
-
-// x += y (the residual stream); on the last layer also hidden_out = fp16(x).
-__global__ void prefill_residual_kernel(float* x, const float* y, int y_ld, int S, int H, uint16_t* out) {
-  const size_t n = (size_t)S * H;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    const int t = (int)(e / H), k = (int)(e % H);
-    const float v = x[e] + y[(size_t)t * y_ld + k];
-    x[e] = v;
-    if (out) out[e] = f2h(v);
+    const int t = (int)(e / (Kp / 4)), k = 4 * (int)(e % (Kp / 4));
+    *reinterpret_cast<uint2*>(out + (size_t)t * out_ld + (k & ~31) + act_pos(k & 31)) =
+        *reinterpret_cast<const uint2*>(x + (size_t)t * x_ld + k);
   }
 }
 
@@ -295,13 +362,16 @@ __global__ void __launch_bounds__(128) prefill_flash_kernel(const float* q, int 
   }
   const float ia = l_a > 0.f ? 1.f / l_a : 0.f, ib = l_b > 0.f ? 1.f / l_b : 0.f;
 #pragma unroll
-  for (int nd = 0; nd < ND; ++nd)
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int dcol = 8 * nd + 2 * tig + c;
-      if (tok_a < S) out[(size_t)tok_a * out_ld + (hk * G + ra % G) * D + dcol] = f2h(o[nd][c] * ia);
-      if (tok_b < S) out[(size_t)tok_b * out_ld + (hk * G + rb % G) * D + dcol] = f2h(o[nd][2 + c] * ib);
-    }
+  for (int nd = 0; nd < ND; ++nd) {
+    const int dcol = 8 * nd + 2 * tig;
+    const int col = (dcol & ~31) + act_pos(dcol & 31);  // the o projection's order (heads are whole 32-blocks)
+    if (tok_a < S)
+      *reinterpret_cast<uint32_t*>(out + (size_t)tok_a * out_ld + (hk * G + ra % G) * D + col) =
+          (uint32_t)f2h(o[nd][0] * ia) | ((uint32_t)f2h(o[nd][1] * ia) << 16);
+    if (tok_b < S)
+      *reinterpret_cast<uint32_t*>(out + (size_t)tok_b * out_ld + (hk * G + rb % G) * D + col) =
+          (uint32_t)f2h(o[nd][2] * ib) | ((uint32_t)f2h(o[nd][3] * ib) << 16);
+  }
 }
 
 template <int D, int G>
@@ -325,24 +395,20 @@ cudaError_t launch_set_int(int* p, int v, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_prefill_embed(const uint16_t* hidden_in, const int* token_ids, const uint16_t* embedding, int H,
-                                 int S, int vocab, float* x, cudaStream_t s) {
-  prefill_embed_kernel<<<(int)std::min<size_t>(((size_t)S * H + 255) / 256, 4096), 256, 0, s>>>(hidden_in, token_ids,
-                                                                                                embedding, H, S, vocab, x);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_prefill_norm(const float* x, int H, const uint16_t* w, float eps, uint16_t* act, int act_ld, int S,
-                                cudaStream_t s) {
-  prefill_norm_kernel<<<S, 256, 0, s>>>(x, H, w, eps, act, act_ld);
+cudaError_t launch_prefill_norm(const PrefillNormArgs& a, cudaStream_t s) {
+  prefill_norm_kernel<<<a.S, kNormThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prefill_rope_append(const PrefillLayerArgs& a, cudaStream_t s) {
-  const size_t n = (size_t)a.S * ((a.Hq + a.Hkv) * (a.d / 2) + a.Hkv * a.d);
-  prefill_rope_append_kernel<<<(int)std::min<size_t>((n + 255) / 256, 8192), 256, 0, s>>>(
-      a.y, a.y_ld, a.S, a.Hq, a.Hkv, a.d, a.pos, a.max_position, a.rope, a.q, a.kpool, a.vpool, a.row, a.cap,
-      a.slot0);
+  const int n = a.S * ((a.Hq + a.Hkv) * (a.d / 8) + a.Hkv * a.d / 4);
+  prefill_rope_append_kernel<<<(n + 255) / 256, 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_act_order(const uint16_t* x, int x_ld, int S, int Kp, uint16_t* out, int out_ld, cudaStream_t s) {
+  act_order_kernel<<<(int)std::min<size_t>(((size_t)S * Kp / 4 + 255) / 256, 4096), 256, 0, s>>>(x, x_ld, S, Kp, out,
+                                                                                                out_ld);
   return cudaGetLastError();
 }
 
@@ -361,18 +427,6 @@ cudaError_t launch_prefill_attention(const PrefillLayerArgs& a, cudaStream_t s) 
   if (a.d == 64) { A(64) }
 #undef A
   return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_prefill_swiglu(const float* y, int y_ld, int S, int F, uint16_t* h, int h_ld, cudaStream_t s) {
-  prefill_swiglu_kernel<<<(int)std::min<size_t>(((size_t)S * F + 255) / 256, 8192), 256, 0, s>>>(y, y_ld, S, F, h,
-                                                                                                 h_ld);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_prefill_residual(float* x, const float* y, int y_ld, int S, int H, uint16_t* out, cudaStream_t s) {
-  prefill_residual_kernel<<<(int)std::min<size_t>(((size_t)S * H + 255) / 256, 4096), 256, 0, s>>>(x, y, y_ld, S, H,
-                                                                                                   out);
-  return cudaGetLastError();
 }
 
 }  // namespace shard

@@ -97,8 +97,10 @@ struct shard_s {
   uint16_t* pf_act = nullptr;      // [C][Kp_H] normalised rows (padding zero)
   uint16_t* pf_attn = nullptr;     // [C][Kp_dq] attention output (padding zero)
   uint16_t* pf_h = nullptr;        // [C][Kp_F] SwiGLU output (padding zero)
-  float* pf_y = nullptr;           // [C][max projection rows] projection outputs
+  float* pf_y = nullptr;           // [parts][C][projection rows] projection outputs
   float* pf_q = nullptr;           // [C][dq] rotated queries
+  uint16_t* dbg_act = nullptr;     // shard_debug_gemm: its input in act_pos order
+  size_t dbg_act_n = 0;
   int debug_skip_arrival = -1;     // test knob (shard_debug_set_wait)
   unsigned wait_limit = 1u << 22;  // polls before a cross-CTA wait gives up
   int* status = nullptr;           // device status word
@@ -234,6 +236,7 @@ void release_shard(shard_s* sh) {
   cudaFree(sh->pf_h);
   cudaFree(sh->pf_y);
   cudaFree(sh->pf_q);
+  cudaFree(sh->dbg_act);
   cudaFree(sh->X);
   cudaFree(sh->acc_qkv);
   cudaFree(sh->acc_gu);
@@ -848,7 +851,7 @@ static int step_impl(shard_t sh, kvstate_t st, const uint16_t* hidden_in, const 
 }
 
 // Prefill chunk: tokens per pass through the layers (buffers scale with it).
-constexpr int kPrefillChunk = 256;
+constexpr int kPrefillChunk = 512;
 
 int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, const int32_t* token_ids, int S,
                   const int32_t* position_ids, const uint8_t* attention_mask, int mask_len, uint16_t* hidden_out,
@@ -871,7 +874,7 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
   CUDA_TRY(cudaSetDevice(sh->device));
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const int C = kPrefillChunk;
-  const int y_rows = std::max(std::max(sh->dq + 2 * sh->dkv, 2 * sh->F), sh->H);
+  const size_t y_floats = (size_t)kGemmMaxParts * C * std::max(sh->dq + 2 * sh->dkv, sh->H);
   if (!sh->pf_x) {
     // all or none: a call that fails here leaves no partial set behind for
     // the next call to mistake for a complete one
@@ -881,7 +884,7 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
     if (e == cudaSuccess) e = cudaMalloc(&act, sizeof(uint16_t) * C * sh->Kp_H);
     if (e == cudaSuccess) e = cudaMalloc(&attn, sizeof(uint16_t) * C * sh->Kp_dq);
     if (e == cudaSuccess) e = cudaMalloc(&hh, sizeof(uint16_t) * C * sh->Kp_F);
-    if (e == cudaSuccess) e = cudaMalloc(&y, sizeof(float) * C * y_rows);
+    if (e == cudaSuccess) e = cudaMalloc(&y, sizeof(float) * y_floats);
     if (e == cudaSuccess) e = cudaMalloc(&q, sizeof(float) * C * sh->dq);
     if (e == cudaSuccess) e = cudaMemset(act, 0, sizeof(uint16_t) * C * sh->Kp_H);
     if (e == cudaSuccess) e = cudaMemset(attn, 0, sizeof(uint16_t) * C * sh->Kp_dq);
@@ -909,12 +912,25 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
   const float eps = static_cast<float>(sh->cfg.rms_eps);
   for (int t0 = 0; t0 < S; t0 += C) {
     const int c = std::min(C, S - t0);
-    CUDA_TRY(launch_prefill_embed(hidden_in ? hidden_in + (size_t)t0 * sh->H : nullptr,
-                                  token_ids ? token_ids + t0 : nullptr, sh->embedding, sh->H, c, sh->cfg.vocab,
-                                  sh->pf_x, s));
+    const size_t qkv_rows = sh->dq + 2 * sh->dkv;
+    // x (+)= ...; act = norm(x) * w
+    PrefillNormArgs na{};
+    na.hidden_in = hidden_in ? hidden_in + (size_t)t0 * sh->H : nullptr;
+    na.token_ids = token_ids ? token_ids + t0 : nullptr;
+    na.embedding = sh->embedding;
+    na.vocab = sh->cfg.vocab;
+    na.y = sh->pf_y;
+    na.y_part = (size_t)c * sh->H;
+    na.x = sh->pf_x;
+    na.H = sh->H;
+    na.S = c;
+    na.eps = eps;
+    na.act = sh->pf_act;
+    na.act_ld = sh->Kp_H;
     for (int l = 0; l < sh->L; ++l) {
       const uint16_t* nrm = sh->norms + (size_t)l * 2 * sh->H;
-      auto gemm = [&](int k, const uint16_t* act, int act_ld) -> cudaError_t {
+      // returns the parts of K that y holds
+      auto gemm = [&](int k, const uint16_t* act, int act_ld, int* parts) -> cudaError_t {
         const PackedOp& p = sh->ops[(size_t)l * N_OPS + k];
         GemmArgs g{};
         g.units = p.units;
@@ -923,17 +939,29 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
         g.act = act;
         g.act_ld = act_ld;
         g.S = c;
-        g.y = sh->pf_y;
-        g.y_ld = k == OP_QKV ? sh->dq + 2 * sh->dkv : k == OP_GU ? 2 * sh->F : sh->H;
+        g.parts = *parts = k == OP_GU ? 1 : gemm_tc_parts(p.n_rb, p.upr, c, sh->cfg.group, sh->num_sms);
+        if (k == OP_GU) {
+          g.h = sh->pf_h;
+          g.h_ld = sh->Kp_F;
+          g.F = sh->F;
+        } else {
+          g.y = sh->pf_y;
+          g.y_ld = k == OP_QKV ? (int)qkv_rows : sh->H;
+          g.y_part = (size_t)c * g.y_ld;
+        }
         g.dims = p.dims;
         g.status = sh->status;
         return launch_gemm_tc(g, sh->cfg.group, s);
       };
-      CUDA_TRY(launch_prefill_norm(sh->pf_x, sh->H, nrm, eps, sh->pf_act, sh->Kp_H, c, s));
-      CUDA_TRY(gemm(OP_QKV, sh->pf_act, sh->Kp_H));
+      na.w = nrm;
+      CUDA_TRY(launch_prefill_norm(na, s));
+      na.hidden_in = nullptr;
+      na.token_ids = nullptr;
       PrefillLayerArgs pa{};
+      CUDA_TRY(gemm(OP_QKV, sh->pf_act, sh->Kp_H, &pa.parts));
       pa.y = sh->pf_y;
-      pa.y_ld = sh->dq + 2 * sh->dkv;
+      pa.y_ld = (int)qkv_rows;
+      pa.y_part = (size_t)c * qkv_rows;
       pa.S = c;
       pa.Hq = sh->Hq;
       pa.Hkv = sh->Hkv;
@@ -954,15 +982,16 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
       pa.attn_ld = sh->Kp_dq;
       CUDA_TRY(launch_prefill_rope_append(pa, s));
       CUDA_TRY(launch_prefill_attention(pa, s));
-      CUDA_TRY(gemm(OP_O, sh->pf_attn, sh->Kp_dq));
-      CUDA_TRY(launch_prefill_residual(sh->pf_x, sh->pf_y, sh->H, c, sh->H, nullptr, s));
-      CUDA_TRY(launch_prefill_norm(sh->pf_x, sh->H, nrm + sh->H, eps, sh->pf_act, sh->Kp_H, c, s));
-      CUDA_TRY(gemm(OP_GU, sh->pf_act, sh->Kp_H));
-      CUDA_TRY(launch_prefill_swiglu(sh->pf_y, 2 * sh->F, c, sh->F, sh->pf_h, sh->Kp_F, s));
-      CUDA_TRY(gemm(OP_DOWN, sh->pf_h, sh->Kp_F));
-      CUDA_TRY(launch_prefill_residual(sh->pf_x, sh->pf_y, sh->H, c, sh->H,
-                                       l + 1 == sh->L ? hidden_out + (size_t)t0 * sh->H : nullptr, s));
+      CUDA_TRY(gemm(OP_O, sh->pf_attn, sh->Kp_dq, &na.parts));
+      na.w = nrm + sh->H;
+      CUDA_TRY(launch_prefill_norm(na, s));
+      int one;
+      CUDA_TRY(gemm(OP_GU, sh->pf_act, sh->Kp_H, &one));
+      CUDA_TRY(gemm(OP_DOWN, sh->pf_h, sh->Kp_F, &na.parts));
     }
+    na.w = nullptr;
+    na.out = hidden_out + (size_t)t0 * sh->H;
+    CUDA_TRY(launch_prefill_norm(na, s));
   }
   CUDA_TRY(launch_set_int(st->lens + row, P + S, s));
   st->cursor[row] += S;
@@ -1119,13 +1148,23 @@ int shard_debug_gemm(shard_t sh, int layer, int op, const uint16_t* x, int x_ld,
     return fail(SHARD_EINVAL, "shard_debug_gemm: x_ld %d must be a multiple of 128 and >= %d; x 16-byte aligned", x_ld,
                 p.Kp);
   CUDA_TRY(cudaSetDevice(sh->device));
+  const size_t need = (size_t)S * p.Kp;
+  if (sh->dbg_act_n < need) {
+    cudaFree(sh->dbg_act);
+    sh->dbg_act = nullptr;
+    sh->dbg_act_n = 0;
+    CUDA_TRY(cudaMalloc(&sh->dbg_act, sizeof(uint16_t) * need));
+    sh->dbg_act_n = need;
+  }
+  CUDA_TRY(launch_act_order(x, x_ld, S, p.Kp, sh->dbg_act, p.Kp, static_cast<cudaStream_t>(cuda_stream)));
   GemmArgs g{};
   g.units = p.units;
   g.n_rb = p.n_rb;
   g.upr = p.upr;
-  g.act = x;
-  g.act_ld = x_ld;
+  g.act = sh->dbg_act;
+  g.act_ld = p.Kp;
   g.S = S;
+  g.parts = 1;
   g.y = y;
   g.y_ld = y_ld;
   g.dims = p.dims;
