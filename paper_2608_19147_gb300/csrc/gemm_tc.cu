@@ -11,15 +11,15 @@
 //   - warp 0 (producer): bulk-copies the step's two units (codes, scales,
 //     zero points) and loads the token tile with two 2-D tensor copies (64
 //     inputs x N tokens each, 128-byte swizzle), several stages ahead;
-//   - warps 20..27 (dequantise): turn the codes into exact fp16 (q - z) and
+//   - warps 12..19 (dequantise): turn the codes into exact fp16 (q - z) and
 //     store them to tensor memory, the A operand; two sets of four warps take
 //     the steps in turn, 2 stages;
 //   - warps 1, 2 (MMA): a thread each, steps in turn, issues tcgen05.mma
 //     (kind::f16, M = 128, N tokens, K = 16 per instruction, A in tensor memory,
 //     B in shared memory) into a ring of accumulators, one per quantisation
 //     group and step, and commits to the step's mbarrier;
-//   - warps 4..19 (epilogue): read the accumulators (tcgen05.ld; warp w owns
-//     lanes 32 (w % 4) .. + 31 = tile rows, a quarter of the token columns),
+//   - warps 4..11 (epilogue): read the accumulators (tcgen05.ld; warp w owns
+//     lanes 32 (w % 4) .. + 31 = tile rows, half the token columns each),
 //     multiply by the row's fp32 group scale and add into registers; at the
 //     end they write their rows' outputs.
 // A in tensor memory: with A in shared memory too, a step of 128 x 128 x 128 moved
@@ -33,10 +33,10 @@
 // What bounds it is the roles' own chains of barrier polls and short dependent
 // work, ~1150 cycles a step against 512 of tensor time: leaving out, one at a
 // time, the MMAs, the dequantisation's arithmetic, the epilogue's loads or the
-// copies changes a step by 2-6 %. Against the first version (A in shared memory,
-// three commits a step by one thread, suspending waits), 512 tokens at 8B width,
-// 4 layers: gate|up 225 -> 159 us per layer, o and down 73 -> 48, q|k|v 61 -> 46;
-// 604 -> 850 TFLOP/s for gate|up alone.
+// copies changes a step by 2-6 %. Per launch, 512 tokens at 8B width: gate|up
+// 225 -> 159 us, o and down 73 -> 48, q|k|v 61 -> 46 against the same kernel with
+// three commits a step by one thread, one dequantise set and suspending waits
+// (which, with A in shared memory, ran at the same ~1 us a step).
 // The token tile sits in the canonical K-major layout with the 128-byte
 // swizzle, as the tensor copy writes it. The
 // arithmetic is the decode projection's: exact (q - z), fp32 sums per group,

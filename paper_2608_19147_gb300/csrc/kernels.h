@@ -207,11 +207,13 @@ struct PrefillLayerArgs {
   uint16_t* kpool;       // this layer's K pool [n_rows][Hkv][cap][d]
   uint16_t* vpool;
   int row, cap, slot0;   // the row and the position in it of the first new entry
-  const int* bt_row;     // the row's beam table
   const uint8_t* mask;   // the row's attention mask
   int P;                 // entries before the first token of this chunk
   uint16_t* attn;        // [S][attn_ld] fp16 attention output, act_pos order
   int attn_ld;
+  float* part;           // attention partials of part_slots (block, kv head, part of the cache) triples,
+  int* part_cnt;         // finished parts per (block, kv head), zero between launches
+  int part_slots;
 };
 // The residual stream x [S][H] and the norm that follows it.
 struct PrefillNormArgs {
@@ -235,6 +237,9 @@ cudaError_t launch_prefill_check(const int* token_ids, int vocab, const int* pos
 cudaError_t launch_prefill_norm(const PrefillNormArgs& a, cudaStream_t s);
 cudaError_t launch_prefill_rope_append(const PrefillLayerArgs& a, cudaStream_t s);
 cudaError_t launch_prefill_attention(const PrefillLayerArgs& a, cudaStream_t s);
+// One-time attribute setup of the attention kernels; size of the partials.
+cudaError_t prefill_setup(int head_dim);
+size_t prefill_part_floats(int slots, int d);
 cudaError_t launch_set_int(int* p, int v, cudaStream_t s);
 
 struct PrologueArgs {

@@ -194,19 +194,37 @@ __global__ void act_order_kernel(const uint16_t* x, int x_ld, int S, int Kp, uin
 }
 
 // Causal attention of the new tokens on the tensor cores (mma.sync m16n8k16),
-// one CTA per (block of 64 / G tokens, kv head hk), 4 warps: query row r of
-// the 64 is token t0 + r / G, query head hk G + r % G, and warp w owns rows
-// 16 w .. + 15, so every K/V tile is read once for all the block's queries.
-// Entry tiles of 64 come through the beam table into shared memory.  Scores
-// S = Q K^T with Q split into fp16 hi + lo parts (together ~22 bits of q, so
-// the scores match an fp32 q); online softmax per row in fp32; O += P V with
-// P split the same way; fp32 accumulators.  Entry j is visible to token t iff
-// j <= P + t and mask[j] != 0.
+// one CTA per (block of 64 / G tokens, kv head hk, part of the cache), 4 warps:
+// query row r of the 64 is token t0 + r / G, query head hk G + r % G, and warp w
+// owns rows 16 w .. + 15, so every K/V tile is read once for all the block's
+// queries. Tiles of 64 entries (a row that may be prefilled holds its entries
+// contiguously) come into shared memory with asynchronous copies, one tile
+// ahead. Scores S = Q K^T with Q split into fp16 hi + lo parts (together ~22
+// bits of q, so the scores match an fp32 q); online softmax per row in fp32;
+// O += P V with P split the same way; fp32 accumulators. Entry j is visible to
+// token t iff j <= P + t and mask[j] != 0.
+// The bound is the tensor pipe (256 MMAs per warp and tile, ~2000 cycles) once
+// the copies run ahead, and the length of a CTA's chain of tiles when there
+// are few blocks: the cache is then cut into parts (launch_attn_t), each CTA
+// leaves (max, sum, unnormalised output) per row, and the last one of a block
+// combines them in order.
+// 8B width, per launch: 512 tokens 83 -> 47 us, 77 tokens on ~900 entries 209 -> 42
+// (before: synchronous tile loads, one CTA per block for the whole cache).
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm_x4(const void* p, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+               : "r"(smem_addr(p)));
+}
+// 16 bytes to shared memory, asynchronously; zeros if !take.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool take) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(take ? 16 : 0)
+               : "memory");
 }
 __device__ __forceinline__ void ldsm_x4_trans(const void* p, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -220,28 +238,58 @@ __device__ __forceinline__ void split_h2(float lo, float hi, uint32_t& h, uint32
   l = (uint32_t)f2h(lo - h2f(a)) | ((uint32_t)f2h(hi - h2f(b)) << 16);
 }
 
+template <int D>
+struct FlashSmem {
+  static constexpr int kLd = D + 8;  // row stride (halves): 16-byte rows, conflict-free fragment reads
+  uint16_t k[2][64][kLd], v[2][64][kLd];
+  uint8_t vis[2][64];
+};
+
 template <int D, int G>
-__global__ void __launch_bounds__(128) prefill_flash_kernel(const float* q, int Hq, int Hkv, const uint16_t* kpool,
-                                                           const uint16_t* vpool, const int* bt_row, int cap,
-                                                           const uint8_t* mask, int P, int S, uint16_t* out,
-                                                           int out_ld) {
+__global__ void __launch_bounds__(128) prefill_flash_kernel(const __grid_constant__ PrefillLayerArgs a) {
   constexpr int TB = 64 / G;  // tokens per CTA
   constexpr int KS = D / 16;  // k16 steps over the head dimension
   constexpr int ND = D / 8;   // n8 tiles over the head dimension
-  constexpr int LD = D + 8;   // shared row stride (halves): 16-byte rows, conflict-free fragment reads
-  __shared__ __align__(16) uint16_t Ks[64][LD];
-  __shared__ __align__(16) uint16_t Vs[64][LD];
-  __shared__ uint8_t vis[64];
+  extern __shared__ __align__(16) uint8_t flash_smem[];
+  __shared__ int s_last;
+  FlashSmem<D>& sm = *reinterpret_cast<FlashSmem<D>*>(flash_smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
   const int t0 = blockIdx.x * TB, hk = blockIdx.y;
+  const int P = a.P, S = a.S;
   const float scale = rsqrtf((float)D);
-  // Q rows as fp16 hi (in Ks) and lo (in Vs), then this warp's fragments
-  for (int e = tid; e < 64 * D; e += 128) {
-    const int r = e / D, c = e % D, t = t0 + r / G;
-    const float v = t < S ? q[(size_t)t * Hq * D + (hk * G + r % G) * D + c] : 0.f;
-    const uint16_t hi = f2h(v);
-    Ks[r][c] = hi;
-    Vs[r][c] = f2h(v - h2f(hi));
+  const int last = P + min(t0 + TB, S) - 1;  // the block's last token's limit
+  const int tiles = last / 64 + 1;
+  const int tile0 = tiles * (int)blockIdx.z / (int)gridDim.z, tile1 = tiles * (int)(blockIdx.z + 1) / (int)gridDim.z;
+  const uint16_t* kp = a.kpool + ((size_t)a.row * a.Hkv + hk) * a.cap * D;
+  const uint16_t* vp = a.vpool + ((size_t)a.row * a.Hkv + hk) * a.cap * D;
+  // Q rows as fp16 hi (in K's second buffer) and lo (in V's), then this warp's
+  // fragments; the first tile's copies run meanwhile
+  auto copy_tile = [&](int tile) {
+    const int buf = (tile - tile0) & 1, j0 = 64 * tile;
+    for (int e = tid; e < 64 * (D / 8); e += 128) {
+      const int r = e / (D / 8), c = e % (D / 8);
+      const bool take = j0 + r <= last;
+      const size_t off = (size_t)(take ? j0 + r : 0) * D + 8 * c;
+      cp_async16(&sm.k[buf][r][8 * c], kp + off, take);
+      cp_async16(&sm.v[buf][r][8 * c], vp + off, take);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto mask_of = [&](int tile) -> uint8_t {  // of entry 64 tile + tid, for threads below 64
+    const int j = 64 * tile + tid;
+    return tid < 64 && j <= last ? __ldg(a.mask + j) : 0;
+  };
+  if (tile0 < tile1) copy_tile(tile0);
+  uint8_t seen = tile0 < tile1 ? mask_of(tile0) : 0;
+  for (int e = tid; e < 16 * D; e += 128) {
+    const int r = 4 * e / D, c = 4 * e % D, t = t0 + r / G;
+    const float4 v = t < S ? *reinterpret_cast<const float4*>(a.q + (size_t)t * a.Hq * D + (hk * G + r % G) * D + c)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t h0, l0, h1, l1;
+    split_h2(v.x, v.y, h0, l0);
+    split_h2(v.z, v.w, h1, l1);
+    *reinterpret_cast<uint2*>(&sm.k[1][r][c]) = make_uint2(h0, h1);
+    *reinterpret_cast<uint2*>(&sm.v[1][r][c]) = make_uint2(l0, l1);
   }
   __syncthreads();
   const int ra = 16 * warp + gid, rb = ra + 8;  // this thread's two query rows
@@ -249,14 +297,14 @@ __global__ void __launch_bounds__(128) prefill_flash_kernel(const float* q, int 
 #pragma unroll
   for (int ks = 0; ks < KS; ++ks) {
     const int c = 16 * ks + 2 * tig;
-    qh[ks][0] = *reinterpret_cast<const uint32_t*>(&Ks[ra][c]);
-    qh[ks][1] = *reinterpret_cast<const uint32_t*>(&Ks[rb][c]);
-    qh[ks][2] = *reinterpret_cast<const uint32_t*>(&Ks[ra][c + 8]);
-    qh[ks][3] = *reinterpret_cast<const uint32_t*>(&Ks[rb][c + 8]);
-    ql[ks][0] = *reinterpret_cast<const uint32_t*>(&Vs[ra][c]);
-    ql[ks][1] = *reinterpret_cast<const uint32_t*>(&Vs[rb][c]);
-    ql[ks][2] = *reinterpret_cast<const uint32_t*>(&Vs[ra][c + 8]);
-    ql[ks][3] = *reinterpret_cast<const uint32_t*>(&Vs[rb][c + 8]);
+    qh[ks][0] = *reinterpret_cast<const uint32_t*>(&sm.k[1][ra][c]);
+    qh[ks][1] = *reinterpret_cast<const uint32_t*>(&sm.k[1][rb][c]);
+    qh[ks][2] = *reinterpret_cast<const uint32_t*>(&sm.k[1][ra][c + 8]);
+    qh[ks][3] = *reinterpret_cast<const uint32_t*>(&sm.k[1][rb][c + 8]);
+    ql[ks][0] = *reinterpret_cast<const uint32_t*>(&sm.v[1][ra][c]);
+    ql[ks][1] = *reinterpret_cast<const uint32_t*>(&sm.v[1][rb][c]);
+    ql[ks][2] = *reinterpret_cast<const uint32_t*>(&sm.v[1][ra][c + 8]);
+    ql[ks][3] = *reinterpret_cast<const uint32_t*>(&sm.v[1][rb][c + 8]);
   }
   const int tok_a = t0 + ra / G, tok_b = t0 + rb / G;
   const int lim_a = P + tok_a, lim_b = P + tok_b;  // causal limits
@@ -264,35 +312,33 @@ __global__ void __launch_bounds__(128) prefill_flash_kernel(const float* q, int 
 #pragma unroll
   for (int nd = 0; nd < ND; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
   float m_a = -INFINITY, m_b = -INFINITY, l_a = 0.f, l_b = 0.f;
-  const int last = P + min(t0 + TB, S) - 1;  // the block's last token's limit
-  for (int j0 = 0; j0 <= last; j0 += 64) {
-    const int nj = min(64, last + 1 - j0);
-    __syncthreads();  // the previous tile (or the Q staging) is read
-    for (int e = tid; e < 64 * (D / 8); e += 128) {
-      const int r = e / (D / 8), c = e % (D / 8);
-      uint4 kv4 = make_uint4(0, 0, 0, 0), vv4 = kv4;
-      if (r < nj) {
-        const int sl = __ldg(bt_row + j0 + r);
-        const size_t off = (((size_t)(sl / cap) * Hkv + hk) * cap + sl % cap) * D;
-        kv4 = *reinterpret_cast<const uint4*>(kpool + off + 8 * c);
-        vv4 = *reinterpret_cast<const uint4*>(vpool + off + 8 * c);
-      }
-      *reinterpret_cast<uint4*>(&Ks[r][8 * c]) = kv4;
-      *reinterpret_cast<uint4*>(&Vs[r][8 * c]) = vv4;
+  for (int tile = tile0; tile < tile1; ++tile) {
+    const int buf = (tile - tile0) & 1, j0 = 64 * tile;
+    if (tid < 64) sm.vis[buf][tid] = seen;
+    __syncthreads();  // the other buffer (the previous tile, or the Q staging) is read
+    if (tile + 1 < tile1) {
+      copy_tile(tile + 1);
+      seen = mask_of(tile + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    if (tid < 64) vis[tid] = tid < nj && mask[j0 + tid] ? 1 : 0;
     __syncthreads();
+    const uint16_t (*Ks)[FlashSmem<D>::kLd] = sm.k[buf], (*Vs)[FlashSmem<D>::kLd] = sm.v[buf];
+    const uint8_t* vis = sm.vis[buf];
     float sc[8][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks)
+    for (int ks = 0; ks < KS; ks += 2)
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&Ks[8 * nt + gid][16 * ks + 2 * tig]);
-        const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&Ks[8 * nt + gid][16 * ks + 8 + 2 * tig]);
+        uint32_t b0, b1, b2, b3;  // entries 8 nt .. + 7, inputs 16 ks .. + 31
+        ldsm_x4(&Ks[8 * nt + (lane & 7)][16 * ks + 8 * (lane >> 3)], b0, b1, b2, b3);
         mma16816(sc[nt], qh[ks], b0, b1);
         mma16816(sc[nt], ql[ks], b0, b1);
+        mma16816(sc[nt], qh[ks + 1], b2, b3);
+        mma16816(sc[nt], ql[ks + 1], b2, b3);
       }
     // mask and scale; row maxima over the quad that shares a row
     float mx_a = -INFINITY, mx_b = -INFINITY;
@@ -360,26 +406,114 @@ __global__ void __launch_bounds__(128) prefill_flash_kernel(const float* q, int 
       }
     }
   }
-  const float ia = l_a > 0.f ? 1.f / l_a : 0.f, ib = l_b > 0.f ? 1.f / l_b : 0.f;
+  // output rows in the o projection's order (heads are whole 32-blocks)
+  auto out_row = [&](int r) { return a.attn + (size_t)(t0 + r / G) * a.attn_ld + (hk * G + r % G) * D; };
+  if (gridDim.z == 1) {
+    const float ia = l_a > 0.f ? 1.f / l_a : 0.f, ib = l_b > 0.f ? 1.f / l_b : 0.f;
+#pragma unroll
+    for (int nd = 0; nd < ND; ++nd) {
+      const int dcol = 8 * nd + 2 * tig, col = (dcol & ~31) + act_pos(dcol & 31);
+      if (tok_a < S)
+        *reinterpret_cast<uint32_t*>(out_row(ra) + col) = (uint32_t)f2h(o[nd][0] * ia) | ((uint32_t)f2h(o[nd][1] * ia) << 16);
+      if (tok_b < S)
+        *reinterpret_cast<uint32_t*>(out_row(rb) + col) = (uint32_t)f2h(o[nd][2] * ib) | ((uint32_t)f2h(o[nd][3] * ib) << 16);
+    }
+    return;
+  }
+  // this part's rows: (max, sum, 2 unused, output[D])
+  constexpr int kRow = D + 4;
+  const int blk = blockIdx.x * a.Hkv + hk;
+  float* part = a.part + (size_t)blk * gridDim.z * 64 * kRow;
+  float* mine = part + (size_t)blockIdx.z * 64 * kRow;
 #pragma unroll
   for (int nd = 0; nd < ND; ++nd) {
-    const int dcol = 8 * nd + 2 * tig;
-    const int col = (dcol & ~31) + act_pos(dcol & 31);  // the o projection's order (heads are whole 32-blocks)
-    if (tok_a < S)
-      *reinterpret_cast<uint32_t*>(out + (size_t)tok_a * out_ld + (hk * G + ra % G) * D + col) =
-          (uint32_t)f2h(o[nd][0] * ia) | ((uint32_t)f2h(o[nd][1] * ia) << 16);
-    if (tok_b < S)
-      *reinterpret_cast<uint32_t*>(out + (size_t)tok_b * out_ld + (hk * G + rb % G) * D + col) =
-          (uint32_t)f2h(o[nd][2] * ib) | ((uint32_t)f2h(o[nd][3] * ib) << 16);
+    *reinterpret_cast<float2*>(mine + ra * kRow + 4 + 8 * nd + 2 * tig) = make_float2(o[nd][0], o[nd][1]);
+    *reinterpret_cast<float2*>(mine + rb * kRow + 4 + 8 * nd + 2 * tig) = make_float2(o[nd][2], o[nd][3]);
+  }
+  if (tig == 0) {
+    *reinterpret_cast<float2*>(mine + ra * kRow) = make_float2(m_a, l_a);
+    *reinterpret_cast<float2*>(mine + rb * kRow) = make_float2(m_b, l_b);
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    s_last = atomicAdd(a.part_cnt + blk, 1) == (int)gridDim.z - 1;
+    if (s_last) a.part_cnt[blk] = 0;  // ready for the next launch
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // each row's weight of every part, then the rows' values with several parts'
+  // loads in flight
+  const int parts = gridDim.z;
+  float* wgt = reinterpret_cast<float*>(flash_smem);  // [parts][64]
+  if (tid < 64) {
+    float M = -INFINITY, den = 0.f;
+    for (int z = 0; z < parts; ++z) M = fmaxf(M, __ldcg(part + ((size_t)z * 64 + tid) * kRow));
+    for (int z = 0; z < parts; ++z) {
+      const float2 ml = __ldcg(reinterpret_cast<const float2*>(part + ((size_t)z * 64 + tid) * kRow));
+      const float w = ml.x == -INFINITY ? 0.f : expf(ml.x - M);
+      wgt[z * 64 + tid] = w;
+      den = fmaf(ml.y, w, den);
+    }
+    wgt[parts * 64 + tid] = den > 0.f ? 1.f / den : 0.f;
+  }
+  __syncthreads();
+  constexpr int kAt = 4, kRows = 128 / (D / 4);  // rows per thread and batch; rows per pass of the CTA
+  const int c = 4 * (tid % (D / 4));
+  for (int r0 = tid / (D / 4); r0 < 64; r0 += kAt * kRows) {
+    float4 num[kAt];
+#pragma unroll
+    for (int i = 0; i < kAt; ++i) num[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int z = 0; z < parts; ++z)
+#pragma unroll
+      for (int i = 0; i < kAt; ++i) {
+        const int r = r0 + i * kRows;
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(part + ((size_t)z * 64 + r) * kRow + 4 + c));
+        const float w = wgt[z * 64 + r];
+        num[i].x = fmaf(v.x, w, num[i].x);
+        num[i].y = fmaf(v.y, w, num[i].y);
+        num[i].z = fmaf(v.z, w, num[i].z);
+        num[i].w = fmaf(v.w, w, num[i].w);
+      }
+#pragma unroll
+    for (int i = 0; i < kAt; ++i) {
+      const int r = r0 + i * kRows;
+      if (t0 + r / G >= S) continue;
+      const float k = wgt[parts * 64 + r];
+      *reinterpret_cast<uint2*>(out_row(r) + (c & ~31) + act_pos(c & 31)) =
+          make_uint2((uint32_t)f2h(num[i].x * k) | ((uint32_t)f2h(num[i].y * k) << 16),
+                     (uint32_t)f2h(num[i].z * k) | ((uint32_t)f2h(num[i].w * k) << 16));
+    }
   }
 }
 
 template <int D, int G>
 cudaError_t launch_attn_t(const PrefillLayerArgs& a, cudaStream_t s) {
   static_assert(64 % G == 0, "64 query rows per CTA");
-  prefill_flash_kernel<D, G><<<dim3((a.S + 64 / G - 1) / (64 / G), a.Hkv), 128, 0, s>>>(
-      a.q, a.Hq, a.Hkv, a.kpool, a.vpool, a.bt_row, a.cap, a.mask, a.P, a.S, a.attn, a.attn_ld);
+  constexpr int kSmem = (int)sizeof(FlashSmem<D>);
+  const int blocks = (a.S + 64 / G - 1) / (64 / G), tiles = (a.P + a.S + 63) / 64;
+  // parts of the cache: as many CTAs as partial slots, at least two tiles each
+  // (and no more than one CTA should combine)
+  const int parts = std::max(1, std::min(std::min(a.part_slots / (blocks * a.Hkv), tiles / 2), 32));
+  prefill_flash_kernel<D, G><<<dim3(blocks, a.Hkv, parts), 128, kSmem, s>>>(a);
   return cudaGetLastError();
+}
+
+
+template <int D, int G>
+cudaError_t setup_attn_t() {
+  return cudaFuncSetAttribute(prefill_flash_kernel<D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(FlashSmem<D>));
+}
+template <int D>
+cudaError_t setup_attn_d() {
+  cudaError_t e = setup_attn_t<D, 1>();
+  if (e == cudaSuccess) e = setup_attn_t<D, 2>();
+  if (e == cudaSuccess) e = setup_attn_t<D, 4>();
+  if (e == cudaSuccess) e = setup_attn_t<D, 8>();
+  return e == cudaSuccess ? setup_attn_t<D, 16>() : e;
 }
 
 }  // namespace
@@ -411,6 +545,9 @@ cudaError_t launch_act_order(const uint16_t* x, int x_ld, int S, int Kp, uint16_
                                                                                                 out_ld);
   return cudaGetLastError();
 }
+
+cudaError_t prefill_setup(int head_dim) { return head_dim == 128 ? setup_attn_d<128>() : setup_attn_d<64>(); }
+size_t prefill_part_floats(int slots, int d) { return (size_t)slots * 64 * (d + 4); }
 
 cudaError_t launch_prefill_attention(const PrefillLayerArgs& a, cudaStream_t s) {
   const int G = a.Hq / a.Hkv;

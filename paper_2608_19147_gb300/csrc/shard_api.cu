@@ -99,6 +99,8 @@ struct shard_s {
   uint16_t* pf_h = nullptr;        // [C][Kp_F] SwiGLU output (padding zero)
   float* pf_y = nullptr;           // [parts][C][projection rows] projection outputs
   float* pf_q = nullptr;           // [C][dq] rotated queries
+  float* pf_part = nullptr;        // attention partials
+  int* pf_cnt = nullptr;           // attention parts finished, zero between launches
   uint16_t* dbg_act = nullptr;     // shard_debug_gemm: its input in act_pos order
   size_t dbg_act_n = 0;
   int debug_skip_arrival = -1;     // test knob (shard_debug_set_wait)
@@ -236,6 +238,8 @@ void release_shard(shard_s* sh) {
   cudaFree(sh->pf_h);
   cudaFree(sh->pf_y);
   cudaFree(sh->pf_q);
+  cudaFree(sh->pf_part);
+  cudaFree(sh->pf_cnt);
   cudaFree(sh->dbg_act);
   cudaFree(sh->X);
   cudaFree(sh->acc_qkv);
@@ -306,6 +310,7 @@ int shard_create(const shard_config* cfg, const shard_weights_host* w, shard_t* 
   if (c.head_dim != 64 && c.head_dim != 128) return fail(SHARD_EUNSUPPORTED, "head_dim must be 64 or 128");
   CUDA_TRY(gemv_setup());
   CUDA_TRY(gemm_tc_setup());
+  CUDA_TRY(prefill_setup(c.head_dim));
   CUDA_TRY(step_setup(c.group, c.head_dim));
   sh->cfg = c;
   sh->H = c.hidden;
@@ -878,7 +883,9 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
   if (!sh->pf_x) {
     // all or none: a call that fails here leaves no partial set behind for
     // the next call to mistake for a complete one
-    float *x = nullptr, *y = nullptr, *q = nullptr;
+    float *x = nullptr, *y = nullptr, *q = nullptr, *part = nullptr;
+    int* cnt = nullptr;
+    const int slots = 2 * sh->num_sms;
     uint16_t *act = nullptr, *attn = nullptr, *hh = nullptr;
     cudaError_t e = cudaMalloc(&x, sizeof(float) * C * sh->H);
     if (e == cudaSuccess) e = cudaMalloc(&act, sizeof(uint16_t) * C * sh->Kp_H);
@@ -886,6 +893,9 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
     if (e == cudaSuccess) e = cudaMalloc(&hh, sizeof(uint16_t) * C * sh->Kp_F);
     if (e == cudaSuccess) e = cudaMalloc(&y, sizeof(float) * y_floats);
     if (e == cudaSuccess) e = cudaMalloc(&q, sizeof(float) * C * sh->dq);
+    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(float) * prefill_part_floats(slots, sh->d));
+    if (e == cudaSuccess) e = cudaMalloc(&cnt, sizeof(int) * slots);
+    if (e == cudaSuccess) e = cudaMemset(cnt, 0, sizeof(int) * slots);
     if (e == cudaSuccess) e = cudaMemset(act, 0, sizeof(uint16_t) * C * sh->Kp_H);
     if (e == cudaSuccess) e = cudaMemset(attn, 0, sizeof(uint16_t) * C * sh->Kp_dq);
     if (e == cudaSuccess) e = cudaMemset(hh, 0, sizeof(uint16_t) * C * sh->Kp_F);
@@ -896,6 +906,8 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
       cudaFree(hh);
       cudaFree(y);
       cudaFree(q);
+      cudaFree(part);
+      cudaFree(cnt);
       return fail(e == cudaErrorMemoryAllocation ? SHARD_ENOMEM : SHARD_ECUDA, "shard_prefill: work buffers: %s",
                   cudaGetErrorString(e));
     }
@@ -905,10 +917,11 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
     sh->pf_h = hh;
     sh->pf_y = y;
     sh->pf_q = q;
+    sh->pf_part = part;
+    sh->pf_cnt = cnt;
   }
   CUDA_TRY(launch_prefill_check(token_ids, sh->cfg.vocab, position_ids, sh->cfg.max_position, attention_mask, P, S,
                                 sh->status, s));
-  const int* bt_row = st->bt[st->bt_cur] + (size_t)row * st->cap;
   const float eps = static_cast<float>(sh->cfg.rms_eps);
   for (int t0 = 0; t0 < S; t0 += C) {
     const int c = std::min(C, S - t0);
@@ -975,7 +988,9 @@ int shard_prefill(shard_t sh, kvstate_t st, int row, const uint16_t* hidden_in, 
       pa.row = row;
       pa.cap = st->cap;
       pa.slot0 = P + t0;
-      pa.bt_row = bt_row;
+      pa.part = sh->pf_part;
+      pa.part_cnt = sh->pf_cnt;
+      pa.part_slots = 2 * sh->num_sms;
       pa.mask = attention_mask;
       pa.P = P + t0;
       pa.attn = sh->pf_attn;

@@ -62,3 +62,10 @@ def test_prefill_shapes(name, S, P):
 @pytest.mark.parametrize("offset", [1, 2, 4])
 def test_prefill_value_aligned_buffers(offset):
     _run("g128", 40, 10, offset)
+
+
+@pytest.mark.parametrize("name,S,P", [("g128", 3, 2000), ("g64", 17, 3000), ("g32", 70, 1500)])
+def test_prefill_attention_parts(name, S, P):
+    """Few token blocks over a long cache: the cache is cut into parts, some without a visible entry."""
+    _run(name, S, P)
+    _run(name, S, P)
