@@ -1,21 +1,24 @@
 // Standalone launch of one W4A16 projection (the test export
 // shard_debug_gemv, the allocation-free entry point and the LM head use it).
 // The device code is the warp-level projection of gemv_core.cuh, the same
-// code the whole-step kernel runs: kGemvWarps consumer warps and one producer
-// warp per CTA, one CTA per SM.
+// code the whole-step kernel runs: kGemvWarps consumer warps per CTA, one CTA
+// per SM.
+#include <algorithm>
+
 #include "gemv_core.cuh"
 
 namespace shard {
 namespace {
 
+constexpr int kCtasPerSm = 1;
+
 constexpr int kW = kGemvWarps;  // consumer warps per CTA
 constexpr int kBlock = (kW + (kSelfRefill ? 0 : 1)) * 32;
-constexpr int kCtasPerSm = 1;
 
 template <int GPU>
 constexpr size_t smem_bytes() {
-  return (size_t)kW * Geom<GPU>::kGemvSlots * Geom<GPU>::kUnitBytes +
-         (size_t)2 * kW * Geom<GPU>::kGemvSlots * sizeof(uint64_t);
+  constexpr int kSlots = Geom<GPU>::kGemvSlots;
+  return (size_t)kW * kSlots * Geom<GPU>::kUnitBytes + (size_t)2 * kW * kSlots * sizeof(uint64_t);
 }
 
 // 227 KB per CTA, less a margin for the kernel's static shared memory
@@ -28,7 +31,6 @@ __global__ void __launch_bounds__(kBlock, 1) gemv_kernel(const __grid_constant__
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ OpDesc s_op[1];
   __shared__ GemvPhase s_gp;
-  __shared__ WarpRing<GPU, kSlots> s_ring[kW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* rings = smem;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)kW * kSlots * Geom<GPU>::kUnitBytes);
@@ -51,27 +53,28 @@ __global__ void __launch_bounds__(kBlock, 1) gemv_kernel(const __grid_constant__
     return;
   }
   const int g = blockIdx.x * kW + warp, nw = gridDim.x * kW;
-  {
-    WarpRing<GPU, kSlots> r;
-    r.ring = rings + (size_t)warp * kSlots * Geom<GPU>::kUnitBytes;
-    r.full = full + warp * kSlots;
-    r.empty = empty + warp * kSlots;
-    r.n_used = 0;
-    r.timed_out = false;
-    if (kSelfRefill) r.start(s_op, 1, g, nw, lane);  // the weights do not depend on the preceding kernel
-    if (lane == 0) s_ring[warp] = r;
-    __syncwarp();
-  }
-  pdl_launch_dependents();
+  WarpRing<GPU, kSlots> ring;
+  ring.ring = rings + (size_t)warp * kSlots * Geom<GPU>::kUnitBytes;
+  ring.full = full + warp * kSlots;
+  ring.empty = empty + warp * kSlots;
+  ring.n_used = 0;
+  ring.timed_out = false;
+  if (kSelfRefill) ring.start(s_op, 1, g, nw, lane);  // the weights do not depend on the preceding kernel
   pdl_wait();
-  gemv_phase<NT, GPU, kSlots>(&s_ring[warp], &s_op[0], &s_gp, g, nw, lane);
-  if (s_ring[warp].timed_out && lane == 0) atomicOr(a.status, ST_WAIT_TIMEOUT);
+  gemv_run<NT, GPU, kSlots, true>(ring, &s_op[0], &s_gp, g, nw, lane);
+  // a dependent kernel may take the SMs that run out of work (not earlier: its
+  // CTAs would wait beside the ones that still stream)
+  pdl_launch_dependents();
+  if (ring.timed_out && lane == 0) atomicOr(a.status, ST_WAIT_TIMEOUT);
 }
 
 template <int NT, int GPU>
 cudaError_t launch_t(const GemvArgs& a, int grid, cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  // the split's 32-bit arithmetic: (units + 1) x warps below 2^32 (the callers
+  // check it for kCtaWarps warps per CTA)
+  const long long units = (long long)a.n_rb * a.upr + 1;
+  cfg.gridDim = dim3((unsigned)std::min<long long>(grid, ((1ll << 32) - 1) / (units * kW)));
   cfg.blockDim = dim3(kBlock);
   cfg.dynamicSmemBytes = smem_bytes<GPU>();
   cfg.stream = s;
@@ -106,8 +109,9 @@ int gemv_grid(int nt, int num_sms) {
   return kCtasPerSm * num_sms;
 }
 
-// the larger of the two kernels' consumer warp counts: index checks cover both
-int gemv_warps_per_cta() { return kW > kCtaWarps ? kW : kCtaWarps; }
+// warps per CTA that the callers' index checks count with (launch_t takes
+// fewer CTAs where this kernel's own count would overflow)
+int gemv_warps_per_cta() { return kCtaWarps; }
 
 cudaError_t launch_gemv(const GemvArgs& a, int nt, int group, int grid, cudaStream_t s, bool pdl) {
   if (nt == 1) {

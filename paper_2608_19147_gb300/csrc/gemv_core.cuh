@@ -45,7 +45,10 @@ namespace shard {
 constexpr bool kSelfRefill = true;
 constexpr int kRingSlots = 2;  // step kernel: units in flight per consumer warp (a deeper ring takes the L1 that the norm and attention loads use)
 constexpr int kCtaWarps = kSelfRefill ? 12 : 11;   // consumer warps per CTA of the step kernel
-constexpr int kGemvWarps = kSelfRefill ? 12 : 11;  // consumer warps per CTA of the standalone projection kernel
+// Consumer warps per CTA of the standalone projection kernel, whose loop fits 128
+// registers (a warp's unit is a chain of latencies: 128256 x 4096 lm_head, 1
+// token 58.5 -> 53.4 us, 5 tokens 67 -> 60, 8 tokens 72 -> 63 against 12 warps).
+constexpr int kGemvWarps = kSelfRefill ? 16 : 11;
 
 template <int GPU>
 struct Geom {
@@ -54,8 +57,9 @@ struct Geom {
   // the step kernel's slots (group 32 units are larger: two)
   static constexpr int kStepSlots = GPU == 4 ? 2 : kRingSlots;
   // the standalone projection (no attention area competes for shared
-  // memory): four slots per warp where the rings fit in 216 KB, else two
-  static constexpr int kGemvSlots = kGemvWarps * 4 * kUnitBytes <= 216 * 1024 ? 4 : 2;
+  // memory): up to four slots per warp, as many as fit in 216 KB
+  static constexpr int kGemvSlots =
+      kGemvWarps * 4 * kUnitBytes <= 216 * 1024 ? 4 : kGemvWarps * 3 * kUnitBytes <= 216 * 1024 ? 3 : 2;
 };
 
 __device__ __forceinline__ uint32_t hsub2_u32(uint32_t a, uint32_t b) {
@@ -675,8 +679,10 @@ __device__ __forceinline__ void segment_end(const GemvPhase* pp, const float (&t
 // (which is filled in the same order) and hand on each row-block segment of
 // it.  Inlined at one call site (the whole-step kernel's layer loop, which
 // keeps the ring in registers), so no call boundary spills the caller's
-// registers.
-template <int NT, int GPU, int S>
+// registers.  kSeq: two token tiles one after the other per unit, which
+// dequantises twice but holds one tile's activations and group sums at a time
+// (for kernels with 128 registers; the same sums).
+template <int NT, int GPU, int S, bool kSeq = false>
 __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* op, const GemvPhase* pp, int g, int nw,
                                          int lane) {
   const GemvPhase& p = *pp;
@@ -701,8 +707,9 @@ __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* o
   const int act_ld = acts ? p.act_s_ld : p.act_ld, M = p.M;
   int rb = wb / upr;
   int ku = wb - rb * upr;
-  uint4 nxt[NT][2][2];
-  load_act<NT>(nxt, actp, acts, act_ld, M, ku, lane);
+  constexpr int kAt = kSeq ? 1 : NT;  // token tiles at a time
+  uint4 nxt[kAt][2][2];
+  load_act<kAt>(nxt, actp, acts, act_ld, M, ku, lane);
   for (int u = wb; u < we; ++rb) {
     const int seg_begin = u, rb_end = (rb + 1) * upr;
     const int seg_end = we < rb_end ? we : rb_end;
@@ -715,17 +722,37 @@ __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* o
         for (int q = 0; q < 4; ++q) tot[rt][nt][q] = 0.f;
 #pragma unroll 2  // alternating activation registers instead of copies
     for (; u < seg_end; ++u) {
-      uint4 cur[NT][2][2];
+      const uint8_t* U = nullptr;
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
+      for (int t0 = 0; t0 < NT; t0 += kAt) {
+        uint4 cur[kAt][2][2];
 #pragma unroll
-        for (int kc = 0; kc < 2; ++kc)
+        for (int nt = 0; nt < kAt; ++nt)
 #pragma unroll
-          for (int h = 0; h < 2; ++h) cur[nt][kc][h] = nxt[nt][kc][h];
-      if (++ku == upr) ku = 0;
-      if (u + 1 < we) load_act<NT>(nxt, actp, acts, act_ld, M, ku, lane);
-      const uint8_t* U = ring.acquire();
-      if (!ring.timed_out) mma_unit<NT, GPU>(U, cur, tot, lane);
+          for (int kc = 0; kc < 2; ++kc)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) cur[nt][kc][h] = nxt[nt][kc][h];
+        const int t1 = (t0 + kAt) % NT;  // the next tiles, of this unit or the next
+        if (t1 == 0 && ++ku == upr) ku = 0;
+        if (t1 > 0 || u + 1 < we) load_act<kAt>(nxt, actp + (size_t)8 * t1 * act_ld, acts ? acts + 16u * t1 * act_ld : 0u, act_ld, M - 8 * t1, ku, lane);
+        if (t0 == 0) U = ring.acquire();
+        if (!ring.timed_out) {
+          if constexpr (kAt == NT) {
+            mma_unit<NT, GPU>(U, cur, tot, lane);
+          } else {
+            float one[4][1][4];
+#pragma unroll
+            for (int rt = 0; rt < 4; ++rt)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) one[rt][0][e] = tot[rt][t0][e];
+            mma_unit<1, GPU>(U, cur, one, lane);
+#pragma unroll
+            for (int rt = 0; rt < 4; ++rt)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) tot[rt][t0][e] = one[rt][0][e];
+          }
+        }
+      }
       ring.release(lane);
     }
     if (op->q > 0)
@@ -733,17 +760,6 @@ __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* o
     else
       segment_end<NT>(pp, tot, rb, seg_end - seg_begin, upr, lane);
   }
-}
-
-// gemv_run with the ring state in shared memory (the standalone kernel).
-template <int NT, int GPU, int S>
-__device__ __noinline__ void gemv_phase(WarpRing<GPU, S>* ring_io, const OpDesc* op, const GemvPhase* pp, int g, int nw,
-                                        int lane) {
-  WarpRing<GPU, S> ring = *ring_io;
-  gemv_run<NT, GPU, S>(ring, op, pp, g, nw, lane);
-  __syncwarp();
-  if (lane == 0) *ring_io = ring;
-  __syncwarp();
 }
 
 }  // namespace shard

@@ -137,113 +137,111 @@ __global__ void __launch_bounds__(kNormThreads) head_norm_kernel(const uint16_t*
   for (int i = tid; i < H; i += blockDim.x) out[i] = f2h(h2f(h[i]) * r * h2f(w[i]));
 }
 
-struct Top1Part {
+struct __align__(16) Top1Part {
   float max, sum;  // the largest logit; sum of exp(logit - max)
   int idx, pad;    // the lowest id holding max
 };
 
-// Folds (bm, bs, bi) into (am, as, ai), a first: the larger maximum wins,
-// equal maxima keep the lower id, the sums are rescaled to the new maximum.
-// An empty side has max -inf and sum 0.
-__device__ __forceinline__ void top1_combine(float& am, float& as, int& ai, float bm, float bs, int bi) {
-  if (bm == -INFINITY) return;
-  if (am == -INFINITY) {
-    am = bm;
-    as = bs;
-    ai = bi;
-    return;
-  }
-  const float nm = fmaxf(am, bm);
-  as = as * expf(am - nm) + bs * expf(bm - nm);
-  ai = am > bm ? ai : (bm > am ? bi : min(ai, bi));
-  am = nm;
-}
-
-// Butterfly over the 32 lanes; both partners fold the lower lane's part
-// first, so every lane ends with the same bits.
-__device__ __forceinline__ void top1_warp(float& m, float& s, int& i) {
-  const int lane = threadIdx.x & 31;
+// Over the CTA: the largest m, then for it the sum of s exp(m - largest) and the
+// lowest i that holds it, the sums in a fixed order (every thread gets the
+// same bits). A part without a value has m -inf and s 0.
+__device__ __forceinline__ Top1Part top1_block(float m, float s, int i) {
+  constexpr int kWarps = kTopThreads / 32;
+  __shared__ float s_m[kWarps], s_s[kWarps];
+  __shared__ int s_i[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float big = m;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
-    const int i2 = __shfl_xor_sync(0xffffffffu, i, o);
-    if ((lane & o) == 0) {
-      top1_combine(m, s, i, m2, s2, i2);
-    } else {
-      float am = m2, as = s2;
-      int ai = i2;
-      top1_combine(am, as, ai, m, s, i);
-      m = am;
-      s = as;
-      i = ai;
-    }
+  for (int o = 16; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+  if (lane == 0) s_m[warp] = big;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) big = fmaxf(big, s_m[w]);
+  s = m == -INFINITY ? s : s * expf(m - big);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  const unsigned low = __reduce_min_sync(0xffffffffu, m == big ? (unsigned)i : 0x7fffffffu);
+  if (lane == 0) {
+    s_s[warp] = s;
+    s_i[warp] = (int)low;
   }
+  __syncthreads();
+  Top1Part p{big, 0.f, 0x7fffffff, 0};
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    p.sum += s_s[w];
+    p.idx = min(p.idx, s_i[w]);
+  }
+  __syncthreads();
+  return p;
 }
 
-// (chunk, row) CTAs: one pass over the chunk's logits with an online
-// (max, sum of exp) per thread, a fixed-order reduction over the CTA, and
-// the row's last CTA folds the chunks.
+// (chunk, row) CTAs: the chunk's largest logit, the sum of exp relative to it
+// and the lowest id that holds it, each in one reduction over the CTA; the
+// row's last CTA folds the chunks the same way. Bound by its chain of latencies (two
+// L2 round trips, the count, six reductions); it is launched as a dependent of
+// the projection so that its launch does not follow that kernel's end.
 __global__ void __launch_bounds__(kTopThreads) head_top1_kernel(const float* __restrict__ logits, int ld, int V,
                                                                 int chunk, Top1Part* __restrict__ parts,
                                                                 int* __restrict__ done, const int* status,
                                                                 int32_t* __restrict__ token,
                                                                 float* __restrict__ p_max) {
-  __shared__ float s_m[kTopThreads / 32], s_s[kTopThreads / 32];
-  __shared__ int s_i[kTopThreads / 32];
   __shared__ int s_last;
-  const int c = blockIdx.x, m = blockIdx.y, nc = gridDim.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.x, m = blockIdx.y, nc = gridDim.x, tid = threadIdx.x;
   const float* l = logits + (size_t)m * ld;
   const int b = c * chunk, e = min(V, b + chunk);
-  float mx = -INFINITY, sm = 0.f;
-  int ix = 0x7fffffff;
   constexpr int kPer = kTopChunkMax / kTopThreads;
   float x[kPer];
+  pdl_wait();  // the logits
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
-    const int v = b + threadIdx.x + j * kTopThreads;
+    const int v = b + tid + j * kTopThreads;
     x[j] = v < e ? __ldcg(l + v) : -INFINITY;
   }
+  float mx = x[0], sm = 0.f;
 #pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    const int v = b + threadIdx.x + j * kTopThreads;
-    if (v < e) top1_combine(mx, sm, ix, x[j], 1.f, v);  // ids rise along a thread's walk
-  }
-  top1_warp(mx, sm, ix);
-  if (lane == 0) {
-    s_m[warp] = mx;
-    s_s[warp] = sm;
-    s_i[warp] = ix;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    mx = lane < kTopThreads / 32 ? s_m[lane] : -INFINITY;
-    sm = lane < kTopThreads / 32 ? s_s[lane] : 0.f;
-    ix = lane < kTopThreads / 32 ? s_i[lane] : 0x7fffffff;
-    top1_warp(mx, sm, ix);
-    if (lane == 0) {
-      parts[(size_t)m * nc + c] = Top1Part{mx, sm, ix, 0};
-      __threadfence();
-      s_last = atomicAdd(done + m, 1) == nc - 1;
+  for (int j = 1; j < kPer; ++j) mx = fmaxf(mx, x[j]);
+  int ix = 0x7fffffff;
+#pragma unroll
+  for (int j = kPer - 1; j >= 0; --j) {
+    const int v = b + tid + j * kTopThreads;
+    if (v < e) {
+      sm += expf(x[j] - mx);
+      if (x[j] == mx) ix = v;  // ids rise along a thread's walk
     }
   }
+  Top1Part p = top1_block(mx, sm, ix);
+  if (tid == 0) {
+    if (p.idx == 0x7fffffff) p.idx = b;  // not a number anywhere: any valid id
+    parts[(size_t)m * nc + c] = p;
+    __threadfence();
+    s_last = atomicAdd(done + m, 1) == nc - 1;
+  }
   __syncthreads();
-  if (!s_last || warp != 0) return;
-  // the row's last CTA: lane L folds chunks L, L + 32, ... in order, then the
-  // butterfly -- a fixed order, whatever the arrival order of the CTAs
+  if (!s_last) return;
   __threadfence();
   float gm = -INFINITY, gs = 0.f;
   int gi = 0x7fffffff;
-  for (int k = lane; k < nc; k += 32)
-    top1_combine(gm, gs, gi, __ldcg(&parts[(size_t)m * nc + k].max), __ldcg(&parts[(size_t)m * nc + k].sum),
-                 __ldcg(&parts[(size_t)m * nc + k].idx));
-  top1_warp(gm, gs, gi);
-  if (lane == 0) {
+  for (int k = tid; k < nc; k += kTopThreads) {
+    const int4 raw = __ldcg(reinterpret_cast<const int4*>(&parts[(size_t)m * nc + k]));
+    const float pm = __int_as_float(raw.x), ps = __int_as_float(raw.y);
+    if (k == tid) {
+      gm = pm;
+      gs = ps;
+      gi = raw.z;
+    } else {  // (more chunks than threads) ids rise along a thread's walk
+      const float nm = fmaxf(gm, pm);
+      gs = (gm == -INFINITY ? gs : gs * expf(gm - nm)) + (pm == -INFINITY ? ps : ps * expf(pm - nm));
+      if (pm > gm) gi = raw.z;
+      gm = nm;
+    }
+  }
+  const Top1Part r = top1_block(gm, gs, gi);
+  if (tid == 0) {
     // a projection wait that gave up (never expected) marks the row failed
     const bool ok = __ldcg(status) == 0;
-    token[m] = ok ? gi : -1;
-    if (p_max) p_max[m] = ok ? 1.f / gs : __int_as_float(0x7fc00000);
+    token[m] = ok ? (r.idx == 0x7fffffff ? 0 : r.idx) : -1;
+    if (p_max) p_max[m] = ok ? 1.f / r.sum : __int_as_float(0x7fc00000);
     done[m] = 0;  // ready for the next call
   }
 }
@@ -331,13 +329,19 @@ int run(head_s* h, const uint16_t* hidden, int M, int32_t* token, float* p_max, 
   HEAD_CUDA_TRY(launch_gemv(g, nt, c.group, std::min<long long>(h->grid[nt], (long long)h->op.n_rb * h->op.upr), s,
                             true));
   if (token) {
-    // a plain launch: with programmatic dependent launch this kernel measured
-    // ~8 us slower per call
     int nc = 0;
     const int chunk = chunk_of(h, M, &nc);
-    head_top1_kernel<<<dim3(nc, M), kTopThreads, 0, s>>>(logits, ld, c.vocab, chunk, h->parts, h->done, h->status,
-                                                        token, p_max);
-    HEAD_CUDA_TRY(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nc, M);
+    cfg.blockDim = dim3(kTopThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    HEAD_CUDA_TRY(cudaLaunchKernelEx(&cfg, head_top1_kernel, (const float*)logits, ld, (int)c.vocab, chunk, h->parts, h->done,
+                                     (const int*)h->status, token, p_max));
   }
   return SHARD_OK;
 }
