@@ -158,7 +158,7 @@ __device__ __forceinline__ bool wait_count(const int* p, int target, int* status
       return false;
     }
     if ((it & 1023) == 0 && (*reinterpret_cast<volatile int*>(status) & ST_WAIT_TIMEOUT)) return false;
-    __nanosleep(64);
+    __nanosleep(20);
   }
   return true;
 }
@@ -265,8 +265,8 @@ __device__ __noinline__ void prologue_work(const PrologueArgs& a, const StepPara
 // is normalised by CTA m alone, and the others wait for the count of finished
 // rows and read the fp16 result: every CTA reading all M rows of 64-bit sums
 // (H * 8 bytes each, 39 MB over the chip for 8 rows of 4096) costs more than
-// that hand-over (8B width, norm + gate|up: 5 rows 26.6 -> 21.5 us, 8 rows
-// 40 -> 26, 16 rows 80 -> 39).
+// that hand-over (8B width, norm + gate|up: 5 rows 26.6 -> 18.4 us, 8 rows
+// 40 -> 19, 16 rows 80 -> 30, together with the gate|up reduction).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float4 norm_load(bool from_x, const long long* X, const uint16_t* const* rowp, int H, int m,
                                             int k) {
@@ -1071,22 +1071,29 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
       }
       if (!norm_staged) {
         norms_done += M;
-        if (threadIdx.x == 0) {
-          wait_count(a.norm_cnt, norms_done, a.status, a.wait_limit);
-          if (xn_smem) {
-            // the rows were written through the generic proxy; the area was
-            // last used by generic accesses of this CTA
-            asm volatile("fence.proxy.async;" ::: "memory");
-            mbar_arrive_expect_tx(&s_nbar, (uint32_t)M * a.H * 2u);
-            for (int m = 0; m < M; ++m)
-              bulk_g2s(xn + (size_t)m * xn_ld, a.act_h + (size_t)m * a.Kp_H, (uint32_t)a.H * 2u, &s_nbar);
-          }
-        }
-        if (xn_smem) {
-          if (!mbar_wait(&s_nbar, nphase) && threadIdx.x == 0) atomicOr(a.status, ST_WAIT_TIMEOUT);
-          nphase ^= 1u;
-        }
+        if (threadIdx.x == 0) wait_count(a.norm_cnt, norms_done, a.status, a.wait_limit);
         cbar();
+        if (xn_smem) {
+          // plain loads, all in flight: bulk copies cost a proxy fence and a
+          // barrier wait more (8B width, 5 tokens, norm + gate|up 21.0 -> 18.4 us)
+          constexpr int kAhead = 8;
+          const int per = a.H / 8, pieces = M * per;  // of 16 bytes
+          for (int e0 = threadIdx.x; e0 < pieces; e0 += kAhead * kThreads) {
+            uint4 v[kAhead];
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) {
+              const int e = e0 + i * kThreads, m = e / per;
+              v[i] = e < pieces ? __ldcg(reinterpret_cast<const uint4*>(a.act_h + (size_t)m * a.Kp_H) + (e - m * per))
+                                : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) {
+              const int e = e0 + i * kThreads, m = e / per;
+              if (e < pieces) *(reinterpret_cast<uint4*>(xn + (size_t)m * xn_ld) + (e - m * per)) = v[i];
+            }
+          }
+          cbar();
+        }
       }
     } else if (k == 1) {
       // the q|k|v sums and counts are consumed: clear them for the next layer
