@@ -114,13 +114,15 @@ __global__ void kv_gather_kernel(const uint16_t* pool, int n_layers, size_t laye
 
 __global__ void kv_scatter_kernel(uint16_t* pool, int n_layers, size_t layer_stride, int Hkv, int cap, int d, int row,
                                   const uint16_t* in, int n) {
-  const size_t total = (size_t)n_layers * n * Hkv * d;
+  const int d8 = d / 8;  // 16-byte pieces (d is a multiple of 16, `in` 16-byte aligned)
+  const size_t total = (size_t)n_layers * n * Hkv * d8;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int t = static_cast<int>(e % d);
-    const int h = static_cast<int>((e / d) % Hkv);
-    const int j = static_cast<int>((e / ((size_t)d * Hkv)) % n);
-    const int l = static_cast<int>(e / ((size_t)d * Hkv * n));
-    pool[l * layer_stride + (((size_t)row * Hkv + h) * cap + j) * d + t] = in[e];
+    const int t = static_cast<int>(e % d8);
+    const int h = static_cast<int>((e / d8) % Hkv);
+    const int j = static_cast<int>((e / ((size_t)d8 * Hkv)) % n);
+    const int l = static_cast<int>(e / ((size_t)d8 * Hkv * n));
+    *reinterpret_cast<uint4*>(pool + l * layer_stride + (((size_t)row * Hkv + h) * cap + j) * d + 8 * t) =
+        reinterpret_cast<const uint4*>(in)[e];
   }
 }
 
@@ -168,7 +170,7 @@ cudaError_t launch_kv_gather(const uint16_t* pool, int n_layers, size_t layer_st
 
 cudaError_t launch_kv_scatter(uint16_t* pool, int n_layers, size_t layer_stride, int Hkv, int cap, int d, int row,
                               const uint16_t* in, int n, cudaStream_t s) {
-  const size_t total = (size_t)n_layers * n * Hkv * d;
+  const size_t total = (size_t)n_layers * n * Hkv * d / 8;
   if (total == 0) return cudaSuccess;
   kv_scatter_kernel<<<grid_for(total, 256), 256, 0, s>>>(pool, n_layers, layer_stride, Hkv, cap, d, row, in, n);
   return cudaGetLastError();
