@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kBlock, 1) gemv_kernel(const __grid_constant__
   ring.timed_out = false;
   if (kSelfRefill) ring.start(s_op, 1, g, nw, lane);  // the weights do not depend on the preceding kernel
   pdl_wait();
-  gemv_run<NT, GPU, kSlots, true>(ring, &s_op[0], &s_gp, g, nw, lane);
+  gemv_run<NT, GPU, kSlots>(ring, &s_op[0], &s_gp, g, nw, lane);
   // a dependent kernel may take the SMs that run out of work (not earlier: its
   // CTAs would wait beside the ones that still stream)
   pdl_launch_dependents();

@@ -343,9 +343,8 @@ constexpr float kTotScaleHi = 4503599627370496.0f;   // 2^52 = 2^32 * 2^20
 // Group end of one 16-row tile: zero-point correction and scale.  zw: the
 // zero bytes of tiles 2 i and 2 i + 1 (z_lo, 16 z_hi of each), scw: the
 // tile's two scales.
-template <int NT>
-__device__ __forceinline__ void group_end(float (&tot)[NT][4], const float (&acc)[NT][4], const float (&sa)[NT][4],
-                                          uint32_t zw, uint32_t scw, int rt) {
+__device__ __forceinline__ void group_end(float (&tot)[4], const float (&acc)[4], const float (&sa)[4], uint32_t zw,
+                                          uint32_t scw, int rt) {
   const uint32_t p = 2u * (rt & 1);
   // fp16 bits 0x8000 | z and 0x8000 | 16 z: -z * 2^-24 and -16 z * 2^-24
   const uint32_t zp = prmt_u32(zw, 0x80u, p | (4u << 4) | ((p + 1u) << 8) | (4u << 12));
@@ -353,86 +352,21 @@ __device__ __forceinline__ void group_end(float (&tot)[NT][4], const float (&acc
   const float zhi = h2f(static_cast<uint16_t>(zp >> 16));
   const float slo = h2f(static_cast<uint16_t>(scw & 0xFFFFu));
   const float shi = h2f(static_cast<uint16_t>(scw >> 16));
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt) {
-    tot[nt][0] = fmaf(slo, fmaf(zlo, sa[nt][0], acc[nt][0]), tot[nt][0]);
-    tot[nt][1] = fmaf(slo, fmaf(zlo, sa[nt][1], acc[nt][1]), tot[nt][1]);
-    tot[nt][2] = fmaf(shi, fmaf(zhi, sa[nt][0], acc[nt][2]), tot[nt][2]);
-    tot[nt][3] = fmaf(shi, fmaf(zhi, sa[nt][1], acc[nt][3]), tot[nt][3]);
-  }
+  tot[0] = fmaf(slo, fmaf(zlo, sa[0], acc[0]), tot[0]);
+  tot[1] = fmaf(slo, fmaf(zlo, sa[1], acc[1]), tot[1]);
+  tot[2] = fmaf(shi, fmaf(zhi, sa[0], acc[2]), tot[2]);
+  tot[3] = fmaf(shi, fmaf(zhi, sa[1], acc[3]), tot[3]);
 }
 
-// Two token tiles (M > 8): two 16-row tiles at a time.  With all four, their
-// sums beside two units' activations do not fit the registers (1448 bytes of
-// spills in the step kernel, now 272; 16 packed tokens at 8B width, 4 layers:
-// 470 -> 427 us).
+// For one token tile of 8.
 template <int GPU>
-__device__ __forceinline__ void mma_unit2(const uint8_t* __restrict__ U, const uint4 (&act)[2][2][2],
-                                          float (&tot)[4][2][4], int lane) {
+__device__ __forceinline__ void mma_unit(const uint8_t* __restrict__ U, const uint4 (&act)[2][2], float (&tot)[4][4],
+                                         int lane) {
   constexpr int BPG = Geom<GPU>::kBlocksPerGroup;
   constexpr uint32_t kOnes = 0x3C003C00u;  // fp16x2 (1, 1)
   const int gid = lane >> 2;
-#pragma unroll
-  for (int gi = 0; gi < GPU; ++gi) {
-    const uint8_t* meta = U + kCodeBytes + gi * kMetaBytesPerGroup;
-    float sa[2][4];
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) sa[nt][0] = sa[nt][1] = sa[nt][2] = sa[nt][3] = 0.f;
-#pragma unroll
-    for (int r0 = 0; r0 < 4; r0 += 2) {
-      float acc[2][2][4];
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) acc[r][nt][0] = acc[r][nt][1] = acc[r][nt][2] = acc[r][nt][3] = 0.f;
-      uint4 A[2];
-#pragma unroll
-      for (int blk = gi * BPG; blk < (gi + 1) * BPG; ++blk) {
-        const int j = blk & 3;
-        if (blk == gi * BPG || j == 0)
-#pragma unroll
-          for (int r = 0; r < 2; ++r)
-            A[r] = *reinterpret_cast<const uint4*>(U + ((blk >> 2) * 4 + r0 + r) * 512 + lane * 16);
-        uint32_t b0[2], b1[2];
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const uint4 v = act[nt][blk >> 2][(blk >> 1) & 1];
-          b0[nt] = (blk & 1) ? v.z : v.x;
-          b1[nt] = (blk & 1) ? v.w : v.y;
-          if (r0 == 0) mma_16816(sa[nt], kOnes, kOnes, kOnes, kOnes, b0[nt], b1[nt]);
-        }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const uint32_t w = (j == 0) ? A[r].x : (j == 1) ? A[r].y : (j == 2) ? A[r].z : A[r].w;
-          const uint32_t w2 = w >> 8;
-          const uint32_t a0 = w & 0x000F000Fu, a1 = w & 0x00F000F0u;
-          const uint32_t a2 = w2 & 0x000F000Fu, a3 = w2 & 0x00F000F0u;
-#pragma unroll
-          for (int nt = 0; nt < 2; ++nt) mma_16816(acc[r][nt], a0, a1, a2, a3, b0[nt], b1[nt]);
-        }
-      }
-      const uint2 zz = *reinterpret_cast<const uint2*>(meta + 128 + gid * 8);
-      const uint4 sc = *reinterpret_cast<const uint4*>(meta + gid * 16);
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-        group_end<2>(tot[r0 + r], acc[r], sa, r0 == 0 ? zz.x : zz.y, r0 == 0 ? (r ? sc.y : sc.x) : (r ? sc.w : sc.z), r);
-    }
-  }
-}
-
-// NT token tiles of 8.
-template <int NT, int GPU>
-__device__ __forceinline__ void mma_unit(const uint8_t* __restrict__ U, const uint4 (&act)[NT][2][2],
-                                         float (&tot)[4][NT][4], int lane) {
-  if constexpr (NT == 2) {
-    mma_unit2<GPU>(U, act, tot, lane);
-    return;
-  }
-  constexpr int BPG = Geom<GPU>::kBlocksPerGroup;
-  constexpr uint32_t kOnes = 0x3C003C00u;  // fp16x2 (1, 1)
-  const int gid = lane >> 2;
-  float accg[4][NT][4];
-  float sa[NT][4];  // group sums of the activations: tokens 2 tig, 2 tig + 1 (twice)
+  float accg[4][4];
+  float sa[4];  // group sums of the activations: tokens 2 tig, 2 tig + 1 (twice)
 #pragma unroll
   for (int kc = 0; kc < 2; ++kc) {
     uint4 A[4];
@@ -445,31 +379,22 @@ __device__ __forceinline__ void mma_unit(const uint8_t* __restrict__ U, const ui
       const uint8_t* meta = U + kCodeBytes + gi * kMetaBytesPerGroup;
       if (blk % BPG == 0) {
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
+        for (int e = 0; e < 4; ++e) {
+          sa[e] = 0.f;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) sa[nt][e] = 0.f;
-#pragma unroll
-          for (int rt = 0; rt < 4; ++rt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) accg[rt][nt][e] = 0.f;
+          for (int rt = 0; rt < 4; ++rt) accg[rt][e] = 0.f;
         }
       }
-      uint32_t b0[NT], b1[NT];
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const uint4 v = act[nt][kc][j >> 1];
-        b0[nt] = (j & 1) ? v.z : v.x;
-        b1[nt] = (j & 1) ? v.w : v.y;
-        mma_16816(sa[nt], kOnes, kOnes, kOnes, kOnes, b0[nt], b1[nt]);
-      }
+      const uint4 v = act[kc][j >> 1];
+      const uint32_t b0 = (j & 1) ? v.z : v.x, b1 = (j & 1) ? v.w : v.y;
+      mma_16816(sa, kOnes, kOnes, kOnes, kOnes, b0, b1);
 #pragma unroll
       for (int rt = 0; rt < 4; ++rt) {
         const uint32_t w = (j == 0) ? A[rt].x : (j == 1) ? A[rt].y : (j == 2) ? A[rt].z : A[rt].w;
         const uint32_t w2 = w >> 8;
         const uint32_t a0 = w & 0x000F000Fu, a1 = w & 0x00F000F0u;
         const uint32_t a2 = w2 & 0x000F000Fu, a3 = w2 & 0x00F000F0u;
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) mma_16816(accg[rt][nt], a0, a1, a2, a3, b0[nt], b1[nt]);
+        mma_16816(accg[rt], a0, a1, a2, a3, b0, b1);
       }
       if (blk % BPG == BPG - 1) {
         // group end: zero-point correction and scale
@@ -477,7 +402,7 @@ __device__ __forceinline__ void mma_unit(const uint8_t* __restrict__ U, const ui
         const uint4 sc = *reinterpret_cast<const uint4*>(meta + gid * 16);
         const uint32_t scw[4] = {sc.x, sc.y, sc.z, sc.w};
 #pragma unroll
-        for (int rt = 0; rt < 4; ++rt) group_end<NT>(tot[rt], accg[rt], sa, rt < 2 ? zz.x : zz.y, scw[rt], rt);
+        for (int rt = 0; rt < 4; ++rt) group_end(tot[rt], accg[rt], sa, rt < 2 ? zz.x : zz.y, scw[rt], rt);
       }
     }
   }
@@ -497,31 +422,26 @@ struct GemvPhase {
   float* part;           // OpDesc::q > 0: the CTA's partial sums (shared memory), see swiglu_cta_write
 };
 
-// Loads the B fragments of input unit ku for tokens gid (and gid + 8).
-template <int NT>
-__device__ __forceinline__ void load_act(uint4 (&act)[NT][2][2], const uint16_t* actp, uint32_t acts, int act_ld,
-                                         int M, int ku, int lane) {
-  const int gid = lane >> 2, tig = lane & 3;
+// Loads the B fragments of input unit ku for tokens 8 t + gid.
+__device__ __forceinline__ void load_act(uint4 (&act)[2][2], const uint16_t* actp, uint32_t acts, int act_ld, int M,
+                                         int t, int ku, int lane) {
+  const int n = 8 * t + (lane >> 2), tig = lane & 3;
 #pragma unroll
-  for (int nt = 0; nt < NT; ++nt) {
-    const int n = nt * 8 + gid;
+  for (int kc = 0; kc < 2; ++kc)
 #pragma unroll
-    for (int kc = 0; kc < 2; ++kc)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int off = n * act_ld + ku * kUnitK + kc * 64 + h * 32 + tig * 8;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (n < M) {
-          if (acts)
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                         : "r"(acts + 2u * (uint32_t)off));
-          else
-            v = __ldcg(reinterpret_cast<const uint4*>(actp + off));
-        }
-        act[nt][kc][h] = v;
+    for (int h = 0; h < 2; ++h) {
+      const int off = n * act_ld + ku * kUnitK + kc * 64 + h * 32 + tig * 8;
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (n < M) {
+        if (acts)
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                       : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                       : "r"(acts + 2u * (uint32_t)off));
+        else
+          v = __ldcg(reinterpret_cast<const uint4*>(actp + off));
       }
-  }
+      act[kc][h] = v;
+    }
 }
 
 // kv head of q|k|v row-block rb (each row-block lies inside one head: d is a
@@ -579,7 +499,7 @@ static __device__ __noinline__ void finish_store(const GemvPhase* pp, int rb, in
 // ---------------------------------------------------------------------------
 
 template <int NT>
-__device__ __forceinline__ void swiglu_cta_write(const GemvPhase& p, const float (&tot)[4][NT][4], int w, int lane) {
+__device__ __forceinline__ void swiglu_cta_write(const GemvPhase& p, const float (&tot)[NT][4][4], int w, int lane) {
   const int gid = lane >> 2, tig = lane & 3;
   float* slot = p.part + (size_t)w * p.M * kRowsPerBlock;
 #pragma unroll
@@ -590,8 +510,8 @@ __device__ __forceinline__ void swiglu_cta_write(const GemvPhase& p, const float
       for (int c = 0; c < 2; ++c) {
         const int m = nt * 8 + 2 * tig + c;
         if (m < p.M) {
-          slot[m * kRowsPerBlock + rt * 16 + gid] = tot[rt][nt][c] * 16777216.0f;        // 2^24
-          slot[m * kRowsPerBlock + rt * 16 + gid + 8] = tot[rt][nt][2 + c] * 1048576.0f;  // 2^20
+          slot[m * kRowsPerBlock + rt * 16 + gid] = tot[nt][rt][c] * 16777216.0f;        // 2^24
+          slot[m * kRowsPerBlock + rt * 16 + gid + 8] = tot[nt][rt][2 + c] * 1048576.0f;  // 2^20
         }
       }
 }
@@ -622,7 +542,7 @@ static __device__ __forceinline__ void swiglu_cta_finish(const GemvPhase* pp, in
 // Whole end of a q > 0 run (called by every warp whose group owns a row-block,
 // empty K range or not).
 template <int NT>
-__device__ __forceinline__ void swiglu_cta_end(const GemvPhase* pp, const OpDesc* op, const float (&tot)[4][NT][4],
+__device__ __forceinline__ void swiglu_cta_end(const GemvPhase* pp, const OpDesc* op, const float (&tot)[NT][4][4],
                                                int g, int lane) {
   const int q = op->q;
   const int cta = g / kCtaWarps, w = g - cta * kCtaWarps;
@@ -636,7 +556,7 @@ __device__ __forceinline__ void swiglu_cta_end(const GemvPhase* pp, const OpDesc
 // End of one row-block segment (units of row-block rb) of a warp's run: add
 // the sums to the accumulator, then count the units (see EpiArgs).
 template <int NT>
-__device__ __forceinline__ void segment_end(const GemvPhase* pp, const float (&tot)[4][NT][4], int rb, int units,
+__device__ __forceinline__ void segment_end(const GemvPhase* pp, const float (&tot)[NT][4][4], int rb, int units,
                                             int upr, int lane) {
   const GemvPhase& p = *pp;
   const int gid = lane >> 2, tig = lane & 3;
@@ -651,9 +571,9 @@ __device__ __forceinline__ void segment_end(const GemvPhase* pp, const float (&t
         const int m = nt * 8 + 2 * tig + c;
         if (m < p.M) {
           long long* a = p.ep.acc + (size_t)m * p.ep.acc_ld + rb * kRowsPerBlock + rt * 16 + gid;
-          if (rb * kRowsPerBlock + rt * 16 + gid < rows) red_add_s64(a, f2fix(tot[rt][nt][c] * kTotScaleLo));
+          if (rb * kRowsPerBlock + rt * 16 + gid < rows) red_add_s64(a, f2fix(tot[nt][rt][c] * kTotScaleLo));
           if (rb * kRowsPerBlock + rt * 16 + gid + 8 < rows)
-            red_add_s64(a + 8, f2fix(tot[rt][nt][2 + c] * kTotScaleHi));
+            red_add_s64(a + 8, f2fix(tot[nt][rt][2 + c] * kTotScaleHi));
         }
       }
   if (kind == EPI_RESID) return;
@@ -679,10 +599,11 @@ __device__ __forceinline__ void segment_end(const GemvPhase* pp, const float (&t
 // (which is filled in the same order) and hand on each row-block segment of
 // it.  Inlined at one call site (the whole-step kernel's layer loop, which
 // keeps the ring in registers), so no call boundary spills the caller's
-// registers.  kSeq: two token tiles one after the other per unit, which
-// dequantises twice but holds one tile's activations and group sums at a time
-// (for kernels with 128 registers; the same sums).
-template <int NT, int GPU, int S, bool kSeq = false>
+// registers.  Two token tiles (M > 8) go one after the other per unit: that
+// dequantises twice, but holds one tile's activations and group sums at a time.
+// Both at once spilled (1448 bytes in the step kernel, 232 now; 16 packed tokens
+// at 8B width, 4 layers: 470 -> 400 us; 16 rows of the lm_head 148 -> 123 us).
+template <int NT, int GPU, int S>
 __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* op, const GemvPhase* pp, int g, int nw,
                                          int lane) {
   const GemvPhase& p = *pp;
@@ -691,13 +612,13 @@ __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* o
   run_range(*op, g, nw, wb, we);
   if (wb >= we) {
     if (op->q > 0) {  // a group member without units still adds (zero) sums
-      float zero[4][NT][4];
+      float zero[NT][4][4];
 #pragma unroll
-      for (int rt = 0; rt < 4; ++rt)
+      for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
+        for (int rt = 0; rt < 4; ++rt)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) zero[rt][nt][e] = 0.f;
+          for (int e = 0; e < 4; ++e) zero[nt][rt][e] = 0.f;
       swiglu_cta_end<NT>(pp, op, zero, g, lane);
     }
     return;
@@ -707,51 +628,34 @@ __device__ __forceinline__ void gemv_run(WarpRing<GPU, S>& ring, const OpDesc* o
   const int act_ld = acts ? p.act_s_ld : p.act_ld, M = p.M;
   int rb = wb / upr;
   int ku = wb - rb * upr;
-  constexpr int kAt = kSeq ? 1 : NT;  // token tiles at a time
-  uint4 nxt[kAt][2][2];
-  load_act<kAt>(nxt, actp, acts, act_ld, M, ku, lane);
+  uint4 nxt[2][2];
+  load_act(nxt, actp, acts, act_ld, M, 0, ku, lane);
   for (int u = wb; u < we; ++rb) {
     const int seg_begin = u, rb_end = (rb + 1) * upr;
     const int seg_end = we < rb_end ? we : rb_end;
-    float tot[4][NT][4];
+    float tot[NT][4][4];
 #pragma unroll
-    for (int rt = 0; rt < 4; ++rt)
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
+      for (int rt = 0; rt < 4; ++rt)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) tot[rt][nt][q] = 0.f;
-#pragma unroll 2  // alternating activation registers instead of copies
+        for (int e = 0; e < 4; ++e) tot[nt][rt][e] = 0.f;
+    // two units or tiles per pass: alternating activation registers instead of copies
+#pragma unroll(NT == 1 ? 2 : 1)
     for (; u < seg_end; ++u) {
       const uint8_t* U = nullptr;
 #pragma unroll
-      for (int t0 = 0; t0 < NT; t0 += kAt) {
-        uint4 cur[kAt][2][2];
+      for (int t = 0; t < NT; ++t) {
+        uint4 cur[2][2];
 #pragma unroll
-        for (int nt = 0; nt < kAt; ++nt)
+        for (int kc = 0; kc < 2; ++kc)
 #pragma unroll
-          for (int kc = 0; kc < 2; ++kc)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) cur[nt][kc][h] = nxt[nt][kc][h];
-        const int t1 = (t0 + kAt) % NT;  // the next tiles, of this unit or the next
-        if (t1 == 0 && ++ku == upr) ku = 0;
-        if (t1 > 0 || u + 1 < we) load_act<kAt>(nxt, actp + (size_t)8 * t1 * act_ld, acts ? acts + 16u * t1 * act_ld : 0u, act_ld, M - 8 * t1, ku, lane);
-        if (t0 == 0) U = ring.acquire();
-        if (!ring.timed_out) {
-          if constexpr (kAt == NT) {
-            mma_unit<NT, GPU>(U, cur, tot, lane);
-          } else {
-            float one[4][1][4];
-#pragma unroll
-            for (int rt = 0; rt < 4; ++rt)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) one[rt][0][e] = tot[rt][t0][e];
-            mma_unit<1, GPU>(U, cur, one, lane);
-#pragma unroll
-            for (int rt = 0; rt < 4; ++rt)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) tot[rt][t0][e] = one[rt][0][e];
-          }
-        }
+          for (int h = 0; h < 2; ++h) cur[kc][h] = nxt[kc][h];
+        // the next tile's activations, of this unit or the next
+        if (t + 1 == NT && ++ku == upr) ku = 0;
+        if (t + 1 < NT || u + 1 < we) load_act(nxt, actp, acts, act_ld, M, (t + 1) % NT, ku, lane);
+        if (t == 0) U = ring.acquire();
+        if (!ring.timed_out) mma_unit<GPU>(U, cur, tot[t], lane);
       }
       ring.release(lane);
     }
