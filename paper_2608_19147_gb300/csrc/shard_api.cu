@@ -606,10 +606,17 @@ int kv_state_load(kvstate_t st, int row, int layer, const uint16_t* k, const uin
   // head-major pool: a strided copy of 256-byte rows per head took 16 calls a
   // layer (8 rows of 128..2048 entries into 4 layers of the 8B shape: 6.5 -> 2.6 ms)
   const size_t per = (size_t)sh->Hkv * sh->d;  // values per entry
-  const int most = (int)std::max<size_t>(1, kLoadStageBytes / (2 * sizeof(uint16_t) * per));
+  int most = (int)std::max<size_t>(1, std::min<size_t>(len, kLoadStageBytes / (2 * sizeof(uint16_t) * per)));
+  if (len > 0) {
+    cudaError_t e;
+    while ((e = grow_stage(sh, 2 * sizeof(uint16_t) * per * most)) == cudaErrorMemoryAllocation && most > 1) {
+      cudaGetLastError();  // little memory left: smaller pieces
+      most = (most + 1) / 2;
+    }
+    CUDA_TRY(e);
+  }
   for (int j0 = 0; j0 < len; j0 += most) {
     const int n = std::min(most, len - j0);
-    CUDA_TRY(grow_stage(sh, 2 * sizeof(uint16_t) * per * n));
     uint16_t* in = static_cast<uint16_t*>(sh->dstage);
     const size_t bytes = sizeof(uint16_t) * per * n, off = (size_t)layer * st->layer_stride + (size_t)j0 * sh->d;
     CUDA_TRY(cudaMemcpy(in, k + per * j0, bytes, cudaMemcpyHostToDevice));
