@@ -47,6 +47,7 @@
 #include <mutex>
 
 #include "gemv_core.cuh"
+#include "launch.cuh"
 
 namespace shard {
 namespace {
@@ -236,16 +237,28 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
   // the MMAs of step k, up to group gq
   auto wait_done = [&](int k, int gq) { wait(&done[(k % kBStages) * G + gq], (k / kBStages) & 1); };
 
+  auto load_units = [&](int k) {
+    const int su = k % kUStages;
+    mbar_arrive_expect_tx(&u_full[su], 2 * UB);
+    for (int u = 0; u < 2; ++u) {
+      const int rb = rb0 + u < a.n_rb ? rb0 + u : rb0;  // a missing second block repeats the first (unused)
+      bulk_g2s(U_of(su) + (size_t)u * UB, a.units + ((size_t)rb * a.upr + k_begin + k) * UB, UB, &u_full[su]);
+    }
+  };
+  // the weights are constant: the first units come in while the kernel before ends
+  if (tid == 0)
+    for (int k = 0; k < kUStages && k < steps; ++k) load_units(k);
+  pdl_wait();
+  pdl_launch_dependents();
+
   if (warp == 0) {
     // ---- producer: units and token tiles, kUStages / kBStages steps ahead ----
     if (lane == 0) {
       for (int k = 0; k < steps; ++k) {
         const int su = k % kUStages, sb = k % kBStages;
-        wait(&u_empty[su], ((k / kUStages) & 1) ^ 1);
-        mbar_arrive_expect_tx(&u_full[su], 2 * UB);
-        for (int u = 0; u < 2; ++u) {
-          const int rb = rb0 + u < a.n_rb ? rb0 + u : rb0;  // a missing second block repeats the first (unused)
-          bulk_g2s(U_of(su) + (size_t)u * UB, a.units + ((size_t)rb * a.upr + k_begin + k) * UB, UB, &u_full[su]);
+        if (k >= kUStages) {
+          wait(&u_empty[su], ((k / kUStages) & 1) ^ 1);
+          load_units(k);
         }
         if (k >= kBStages) wait_done(k - kBStages, G - 1);
         mbar_arrive_expect_tx(&full[sb], N * 256);
@@ -459,8 +472,7 @@ cudaError_t launch_tc(const GemmArgs& a, cudaStream_t s) {
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   const dim3 grid((a.n_rb + 1) / 2, (a.S + N - 1) / N, a.parts);
-  gemm_tc_kernel<N, GPU><<<grid, kTcThreads, L::kTotal, s>>>(p);
-  return cudaGetLastError();
+  return launch_behind(gemm_tc_kernel<N, GPU>, grid, kTcThreads, L::kTotal, s, p);
 }
 
 template <int N, int GPU>

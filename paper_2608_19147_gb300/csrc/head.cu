@@ -8,7 +8,7 @@
 //                     plain store epilogue, launched with programmatic
 //                     dependent launch so its weight ring fills while the
 //                     norm finishes;
-//   head_top1_kernel  (chunk, row) CTAs: each reduces a chunk of the row's
+//   head_top1_kernel  (chunk, row) CTAs, launched the same way: each reduces a chunk of the row's
 //                     logits to (max, lowest argmax, sum of exp relative to
 //                     the max); the CTA that finishes a row last combines the
 //                     chunks in chunk order (a fixed order: deterministic).

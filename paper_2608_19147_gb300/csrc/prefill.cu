@@ -7,9 +7,16 @@
 // contractions here and run on the tensor cores (gemm_tc.cu), the attention on
 // mma.sync over blocks of tokens (prefill_flash_kernel); the rest are small
 // per-token kernels, launched layer by layer on the caller's stream.
+// Each of a layer's eight kernels is launched behind the one before it
+// (launch.cuh): its CTAs take their places, and a projection's also fill their
+// rings of weights, while that one ends. It lets the next one come only after
+// its own wait, so a kernel sees all kernels before it ended, not just the last.
+// Bound otherwise by launch gaps of 1.5..2.5 us each: 4 layers at 8B width, 77
+// tokens 704 -> 622 us, 512 tokens 1509 -> 1452.
 #include <algorithm>
 
 #include "common.cuh"
+#include "launch.cuh"
 
 namespace shard {
 namespace {
@@ -48,6 +55,8 @@ __global__ void __launch_bounds__(kNormThreads) prefill_norm_kernel(const __grid
   constexpr int kP = 8;
   __shared__ float s_part[kNormThreads / 32];
   const int t = blockIdx.x, tid = threadIdx.x, H4 = a.H / 4;
+  pdl_wait();
+  pdl_launch_dependents();
   float4* xr = reinterpret_cast<float4*>(a.x + (size_t)t * a.H);
   const uint16_t* in = nullptr;
   if (a.hidden_in) {
@@ -138,6 +147,8 @@ __global__ void __launch_bounds__(256) prefill_rope_append_kernel(const __grid_c
   const int d = a.d, half = d / 2, h4 = half / 4;
   const int rot = (a.Hq + a.Hkv) * h4, per_tok = rot + a.Hkv * d / 4;
   const int n = a.S * per_tok;
+  pdl_wait();
+  pdl_launch_dependents();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
     const int t = e / per_tok, r = e % per_tok;
     const float* yr = a.y + (size_t)t * a.y_ld;
@@ -279,6 +290,8 @@ __global__ void __launch_bounds__(128) prefill_flash_kernel(const __grid_constan
     const int j = 64 * tile + tid;
     return tid < 64 && j <= last ? __ldg(a.mask + j) : 0;
   };
+  pdl_wait();
+  pdl_launch_dependents();
   if (tile0 < tile1) copy_tile(tile0);
   uint8_t seen = tile0 < tile1 ? mask_of(tile0) : 0;
   for (int e = tid; e < 16 * D; e += 128) {
@@ -497,8 +510,7 @@ cudaError_t launch_attn_t(const PrefillLayerArgs& a, cudaStream_t s) {
   // parts of the cache: as many CTAs as partial slots, at least two tiles each
   // (and no more than one CTA should combine)
   const int parts = std::max(1, std::min(std::min(a.part_slots / (blocks * a.Hkv), tiles / 2), 32));
-  prefill_flash_kernel<D, G><<<dim3(blocks, a.Hkv, parts), 128, kSmem, s>>>(a);
-  return cudaGetLastError();
+  return launch_behind(prefill_flash_kernel<D, G>, dim3(blocks, a.Hkv, parts), 128, kSmem, s, a);
 }
 
 
@@ -530,14 +542,12 @@ cudaError_t launch_set_int(int* p, int v, cudaStream_t s) {
 }
 
 cudaError_t launch_prefill_norm(const PrefillNormArgs& a, cudaStream_t s) {
-  prefill_norm_kernel<<<a.S, kNormThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_behind(prefill_norm_kernel, a.S, kNormThreads, 0, s, a);
 }
 
 cudaError_t launch_prefill_rope_append(const PrefillLayerArgs& a, cudaStream_t s) {
   const int n = a.S * ((a.Hq + a.Hkv) * (a.d / 8) + a.Hkv * a.d / 4);
-  prefill_rope_append_kernel<<<(n + 255) / 256, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_behind(prefill_rope_append_kernel, (n + 255) / 256, 256, 0, s, a);
 }
 
 cudaError_t launch_act_order(const uint16_t* x, int x_ld, int S, int Kp, uint16_t* out, int out_ld, cudaStream_t s) {

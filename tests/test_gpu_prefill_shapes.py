@@ -69,3 +69,37 @@ def test_prefill_attention_parts(name, S, P):
     """Few token blocks over a long cache: the cache is cut into parts, some without a visible entry."""
     _run(name, S, P)
     _run(name, S, P)
+
+
+@pytest.mark.parametrize("name,S", [("g128", 1), ("g64", 40), ("g128", 515)])
+def test_prefill_launch_order(name, S):
+    """A prefill's kernels are launched ahead of each other's ends: prompts one right after the other give the bits
+    of prompts waited for, also where the second reuses the first one's buffers and row."""
+    shape = SHAPES[name]
+    g = GpuShard(shape, synth.make_weights(shape, 31))
+    st = pkg.kv_state_alloc(g.h, 1, 2 * S)
+    d_in = [to_dev(synth.hidden_in(shape, 8, i, S)) for i in range(4)]
+    d_mask = to_dev(np.ones(2 * S, np.uint8))
+    d_pos = [to_dev(np.arange(P, P + S, dtype=np.int32)) for P in (0, S)]
+    s = torch.cuda.Stream()
+
+    def prompts(wait):
+        out = [torch.zeros_like(d_in[0]) for _ in d_in]
+        torch.cuda.synchronize()
+        for i, x in enumerate(d_in):  # two prompts onto the row, then two again
+            if i == 2:
+                pkg.kv_state_reset(st, 0)
+            pkg.shard_prefill(g.h, st, 0, x.data_ptr(), None, S, d_pos[i % 2].data_ptr(), d_mask.data_ptr(),
+                              (1 + i % 2) * S, out[i].data_ptr(), s.cuda_stream)
+            if wait:
+                pkg.shard_sync_status(g.h, s.cuda_stream)
+        pkg.shard_sync_status(g.h, s.cuda_stream)
+        pkg.kv_state_reset(st, 0)
+        return out
+
+    want = prompts(True)
+    for _ in range(5):
+        for a, b in zip(prompts(False), want):
+            assert torch.equal(a, b)
+    pkg.kv_state_free(st)
+    g.close()
