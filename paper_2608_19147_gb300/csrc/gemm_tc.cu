@@ -34,9 +34,10 @@
 // work, ~1150 cycles a step against 512 of tensor time: leaving out, one at a
 // time, the MMAs, the dequantisation's arithmetic, the epilogue's loads or the
 // copies changes a step by 2-6 %. Per launch, 512 tokens at 8B width: gate|up
-// 225 -> 159 us, o and down 73 -> 48, q|k|v 61 -> 46 against the same kernel with
-// three commits a step by one thread, one dequantise set and suspending waits
-// (which, with A in shared memory, ran at the same ~1 us a step).
+// 149 us, o 25, down 70, q|k|v 42; with three commits a step by one thread, one
+// dequantise set and suspending waits (which, with A in shared memory, ran at the
+// same ~1 us a step) and straight-line code for the outputs 225, 73 (o and down)
+// and 61.
 // The token tile sits in the canonical K-major layout with the 128-byte
 // swizzle, as the tensor copy writes it. The
 // arithmetic is the decode projection's: exact (q - z), fp32 sums per group,
@@ -67,7 +68,7 @@ struct TcSmem {
   static constexpr size_t kUOff = kBOff + kBStages * kB;               // [kUStages][kUnits]
   static constexpr int kHLd = 72;                                      // halves per token of the staged SwiGLU rows
   static constexpr size_t kTotal = kUOff + kUStages * kUnits + 1024;   // + alignment slack
-  static_assert((size_t)N * kHLd * 2 <= kBStages * kB, "SwiGLU staging");
+  static_assert((size_t)N * (kTcRows * 4 + kHLd * 2) <= kBStages * kB, "staged sums");
   // tensor memory: two A stages of 64 columns behind the accumulator ring
   static constexpr int kDStages = N == 128 ? 3 : N == 64 ? 6 : 8;
   static constexpr uint32_t kACol = kDStages * N;
@@ -388,24 +389,31 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
       }
       if (k + 1 < steps) load(k + 1);
     }
-    const int rbr = rb0 + (row >> 6);
-    if (a.h) {
-      // SwiGLU: gate row 16 t + r and up row 16 t + r + 8 of a block (8 lanes
-      // apart) give h index 32 rb + 8 t + r. Through shared memory (every copy
-      // into it is done: the last accumulator is), then whole 16-byte pieces.
-      uint16_t* hs = reinterpret_cast<uint16_t*>(smem);
-      const int t = R >> 4, pos = 32 * (row >> 6) + act_pos(8 * t + (R & 7));
+    // The sums go through shared memory (every copy into it is done: the last
+    // accumulator is) into short loops: straight-line code for every column is
+    // fetched for one use, which cost more than the work (4 layers at 8B width,
+    // 77 tokens 621 -> 538 us, 512 tokens 1453 -> 1387; gate|up of 77 tokens 68 -> 49).
+    float* ys = reinterpret_cast<float*>(smem);  // [N][128 rows]
 #pragma unroll
-      for (int c = 0; c < kPer; ++c) {
-        const float up = __shfl_down_sync(0xffffffffu, tot[c], 8);
-        if (!(R & 8)) hs[(c0 + c) * L::kHLd + pos] = f2h(silu(tot[c]) * up);
-      }
+    for (int c = 0; c < kPer; ++c) ys[(c0 + c) * kTcRows + row] = tot[c];
+    const int live = min(N, a.S - n0);  // the tile's tokens
+    if (a.h) {
+      // SwiGLU: gate row 16 t + r and up row 16 t + r + 8 of a block give h index
+      // 32 rb + 8 t + r; staged to go out in whole 16-byte pieces
+      uint16_t* hs = reinterpret_cast<uint16_t*>(ys + N * kTcRows);
+      const int et = tid - kEpiWarp0 * 32;
+      const int u = (et >> 5) & 1, t = (et >> 3) & 3, r = et & 7;  // kEpiWarps * 32 threads: a multiple of 64
+      const int gate = 64 * u + 16 * t + r, pos = 32 * u + act_pos(8 * t + r);
+      named_bar_sync(1, kEpiWarps * 32);
+#pragma unroll 4
+      for (int c = et >> 6; c < live; c += kEpiWarps / 2)
+        hs[c * L::kHLd + pos] = f2h(silu(ys[c * kTcRows + gate]) * ys[c * kTcRows + gate + 8]);
       named_bar_sync(1, kEpiWarps * 32);
       // positions past F (of the last, ragged block) stay as they are: zero
-      for (int e = tid - kEpiWarp0 * 32; e < N * 8; e += kEpiWarps * 32) {
+      for (int e = et; e < live * 8; e += kEpiWarps * 32) {
         const int c = e >> 3, j = 8 * (e & 7);
         const int blk = rb0 + (j >> 5);
-        if (blk >= a.n_rb || n0 + c >= a.S) continue;
+        if (blk >= a.n_rb) continue;
         const uint16_t* src = hs + c * L::kHLd + j;
         uint16_t* dst = a.h + (size_t)(n0 + c) * a.h_ld + 32 * blk + (j & 31);
         if (32 * blk + 32 <= a.F) {
@@ -415,14 +423,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
             if (32 * blk + act_unpos((j & 31) + i) < a.F) dst[i] = src[i];
         }
       }
-    } else if (rbr < a.n_rb) {
-      // natural row order, [part of K][token][row]
-      const int nat = natural_row(a.dims, rbr * kRowsPerBlock + R);
-      float* y = a.y + (size_t)blockIdx.z * a.y_part;
+    } else if (rb0 + (row >> 6) < a.n_rb) {
+      // natural row order, [part of K][token][row]; each thread its own row
+      const int nat = natural_row(a.dims, (rb0 + (row >> 6)) * kRowsPerBlock + R);
+      float* y = a.y + (size_t)blockIdx.z * a.y_part + (size_t)n0 * a.y_ld + nat;
+      const int c1 = min(c0 + kPer, live);
       if (nat >= 0)
-#pragma unroll
-        for (int c = 0; c < kPer; ++c)
-          if (n0 + c0 + c < a.S) y[(size_t)(n0 + c0 + c) * a.y_ld + nat] = tot[c];
+#pragma unroll 4
+        for (int c = c0; c < c1; ++c) y[(size_t)c * a.y_ld] = ys[c * kTcRows + row];
     }
   }
   if (!ok) atomicOr(a.status, ST_WAIT_TIMEOUT);
