@@ -59,6 +59,13 @@ def test_prefill_shapes(name, S, P):
     _run(name, S, P)
 
 
+@pytest.mark.parametrize("S", [95, 96, 97, 128, 190, 192, 193, 280])
+@pytest.mark.parametrize("name", ["g128", "g64"])
+def test_prefill_token_tiles(name, S):
+    """Both sides of each change between tiles of 96 and 128 tokens, full and ragged last tiles."""
+    _run(name, S, 5)
+
+
 @pytest.mark.parametrize("offset", [1, 2, 4])
 def test_prefill_value_aligned_buffers(offset):
     _run("g128", 40, 10, offset)
