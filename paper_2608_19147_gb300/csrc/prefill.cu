@@ -41,6 +41,24 @@ __global__ void prefill_check_kernel(const int* token_ids, int vocab, const int*
   }
 }
 
+// v plus the parts of a projection's output behind y, in order; a fixed trip
+// count, so that all parts' (and several callers') loads are in flight at once.
+__device__ __forceinline__ float4 add_parts(float4 v, const float* y, size_t y_part, int first, int parts) {
+  float4 u[kGemmMaxParts];
+#pragma unroll
+  for (int p = 0; p < kGemmMaxParts; ++p)
+    if (p >= first) u[p] = p < parts ? *reinterpret_cast<const float4*>(y + p * y_part) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int p = 0; p < kGemmMaxParts; ++p)
+    if (p >= first && p < parts) {
+      v.x += u[p].x;
+      v.y += u[p].y;
+      v.z += u[p].z;
+      v.w += u[p].w;
+    }
+  return v;
+}
+
 __global__ void set_int_kernel(int* p, int v) { *p = v; }
 
 // One CTA per token: the residual x[t] (first the input row, later x[t] plus the
@@ -73,15 +91,7 @@ __global__ void __launch_bounds__(kNormThreads) prefill_norm_kernel(const __grid
       const uint2 u = *reinterpret_cast<const uint2*>(in + 4 * c);
       return make_float4(h2f(u.x & 0xFFFFu), h2f(u.x >> 16), h2f(u.y & 0xFFFFu), h2f(u.y >> 16));
     }
-    float4 v = xr[c];
-    for (int p = 0; p < a.parts; ++p) {
-      const float4 y = *(reinterpret_cast<const float4*>(a.y + p * a.y_part + (size_t)t * a.H) + c);
-      v.x += y.x;
-      v.y += y.y;
-      v.z += y.z;
-      v.w += y.w;
-    }
-    return v;
+    return add_parts(xr[c], a.y + (size_t)t * a.H + 4 * c, a.y_part, 0, a.parts);
   };
   auto halves = [](float4 v) {
     return make_uint2((uint32_t)f2h(v.x) | ((uint32_t)f2h(v.y) << 16), (uint32_t)f2h(v.z) | ((uint32_t)f2h(v.w) << 16));
@@ -103,10 +113,19 @@ __global__ void __launch_bounds__(kNormThreads) prefill_norm_kernel(const __grid
   }
   float4 v[kP];
   float ss = 0.f;
+  if (in) {
 #pragma unroll
-  for (int i = 0; i < kP; ++i) {
-    const int c = tid + i * kNormThreads;
-    v[i] = c < H4 ? get(c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < kP; ++i) {
+      const int c = tid + i * kNormThreads;
+      v[i] = c < H4 ? get(c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kP; ++i) {
+      const int c = tid + i * kNormThreads;
+      v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < H4) v[i] = add_parts(xr[c], a.y + (size_t)t * a.H + 4 * c, a.y_part, 0, a.parts);
+    }
   }
 #pragma unroll
   for (int i = 0; i < kP; ++i) {
@@ -153,15 +172,7 @@ __global__ void __launch_bounds__(256) prefill_rope_append_kernel(const __grid_c
     const int t = e / per_tok, r = e % per_tok;
     const float* yr = a.y + (size_t)t * a.y_ld;
     auto get = [&](int row) {
-      float4 v = *reinterpret_cast<const float4*>(yr + row);
-      for (int p = 1; p < a.parts; ++p) {
-        const float4 u = *reinterpret_cast<const float4*>(yr + p * a.y_part + row);
-        v.x += u.x;
-        v.y += u.y;
-        v.z += u.z;
-        v.w += u.w;
-      }
-      return v;
+      return add_parts(*reinterpret_cast<const float4*>(yr + row), yr + row, a.y_part, 1, a.parts);
     };
     auto halves = [](float4 v) {
       return make_uint2((uint32_t)f2h(v.x) | ((uint32_t)f2h(v.y) << 16), (uint32_t)f2h(v.z) | ((uint32_t)f2h(v.w) << 16));
