@@ -48,6 +48,12 @@ int shard_debug_gemv(shard_t shard, int layer, int op, const uint16_t* x, int M,
 int shard_debug_gemm(shard_t shard, int layer, int op, const uint16_t* x, int x_ld, int S, float* y, int y_ld,
                      void* cuda_stream);
 
+/* The many-token projection's token tile for S tokens and its rings, for a
+ * model of its barriers: rings[0..5] = stages of weight units, of token tiles
+ * and of the dequantised A operand, accumulators, MMA-issuing threads,
+ * dequantise sets.  Host only: needs no shard and no GPU. */
+int shard_debug_gemm_rings(int S, int group, int* tile, int* rings);
+
 /* Phase durations of the last completed shard_step, from the GPU's global
  * timer read by one thread at the end of each grid-barrier wait of the step
  * kernel: us[i] is the time between the end of wait i and the end of wait

@@ -59,6 +59,13 @@ constexpr int kTcThreads = kTcWarps * 32;
 constexpr int kMmaWarp0 = 1, kMmaWarps = 2, kEpiWarp0 = 4, kEpiWarps = 8, kDqWarp0 = 12, kDqSets = 2;
 constexpr int kUStages = 6, kBStages = 4, kAStages = 2;
 
+// Accumulators in tensor memory for tiles of N tokens with g groups per step:
+// what the columns hold, and no more than the completion barriers can tell apart.
+constexpr int tc_accumulators(int N, int g) {
+  const int fit = N == 128 ? 3 : N == 96 ? 4 : N == 64 ? 6 : 8;
+  return fit < kBStages * g ? fit : kBStages * g;
+}
+
 template <int N, int GPU>
 struct TcSmem {
   static constexpr size_t kUnit = Geom<GPU>::kUnitBytes;
@@ -70,16 +77,23 @@ struct TcSmem {
   static constexpr size_t kTotal = kUOff + kUStages * kUnits + 1024;   // + alignment slack
   static_assert((size_t)N * (kTcRows * 4 + kHLd * 2) <= kBStages * kB, "staged sums");
   // tensor memory: two A stages of 64 columns behind the accumulator ring
-  static constexpr int kDStages = N == 128 ? 3 : N == 96 ? 4 : N == 64 ? 6 : 8;
+  static constexpr int kDStages = tc_accumulators(N, GPU);
   static constexpr uint32_t kACol = kDStages * N;
   static constexpr uint32_t kCols = 512;
   static_assert(kACol + kAStages * 64 <= kCols, "tensor memory");
-  // Two threads issue steps in turn and may be a step apart: an accumulator's
-  // barrier must not be two phases behind the one that is waited for (parity
-  // waits could not tell). A thread that issues accumulator q has issued q - G
-  // - 1 or later before, so q - G - 1 - kDStages has been read; q - 2 kDStages
-  // must be no later.
+  // A parity wait tells a phase from its neighbours only: neither side of a
+  // barrier may get two phases away from a waiter.
+  // d_empty: two threads issue steps in turn and may be a step apart. A thread
+  // that issues accumulator q has issued q - G - 1 or later before, so q - G -
+  // 1 - kDStages has been read; q - 2 kDStages must be no later.
   static_assert(kDStages >= GPU + 1, "accumulator ring");
+  // done: the epilogue warp that is furthest behind still waits for group q, and
+  // the MMAs have gone on as far as the accumulators let them, up to group q +
+  // kDStages - 1. The barrier's next phase is group q + kBStages G and must not be
+  // among them. (Its other waiters cannot be overtaken: the phase takes a token
+  // tile that the producer sends after its wait for the last one, and four
+  // arrivals of the dequantise set that waits.)
+  static_assert(kDStages <= kBStages * GPU, "completion barriers");
 };
 
 // Shared-memory matrix descriptor, K-major with the 128-byte swizzle: 8-row
@@ -513,6 +527,15 @@ cudaError_t gemm_tc_setup() {
 int gemm_tc_tile(int S, int group) {
   if (S <= 64 || group == 32) return S > 32 ? 64 : 32;
   return (S + 95) / 96 == (S + 127) / 128 ? 96 : 128;
+}
+
+void gemm_tc_rings(int tile, int group, int (&r)[6]) {
+  r[0] = kUStages;
+  r[1] = kBStages;
+  r[2] = kAStages;
+  r[3] = tc_accumulators(tile, kUnitK / group);
+  r[4] = kMmaWarps;
+  r[5] = kDqSets;
 }
 
 // Parts of K for a projection of n_rb row-blocks and upr units on `sms` SMs:

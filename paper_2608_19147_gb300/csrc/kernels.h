@@ -187,6 +187,8 @@ struct GemmArgs {
 };
 cudaError_t gemm_tc_setup();
 int gemm_tc_tile(int S, int group);
+// The kernel's rings for a token tile: stages of units, token tiles and A, accumulators; MMA threads, dequantise sets.
+void gemm_tc_rings(int tile, int group, int (&r)[6]);
 // Parts of K for a projection of S tokens on `sms` SMs, at most kGemmMaxParts.
 constexpr int kGemmMaxParts = 4;
 int gemm_tc_parts(int n_rb, int upr, int S, int group, int sms);

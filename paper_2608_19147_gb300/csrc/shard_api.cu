@@ -1,5 +1,6 @@
 // Host side of libshard: the C ABI declared in include/shard.h and
 // include/shard_debug.h.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1206,6 +1207,16 @@ int shard_debug_gemm(shard_t sh, int layer, int op, const uint16_t* x, int x_ld,
   g.dims = p.dims;
   g.status = sh->status;
   CUDA_TRY(launch_gemm_tc(g, sh->cfg.group, static_cast<cudaStream_t>(cuda_stream)));
+  return SHARD_OK;
+}
+
+int shard_debug_gemm_rings(int S, int group, int* tile, int* rings) {
+  if (S < 1 || (group != 32 && group != 64 && group != 128) || !tile || !rings)
+    return fail(SHARD_EINVAL, "shard_debug_gemm_rings: bad argument");
+  int r[6];
+  *tile = gemm_tc_tile(S, group);
+  gemm_tc_rings(*tile, group, r);
+  std::copy(r, r + 6, rings);
   return SHARD_OK;
 }
 
