@@ -126,7 +126,7 @@ enum EpiKind { EPI_STORE = 0, EPI_QKV = 1, EPI_RESID = 2, EPI_SWIGLU = 3 };
 //   EPI_RESID   acc = the residual stream X [16][H] (fixed point): x += W a.
 //   EPI_QKV     acc = q|k|v sums [16][acc_ld] in the op's row order; each
 //               segment then adds its unit count to cnt[kv head of the
-//               row-block] (release), which the attention items wait for.
+//               row-block] (release), which the attention waits for.
 //   EPI_SWIGLU  acc = gate|up sums [16][acc_ld]; cnt[row-block] counts the
 //               units added; the contributor that completes a row-block reads
 //               the sums, writes h = fp16(silu(gate) * up) and clears the
@@ -300,7 +300,7 @@ struct StepKernelArgs {
   const uint8_t* mask;
   int mask_stride;
   int packed;                // mask row per token (one request), no implicit causal bound
-  float* attn_part;          // [item][16*G][d+4]; rows are cut into items only while every CTA has one at most
+  float* attn_part;          // attention partials of rows of several chunks, [request][kv head][chunk][query][d+4]
   int* attn_cnt;             // [16][Hkv] finished chunks per (request, kv head), zero between steps
   int* status;
   unsigned long long* barrier;         // grid-barrier counter (monotonic)
@@ -311,28 +311,30 @@ struct StepKernelArgs {
   int* exit_count;           // CTAs finished in this launch (zero between launches; the last resets it)
   int debug_skip_arrival;    // test knob: >= 0 makes CTA 1 skip that grid barrier's arrival
   unsigned wait_limit;       // polls before a cross-CTA wait gives up
-  uint32_t area_bytes;       // shared memory for attention items and normalised rows (step_area_bytes)
+  uint32_t area_bytes;       // shared memory for the attention and normalised rows (step_area_bytes)
   int gu_part;               // 1: shared memory holds the gate|up partial sums (OpDesc::q may be used)
 };
 // One-time attribute setup of the step kernel variants for a group size and
 // head dim; number of grid barriers per step; launch (cooperative, one CTA
 // per SM).
 cudaError_t step_setup(int group, int head_dim);
+// Dynamic shared memory that every step kernel of a group size and head dim may take (after step_setup).
+size_t step_dyn_limit(int group, int head_dim);
 // Warps per row-block for the shared-memory reduction of a gate|up
 // projection of n_rb row-blocks of upr units on `grid` CTAs (0: the
-// grid-wide split), when the kernel's shared memory for L layers leaves room
-// for the partial sums.
-int step_gu_split(int n_rb, int upr, int grid, int group, int L);
+// grid-wide split).
+int step_gu_split(int n_rb, int upr, int grid);
 // Whether the kernel's shared memory for L layers has room for the partial
 // sums of the largest step.
-bool step_gu_part_fits(int group, int L);
+bool step_gu_part_fits(int group, int L, size_t limit);
 // Shared memory of the attention / normalised-row area for steps of M tokens.
-size_t step_area_bytes(int group, int H, int L, bool part, int M);
+size_t step_area_bytes(int group, int H, int L, bool part, int M, size_t limit);
 int step_barriers(int n_layers);
 cudaError_t launch_step(const StepKernelArgs& a, int nt, int group, int grid, cudaStream_t s);
-// Size of the attention partials for a grid of that many CTAs.
+// Size of the attention partials: a row that is cut has no more chunks, over all kv
+// heads, than CTAs, and a step has no more than 16 G queries of a kv head.
 size_t step_attention_part_floats(int grid, int G, int d);
-constexpr int kAttnChunkMin = 64;  // fewest cache entries per attention item
+constexpr int kAttnChunkMin = 64;  // fewest cache entries per attention chunk
 
 // Weight repacking (one fused op; all source pointers device).
 // Source matrices of a fused op (q, k, v for OP_QKV; gate, up for OP_GU; one

@@ -470,20 +470,21 @@ int shard_create(const shard_config* cfg, const shard_weights_host* w, shard_t* 
   CUDA_TRY(cudaMalloc(&sh->norm_cnt, sizeof(int)));
   CUDA_TRY(cudaMalloc(&sh->exit_count, sizeof(int)));
   CUDA_TRY(cudaMemset(sh->exit_count, 0, sizeof(int)));
+  const size_t limit = step_dyn_limit(sh->cfg.group, sh->d);
+  sh->gu_part = step_gu_part_fits(sh->cfg.group, sh->L, limit);
   {
     std::vector<OpDesc> od(sh->ops.size());
     for (size_t i = 0; i < od.size(); ++i) {
       const auto& o = sh->ops[i];
       // gate|up (op 2 of each layer): shared-memory reduction when it fits
-      const int q = i % 4 == 2 ? step_gu_split(o.n_rb, o.upr, sh->num_sms, sh->cfg.group, sh->L) : 0;
+      const int q = i % 4 == 2 && sh->gu_part ? step_gu_split(o.n_rb, o.upr, sh->num_sms) : 0;
       od[i] = OpDesc{o.units, o.n_rb, o.upr, q};
     }
     CUDA_TRY(cudaMalloc(&sh->ops_dev, sizeof(OpDesc) * od.size()));
     CUDA_TRY(cudaMemcpy(sh->ops_dev, od.data(), sizeof(OpDesc) * od.size(), cudaMemcpyHostToDevice));
   }
-  sh->gu_part = step_gu_part_fits(sh->cfg.group, sh->L);
   for (int m = 1; m <= kMaxTokens; ++m)
-    sh->area_bytes[m] = (uint32_t)step_area_bytes(sh->cfg.group, sh->H, sh->L, sh->gu_part, m);
+    sh->area_bytes[m] = (uint32_t)step_area_bytes(sh->cfg.group, sh->H, sh->L, sh->gu_part, m, limit);
   sh->n_barriers = step_barriers(sh->L);
   CUDA_TRY(cudaMalloc(&sh->barrier, sizeof(unsigned long long)));
   CUDA_TRY(cudaMalloc(&sh->phase_clock, sizeof(unsigned long long) * (sh->n_barriers + 1)));

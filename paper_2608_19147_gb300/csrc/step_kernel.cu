@@ -169,7 +169,10 @@ __device__ __forceinline__ bool wait_count(const int* p, int target, int* status
 // entries; K/V stay where they are), the new entries' slots -- and the
 // device-side argument checks.  Every CTA derives the same values.
 // ---------------------------------------------------------------------------
-__device__ __noinline__ void prologue_params(const PrologueArgs& a, StepParams* sp, const uint16_t** rowp) {
+// `plan` runs on warp 2 once the lengths are known, behind the other checks' loads.
+template <class Plan>
+__device__ __noinline__ void prologue_params(const PrologueArgs& a, StepParams* sp, const uint16_t** rowp,
+                                             const Plan& plan) {
   __shared__ int s_err;
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -203,6 +206,7 @@ __device__ __noinline__ void prologue_params(const PrologueArgs& a, StepParams* 
     sp->req_len[tid] = L;
   }
   __syncthreads();
+  if (tid >> 5 == 2) plan(tid & 31);
   if (tid < a.M) {
     const int m = tid, b = sp->tok_req[m], i = sp->tok_idx[m], j = sp->req_P[b] + i;
     // a token must see its own entry (packed: in its own mask row, Section 8.6)
@@ -401,10 +405,15 @@ __device__ __forceinline__ void rmsnorm_staged(const long long* X, int H, const 
 }
 
 // ---------------------------------------------------------------------------
-// Attention.  Item = (request b, kv head hk, chunk c of cs entries); one CTA
-// per item.  cs is the smallest multiple of 16, from kAttnChunkMin up, that
-// gives no more items than CTAs; when there are more (request, kv head) pairs
-// than CTAs, an item is a whole row and CTAs take several.
+// Attention.  Chunk = (request b, kv head hk, cs entries): cs is the smallest
+// multiple of 16, from kAttnChunkMin up, that gives no more chunks than CTAs for
+// that row alone (the whole row when it has more kv heads than that).  A chunk's
+// result, and the order in which a row's chunks meet, depend on the row's length
+// and queries only, so a row has the same bits alone and in any batch.  A CTA
+// takes a unit, a run of chunks of one (request, kv head): one each while all
+// rows' chunks find a CTA, longer runs (the same share of entries for every CTA)
+// when they do not; when there are more (request, kv head) pairs than CTAs, a unit
+// is a whole row and CTAs take several.
 //
 // The bound is the K/V stream (32 KB per 64 entries of a head at d = 128, each
 // byte read once) and, for short caches, the chain of dependent L2 round
@@ -417,18 +426,23 @@ __device__ __forceinline__ void rmsnorm_staged(const long long* X, int H, const 
 //     keeps its next block's rows in flight while it works on the last;
 //   - queries go in tiles of 8: a tile's 16 MMA rows are the 8 queries' fp16
 //     values and what that rounding left out (after scaling each query by a
-//     power of two to a largest value in [1, 2)), so the scores carry an fp32
-//     query at one MMA per tile; probabilities (times 2^12) are split the
-//     same way for the value sum.  Sums are fp32, the softmax is online per
-//     warp.
+//     power of two to a largest value in [1, 2)), 22 to 23 bits of the row's
+//     largest value at one MMA per tile; probabilities (times 2^12) are split
+//     the same way for the value sum.  Sums are fp32, the softmax is online per
+//     warp.  Against 64 bits the outputs before rounding are about half as far off
+//     as with fp32 queries and probabilities in chains of FMAs (2.1e-3..9.3e-3 of
+//     the fp16 outputs rounded the other way, now 1.2e-3..3.8e-3; 30..4000 entries,
+//     1..16 tokens, scores of deviation 1 and 6).
 // A warp holds one query tile; kWarps / tiles warps side by side take different
 // blocks (a tile's blocks meet the other tiles' reads of them in L1), and the
-// CTA adds their pieces in shared memory in a fixed order.  Two tiles per warp
+// CTA adds a chunk's pieces in shared memory in a fixed order (in a run of chunks a
+// warp works through a tile of a chunk alone, attn_run).  Two tiles per warp
 // would halve the L1 reads, but their accumulators and the rows in flight do
-// not fit 168 registers.  Chunks of one
-// (request, kv head) meet in `part`: the CTA that finishes the last one merges
-// when that is little to read, else every chunk's CTA waits for the others
-// and merges its share of the queries.
+// not fit 168 registers.  Chunks of one (request, kv head) meet in `part`: the CTA
+// that finishes the last one merges when that is little to read, else every unit's
+// CTA waits for the others and merges its share of the queries.  Steps of one
+// request and of several are kernels of their own (kMany): with both in one, its
+// registers and code made every step 2 to 4 % slower.
 //
 // First layer's attention phase, against the CUDA-core version before it (a warp
 // per query over 64-entry tiles in shared memory, a CTA's items one after
@@ -441,7 +455,7 @@ __device__ __forceinline__ void rmsnorm_staged(const long long* X, int H, const 
 // output starts 16-byte aligned.
 __host__ __device__ constexpr int part_stride(int d) { return d + 4; }
 
-constexpr int kAttnQ = 64;        // queries per pass over an item's entries
+constexpr int kAttnQ = 64;        // queries per pass over a chunk's entries
 constexpr int kAttnWin = 1024;    // entries whose slots and visibility are staged at a time
 constexpr float kProbScale = 4096.f;
 
@@ -452,54 +466,83 @@ struct AttnView {
   uint16_t* kpool;          // layer 0; layer l at + l * layer_stride
   uint16_t* vpool;
   size_t layer_stride;
-  int cap, Hq, Hkv, d, qmax;
-  float* part;              // [item][16 * G queries][d + 4]
-  int* cnt;                 // finished chunks per (request, kv head)
+  int cap, Hq, Hkv, d;
+  float* part;              // [request][kv head][chunk][query][d + 4], AttnPlan::part0
   const int* cnt_kv;        // q|k|v units finished per kv head
   int kv_units;             // units per kv head when its q|k|v rows are complete
   const int* bt;            // beam table (entry -> physical slot) of this step
   const uint8_t* mask;
   int mask_stride;
   int packed;               // a mask row per token of request 0 instead of one per request
-  int cs;                   // entries per item this step
-  int total;                // items this step
   uint32_t limit;
   uint16_t* out;
   int out_ld;
 };
 
-__device__ __forceinline__ int n_chunks_of(int L, int cs) { return (L + cs - 1) / cs; }
+// A quotient in code that runs once per launch: inlined divisions are a good part
+// of such code, and fetching it is what it costs.
+__device__ __noinline__ unsigned quotient(unsigned a, unsigned b) { return a / b; }
+__device__ __forceinline__ int n_chunks_of(int L, int cs) { return (int)quotient(L + cs - 1, cs); }
 
-// The step's item size and count (one warp; lane b takes request b).
-__device__ __forceinline__ void attn_plan(const StepParams* sp, int Hkv, int grid, int lane, int& cs, int& total) {
-  const int L = lane < sp->B ? sp->req_len[lane] : 0;
+// Entries per chunk of a row of L entries: a function of the row alone.  (A row's
+// entries times kv heads fit 32 bits: the pool holds 256 bytes or more for each.)
+__device__ __forceinline__ int chunk_entries(int L, int Hkv, int grid) {
+  int cs = max(kAttnChunkMin, (int)(quotient((unsigned)L * Hkv + grid - 1, grid) + 15) / 16 * 16);
+  // rounding up can need a little more than the even share
+  while (cs < L && Hkv * n_chunks_of(L, cs) > grid) cs += 16 * max(1, cs / 256);
+  return min(cs, L);
+}
+
+// The attention of a step of several requests: filled by one warp, lane b for request b.
+struct AttnPlan {
+  int cs[kMaxRequests];     // entries per chunk of a request,
+  int run[kMaxRequests];    // chunks per unit,
+  int unit0[kMaxRequests];  // its first unit,
+  int part0[kMaxRequests];  // and its first partial (rows of several chunks have them)
+};
+
+// Sum of v over the lanes before this one.
+__device__ __forceinline__ int lanes_before(int v, int lane) {
+  int t = v;
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, t, o);
+    if (lane >= o) t += u;
+  }
+  return t - v;
+}
+
+// Runs grow from the even share of all entries until every unit finds a CTA, or
+// are whole rows.  Returns the number of units.
+__device__ __forceinline__ int attn_plan(const StepParams* sp, int G, int Hkv, int grid, int lane, AttnPlan* plan) {
   const unsigned all = 0xffffffffu;
-  const int longest = __reduce_max_sync(all, L), sum = __reduce_add_sync(all, L);
-  cs = max(kAttnChunkMin, (int)(((long long)sum * Hkv + grid - 1) / grid + 15) / 16 * 16);
-  // rounding up per row can need a little more than the even share
-  while (cs < longest) {
-    total = Hkv * __reduce_add_sync(all, n_chunks_of(L, cs));
-    if (total <= grid) return;
-    cs += 16 * max(1, cs / 256);
+  const bool mine = lane < sp->B;
+  const int L = mine ? sp->req_len[lane] : 0;
+  const int cs = mine ? chunk_entries(L, Hkv, grid) : 1, nc = mine ? n_chunks_of(L, cs) : 0;
+  int share = max(kAttnChunkMin, (int)quotient((unsigned)__reduce_add_sync(all, L) * Hkv + grid - 1, grid));
+  int run, units, total;
+#pragma unroll 1
+  for (;;) {
+    run = min(max((int)quotient(share, cs), 1), nc);
+    units = mine ? Hkv * n_chunks_of(nc, run) : 0;
+    total = __reduce_add_sync(all, units);
+    if (total <= grid || __all_sync(all, run == nc)) break;
+    share += 16 * max(1, share / 256);
   }
-  cs = longest;
-  total = Hkv * sp->B;
+  const int unit0 = lanes_before(units, lane);
+  const int queries = mine ? G * (sp->req_tok0[lane + 1] - sp->req_tok0[lane]) : 0;
+  const int part0 = lanes_before(nc > 1 ? Hkv * nc * queries : 0, lane);
+  if (mine) {
+    plan->cs[lane] = cs;
+    plan->run[lane] = run;
+    plan->unit0[lane] = unit0;
+    plan->part0[lane] = part0;
+  }
+  __syncwarp();
+  return total;
 }
 
-// Finds the item's (b, hk, c) from a flat index.
-__device__ __forceinline__ void decode_item(const StepParams* sp, int Hkv, int cs, int item, int& b, int& hk, int& c) {
-  hk = c = 0;
-  for (b = 0; b < sp->B - 1; ++b) {
-    const int per = Hkv * n_chunks_of(sp->req_len[b], cs);
-    if (item < per) break;
-    item -= per;
-  }
-  const int nc = n_chunks_of(sp->req_len[b], cs);
-  hk = item / nc;
-  c = item - hk * nc;
-}
-
-// Shared-memory layout of one attention item.  Query rows are padded so that
+// Shared-memory layout of a unit's attention.  Query rows are padded so that
 // the two rows of a quarter-warp's 16-byte loads fall on different banks.
 template <int DPL>
 struct AttnSmem {
@@ -510,7 +553,7 @@ struct AttnSmem {
   static constexpr size_t kVis = (size_t)kAttnWin * 2;            // bit t: token t sees the entry
   static constexpr size_t kScale = (size_t)kAttnQ * 4;            // score scale of each query
   static constexpr size_t kLoop = 2 * kQ + kRows + kVis + kScale;
-  // the same space, once the entries are done: a tile's pieces of every warp
+  // the same space, once a chunk's entries are done: a tile's pieces of every warp
   static constexpr int kOld = part_stride(d);                     // floats per query of a piece
   static constexpr size_t kPieces = (size_t)kWarps * 8 * kOld * 4;
   static constexpr size_t kMl = (size_t)kWarps * 8 * 8;           // (max, sum) per piece and query
@@ -640,17 +683,256 @@ __device__ __forceinline__ void attn_merge_warp(const float* base, size_t cstrid
 // at d = 128; 64 of them are one batch of loads per warp).
 constexpr int kMergeAlone = 64;
 
-// One item, processed by the CTA's consumer warps.
-template <int DPL>
-__device__ __forceinline__ void attn_item_cta(const AttnView* ap, int layer, const StepParams* sp, int item,
-                                              uint8_t* area, int* status) {
-  const AttnView& a = *ap;
+// attn_run's warps share the area with their scores: below this many (chunks of more
+// than 16 blocks for one query tile, of more than 11 for three) a unit goes chunk by
+// chunk.  Layer 0's attention at 8B width, run / chunk by chunk: 4 rows of 2000
+// entries 20 / 37 us, of 3500 (6 warps) 33 / 48, of 4300 (5) 63 / 58, of 5500 (4)
+// 78 / 61, of 7500 (3) 140 / 76; 3 rows of 5 tokens on 2000 (8) 31 / 49, on 3000 (5)
+// 45 / 48, on 5000 (3) 128 / 83.
+constexpr int kRunWarps = 5;
+
+// A CTA's unit, laid out once per launch (by one thread) for all layers.
+struct AttnUnit {
+  int total;                // the step's units
+  int hk, tok0, nb, Q, P;
+  int row;                  // of the mask and the beam table
+  int cs, nc, c0, c1;       // entries per chunk, chunks of the row, this unit's
+  int end;                  // the entry after the row's last
+  int u, units;             // its place among the units of its (request, kv head)
+  int part0;                // the (request, kv head)'s first partial
+  int* cnt;                 // finished chunks of the (request, kv head)
+  // attn_run, for units of several chunks (warps = 0: chunk by chunk, attn_chunk)
+  int warps;                // that take part
+  uint32_t qlo, rows;       // byte offsets in the area
+};
+
+// A step of one request: every chunk is a unit.
+__device__ __forceinline__ void attn_one_row(const StepParams& sp, int Hkv, int grid, AttnUnit& n) {
+  n.cs = chunk_entries(sp.req_len[0], Hkv, grid);
+  n.nc = n_chunks_of(sp.req_len[0], n.cs);
+  n.total = Hkv * n.nc;
+}
+
+template <int DPL, bool kMany>
+__device__ __noinline__ void attn_unit_init(const AttnPlan& plan, const StepParams& sp, int G, int Hkv, int* cnt,
+                                            uint32_t area_bytes, int unit, AttnUnit& n) {
   using S = AttnSmem<DPL>;
-  constexpr int d = S::d, half = d / 2;
-  constexpr int KJ = d / 32;   // 16-byte pieces of a lane's K row share
-  constexpr int VJ = d / 64;   // 16-byte pieces of a lane's V row share
-  int b, hk, c;
-  decode_item(sp, a.Hkv, a.cs, item, b, hk, c);
+  int b = 0, run = 1, part0 = 0;
+  if (kMany) {
+    b = sp.B - 1;
+#pragma unroll 1
+    while (plan.unit0[b] > unit) --b;
+    unit -= plan.unit0[b];
+    run = plan.run[b];
+    part0 = plan.part0[b];
+    n.cs = plan.cs[b];
+    n.nc = n_chunks_of(sp.req_len[b], n.cs);
+  }
+  const int units = kMany ? n_chunks_of(n.nc, run) : n.nc, hk = (int)quotient(unit, units);
+  const int u = unit - hk * units, nb = sp.req_tok0[b + 1] - sp.req_tok0[b], Q = nb * G;
+  n.row = b;
+  n.hk = hk;
+  n.tok0 = sp.req_tok0[b];
+  n.nb = nb;
+  n.Q = Q;
+  n.P = sp.req_P[b];
+  n.end = sp.req_len[b];
+  n.u = u;
+  n.units = units;
+  n.c0 = u * run;
+  n.c1 = min(n.c0 + run, n.nc);
+  n.part0 = part0 + hk * n.nc * Q;
+  n.cnt = cnt + b * Hkv + hk;
+  if (kMany) {
+    // a warp's scores take 512 bytes a block of its chunk, behind the queries and the entries' rows
+    const int nqt = (Q + 7) >> 3, nblk = (n.cs + 15) >> 4;
+    n.qlo = nqt * 8 * S::kQld * 2;
+    n.rows = 2 * n.qlo;
+    const int room = (int)area_bytes - (int)n.rows - (int)(S::kRows + S::kVis + S::kScale);
+    const int fit = room > 0 ? min((int)quotient(room, 512 * nblk), kWarps) : 0;
+    n.warps = n.c1 - n.c0 > 1 && Q <= kAttnQ && n.cs <= kAttnWin && fit >= kRunWarps ? fit : 0;
+  }
+}
+
+// K rows of block blk: entries gid and gid + 8; a lane's share of each is d / 4 values.
+template <int DPL>
+__device__ __forceinline__ void attn_load_k(uint4 (&kf)[2][DPL], const uint16_t* kpool, const uint32_t* rows_s, int blk,
+                                            int gid, int tig) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const uint4* p = reinterpret_cast<const uint4*>(kpool + (size_t)rows_s[16 * blk + 8 * i + gid] * (32 * DPL)) + tig;
+#pragma unroll
+    for (int j = 0; j < DPL; ++j) kf[i][j] = p[4 * j];
+  }
+}
+
+// V rows of block blk: entries 2 tig, + 1, + 8, + 9; a lane's share of each is d / 8 values.
+template <int DPL>
+__device__ __forceinline__ void attn_load_v(uint4 (&vf)[4][DPL / 2], const uint16_t* vpool, const uint32_t* rows_s,
+                                            int blk, int gid, int tig) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const uint4* p = reinterpret_cast<const uint4*>(
+                         vpool + (size_t)rows_s[16 * blk + 8 * (r >> 1) + 2 * tig + (r & 1)] * (32 * DPL)) + gid;
+#pragma unroll
+    for (int j = 0; j < DPL / 2; ++j) vf[r][j] = p[8 * j];
+  }
+}
+
+// Scores of query gid (qh, ql: its values and their remainders; qs: its scale, tk:
+// its token) and entries 2 tig, + 1, + 8, + 9 of a block, -inf where it does not
+// see them (vis: the block's bits).
+template <int DPL>
+__device__ __forceinline__ void attn_scores(float (&x)[4], const uint4 (&kf)[2][DPL], const uint16_t* qh,
+                                            const uint16_t* ql, const uint16_t* vis, int tk, float qs, int tig) {
+  const uint32_t va = *reinterpret_cast<const uint32_t*>(vis + 2 * tig) >> tk;
+  const uint32_t vb = *reinterpret_cast<const uint32_t*>(vis + 8 + 2 * tig) >> tk;
+  float s[2][2][4];  // two chains per 8 entries
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) s[i][e][0] = s[i][e][1] = s[i][e][2] = s[i][e][3] = 0.f;
+#pragma unroll
+  for (int j = 0; j < DPL; ++j) {
+    const uint4 h = *reinterpret_cast<const uint4*>(qh + 32 * j);
+    const uint4 l = *reinterpret_cast<const uint4*>(ql + 32 * j);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      mma_16816(s[i][0], h.x, l.x, h.y, l.y, kf[i][j].x, kf[i][j].y);
+      mma_16816(s[i][1], h.z, l.z, h.w, l.w, kf[i][j].z, kf[i][j].w);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float (&u)[2][4] = s[i >> 1];
+    const int e = i & 1;
+    const bool see = ((i < 2 ? va : vb) >> (16 * e)) & 1u;
+    x[i] = see ? ((u[0][e] + u[1][e]) + (u[0][2 + e] + u[1][2 + e])) * qs : -INFINITY;
+  }
+}
+
+__device__ __forceinline__ float attn_block_max(const float (&x)[4]) {
+  float mn = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+  mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
+  return fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
+}
+
+// A block's probabilities and value sum into the running (mx, den, o): online softmax.
+template <int DPL>
+__device__ __forceinline__ void attn_values(const float (&x)[4], const uint4 (&vf)[4][DPL / 2], float (&o)[2 * DPL][4],
+                                            float& mx, float& den, int tig) {
+  const float mn = fmaxf(attn_block_max(x), mx);
+  if (__any_sync(0xffffffffu, mn > mx)) {
+    const float alpha = mx == -INFINITY ? 0.f : expf(mx - mn);
+    den *= alpha;
+    const float a0 = __shfl_sync(0xffffffffu, alpha, 8 * tig), a1 = __shfl_sync(0xffffffffu, alpha, 8 * tig + 4);
+#pragma unroll
+    for (int i = 0; i < 2 * DPL; ++i) {
+      o[i][0] *= a0;
+      o[i][1] *= a1;
+      o[i][2] *= a0;
+      o[i][3] *= a1;
+    }
+    mx = mn;
+  }
+  uint32_t ph[2], pl[2];  // the probabilities as the value sum's B fragments
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float p0 = x[2 * i] == -INFINITY ? 0.f : expf(x[2 * i] - mn) * kProbScale;
+    const float p1 = x[2 * i + 1] == -INFINITY ? 0.f : expf(x[2 * i + 1] - mn) * kProbScale;
+    den += p0 + p1;
+    const uint16_t u = f2h(p0), w = f2h(p1);
+    ph[i] = (uint32_t)u | ((uint32_t)w << 16);
+    pl[i] = pack_h2(p0 - h2f(u), p1 - h2f(w));
+  }
+  // O^T += V^T P^T: a lane's 32-bit word u of the four entries' rows
+  // holds dims 2 u and 2 u + 1 of its 8: rows gid and gid + 8 of a tile
+#pragma unroll
+  for (int i = 0; i < 2 * DPL; ++i) {
+    const int j = i >> 2, u = i & 3;
+    auto word = [&](const uint4& v) { return u == 0 ? v.x : u == 1 ? v.y : u == 2 ? v.z : v.w; };
+    const uint32_t r0 = word(vf[0][j]), r1 = word(vf[1][j]), r2 = word(vf[2][j]), r3 = word(vf[3][j]);
+    const uint32_t f0 = prmt_u32(r0, r1, 0x5410u), f1 = prmt_u32(r0, r1, 0x7632u);
+    const uint32_t f2 = prmt_u32(r2, r3, 0x5410u), f3 = prmt_u32(r2, r3, 0x7632u);
+    mma_16816(o[i], f0, f1, f2, f3, ph[0], ph[1]);
+    mma_16816(o[i], f0, f1, f2, f3, pl[0], pl[1]);
+  }
+}
+
+// Query 2 tig + e of a tile's value sums, as a lane holds them: 8 values of each 64 from 8 gid on.
+template <int DPL>
+__device__ __forceinline__ void attn_store_o(float* row, const float (&o)[2 * DPL][4], int e, int gid) {
+#pragma unroll
+  for (int j = 0; j < DPL / 2; ++j) {
+    *reinterpret_cast<float4*>(row + 8 * gid + 64 * j) =
+        make_float4(o[4 * j][e], o[4 * j][2 + e], o[4 * j + 1][e], o[4 * j + 1][2 + e]);
+    *reinterpret_cast<float4*>(row + 8 * gid + 64 * j + 4) =
+        make_float4(o[4 * j + 2][e], o[4 * j + 2][2 + e], o[4 * j + 3][e], o[4 * j + 3][2 + e]);
+  }
+}
+
+// Entries j0 .. j0 + nw of the unit's row: their pool rows and visibility (bit t:
+// token t sees the entry); entries that fill up the last block repeat the last one
+// and are seen by nobody.
+__device__ __forceinline__ void attn_stage(const AttnView& a, const AttnUnit& n, int j0, int nw, uint32_t* rows_s,
+                                           uint16_t* vis_s, int tid) {
+  const int P = n.P, nb = n.nb, hk = n.hk, row = n.row;
+  for (int e = tid; e < (nw + 15) / 16 * 16; e += kThreads) {
+    const int j = j0 + min(e, nw - 1);
+    const int slot = __ldcg(a.bt + (size_t)row * a.cap + j);
+    uint32_t bits = 0;
+    if (e < nw) {
+      if (a.packed) {  // a mask row per token, and no causal bound of its own
+        const uint8_t* mp = a.mask + (size_t)n.tok0 * a.mask_stride + j;
+#pragma unroll 4
+        for (int t = 0; t < nb; ++t) bits |= (__ldcg(mp + (size_t)t * a.mask_stride) != 0 ? 1u : 0u) << t;
+      } else if (__ldcg(a.mask + (size_t)row * a.mask_stride + j) != 0) {
+        bits = 0xFFFFu << max(j - P, 0);  // token t sees entries up to P + t
+      }
+    }
+    const uint32_t pr = (uint32_t)slot / (uint32_t)a.cap;
+    rows_s[e] = (pr * a.Hkv + hk) * (uint32_t)a.cap + ((uint32_t)slot - pr * (uint32_t)a.cap);
+    vis_s[e] = (uint16_t)bits;
+  }
+}
+
+// Of entries j0 .. j0 + nj, the ones this step appends (they lie in the row's last
+// chunks): k rotated by its token's position, both rounded to fp16.
+template <int DPL>
+__device__ __forceinline__ void attn_append(const AttnView& a, const AttnUnit& n, const StepParams* sp, int j0, int nj,
+                                            uint16_t* kpool, uint16_t* vpool, int tid) {
+  constexpr int d = 32 * DPL, half = d / 2;
+  const int P = n.P, hk = n.hk, tok0 = n.tok0;
+  const int r0 = max(P - j0, 0), nnew = nj - r0;
+  if (nnew <= 0) return;
+  const int k_first = a.Hq * d, v_first = (a.Hq + a.Hkv) * d;
+  for (int e = tid; e < nnew * d; e += kThreads) {
+    const int r = e / d, i = e - r * d;
+    const int m = tok0 + (j0 + r0 + r - P);
+    const long long* row = a.acc + (size_t)m * a.acc_ld;
+    const int sl = sp->tok_slot[m];
+    const size_t at = (((size_t)(sl / a.cap) * a.Hkv + hk) * a.cap + sl % a.cap) * d;
+    if (i < half) {
+      const int R = rot_row(k_first, hk, i, d);
+      const float lo = fixed_to_f32(__ldcg(row + R)), hi = fixed_to_f32(__ldcg(row + R + 8));
+      const float2 cs = a.rope[(size_t)sp->tok_pos[m] * half + i];
+      kpool[at + i] = f2h(lo * cs.x - hi * cs.y);
+      kpool[at + half + i] = f2h(hi * cs.x + lo * cs.y);
+    } else {
+      const int i2 = 2 * (i - half);
+      const long long* vr = row + v_first + hk * d + i2;
+      *reinterpret_cast<uint32_t*>(vpool + at + i2) = pack_h2(fixed_to_f32(__ldcg(vr)), fixed_to_f32(__ldcg(vr + 1)));
+    }
+  }
+}
+
+// One chunk by the CTA's consumer warps: its partials, or the outputs of a row of
+// one chunk.
+template <int DPL>
+__device__ __forceinline__ void attn_chunk(const AttnView& a, const AttnUnit& n, int c, int layer, const StepParams* sp,
+                                           uint8_t* area, int* status) {
+  using S = AttnSmem<DPL>;
+  constexpr int d = S::d;
   uint16_t* kpool = a.kpool + (size_t)layer * a.layer_stride;
   uint16_t* vpool = a.vpool + (size_t)layer * a.layer_stride;
   uint16_t* qhi = reinterpret_cast<uint16_t*>(area);
@@ -661,55 +943,15 @@ __device__ __forceinline__ void attn_item_cta(const AttnView* ap, int layer, con
   float* pieces = reinterpret_cast<float*>(area);
   float2* ml_s = reinterpret_cast<float2*>(area + S::kPieces);
   const int tid = opaque(threadIdx.x), warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
-  const int L = sp->req_len[b], P = sp->req_P[b];
-  const int tok0 = sp->req_tok0[b], nb = sp->req_tok0[b + 1] - tok0;
-  const int G = a.Hq / a.Hkv, Q = nb * G;
-  const int j0 = c * a.cs, nj = min(a.cs, L - j0), nc = n_chunks_of(L, a.cs);
+  const int hk = n.hk, tok0 = n.tok0, P = n.P, Q = n.Q, nc = n.nc;
+  const int G = a.Hq / a.Hkv;
+  const int j0 = c * n.cs, nj = min(n.cs, n.end - j0);
 
-  uint4 kf[2][KJ], vf[4][VJ];
+  uint4 kf[2][DPL], vf[4][DPL / 2];
 #pragma unroll
-  for (int j = 0; j < KJ; ++j) kf[0][j] = kf[1][j] = make_uint4(0, 0, 0, 0);
+  for (int j = 0; j < DPL; ++j) kf[0][j] = kf[1][j] = make_uint4(0, 0, 0, 0);
 #pragma unroll
-  for (int j = 0; j < VJ; ++j) vf[0][j] = vf[1][j] = vf[2][j] = vf[3][j] = make_uint4(0, 0, 0, 0);
-  // K rows: entries gid and gid + 8 of the block; V rows: entries 2 tig, + 1, + 8, + 9
-  auto load_k = [&](int blk) {
-#pragma unroll
-    for (int n = 0; n < 2; ++n) {
-      const uint4* p = reinterpret_cast<const uint4*>(kpool + (size_t)rows_s[16 * blk + 8 * n + gid] * d) + tig;
-#pragma unroll
-      for (int j = 0; j < KJ; ++j) kf[n][j] = p[4 * j];
-    }
-  };
-  auto load_v = [&](int blk) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const uint4* p =
-          reinterpret_cast<const uint4*>(vpool + (size_t)rows_s[16 * blk + 8 * (r >> 1) + 2 * tig + (r & 1)] * d) + gid;
-#pragma unroll
-      for (int j = 0; j < VJ; ++j) vf[r][j] = p[8 * j];
-    }
-  };
-  // the window's pool rows and visibility; entries that fill up the last
-  // block repeat the window's last one and are seen by nobody
-  auto stage = [&](int w0, int nw) {
-    for (int e = tid; e < (nw + 15) / 16 * 16; e += kThreads) {
-      const int j = j0 + w0 + min(e, nw - 1);
-      const int slot = __ldcg(a.bt + (size_t)b * a.cap + j);
-      uint32_t bits = 0;
-      if (e < nw) {
-        if (a.packed) {  // a mask row per token, and no causal bound of its own
-          const uint8_t* mp = a.mask + (size_t)tok0 * a.mask_stride + j;
-#pragma unroll 4
-          for (int t = 0; t < nb; ++t) bits |= (__ldcg(mp + (size_t)t * a.mask_stride) != 0 ? 1u : 0u) << t;
-        } else if (__ldcg(a.mask + (size_t)b * a.mask_stride + j) != 0) {
-          bits = 0xFFFFu << max(j - P, 0);  // token t sees entries up to P + t
-        }
-      }
-      const uint32_t pr = (uint32_t)slot / (uint32_t)a.cap;
-      rows_s[e] = (pr * a.Hkv + hk) * (uint32_t)a.cap + ((uint32_t)slot - pr * (uint32_t)a.cap);
-      vis_s[e] = (uint16_t)bits;
-    }
-  };
+  for (int j = 0; j < DPL / 2; ++j) vf[0][j] = vf[1][j] = vf[2][j] = vf[3][j] = make_uint4(0, 0, 0, 0);
 
   for (int q0 = 0; q0 < Q; q0 += kAttnQ) {
     const int qn = min(kAttnQ, Q - q0), nqt = (qn + 7) >> 3;
@@ -717,130 +959,45 @@ __device__ __forceinline__ void attn_item_cta(const AttnView* ap, int layer, con
     const int qt = warp / eg, g = warp - qt * eg;
     const bool active = qt < nqt;
     const int tk = (q0 + min(8 * qt + gid, qn - 1)) / G;  // the token of query gid
-    float o[4 * VJ][4], mx = -INFINITY, den = 0.f, qs = 0.f;
+    float o[2 * DPL][4], mx = -INFINITY, den = 0.f, qs = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4 * VJ; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+    for (int i = 0; i < 2 * DPL; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
     for (int w0 = 0; w0 < nj; w0 += kAttnWin) {
       const int nw = min(kAttnWin, nj - w0), nblk = (nw + 15) >> 4;
       const bool first = q0 == 0 && w0 == 0;
       bool have = false;
       if (w0 > 0) cbar();  // the previous window's entries are done
-      if (first || nj > kAttnWin || q0 > 0) stage(w0, nw);  // (the pieces overwrote it between passes)
+      if (first || nj > kAttnWin || q0 > 0)
+        attn_stage(a, n, j0 + w0, nw, rows_s, vis_s, tid);  // (the pieces overwrote it between passes)
       if (first) {
         cbar();
         // a block of entries from earlier steps loads during the wait for q|k|v
         have = active && g < nblk && j0 + 16 * g + 16 <= P;
         if (have) {
-          load_k(g);
-          load_v(g);
+          attn_load_k<DPL>(kf, kpool, rows_s, g, gid, tig);
+          attn_load_v<DPL>(vf, vpool, rows_s, g, gid, tig);
         }
         if (tid == 0) wait_count(a.cnt_kv + hk, a.kv_units, status, a.limit);
         cbar();
-        // the entries this step appends (they lie in the request's last
-        // chunks): k rotated by its token's position, both rounded to fp16
-        const int r0 = max(P - j0, 0), nnew = nj - r0;
-        if (nnew > 0) {
-          const int k_first = a.Hq * d, v_first = (a.Hq + a.Hkv) * d;
-          for (int e = tid; e < nnew * d; e += kThreads) {
-            const int r = e / d, i = e - r * d;
-            const int m = tok0 + (j0 + r0 + r - P);
-            const long long* row = a.acc + (size_t)m * a.acc_ld;
-            const int sl = sp->tok_slot[m];
-            const size_t at = (((size_t)(sl / a.cap) * a.Hkv + hk) * a.cap + sl % a.cap) * d;
-            if (i < half) {
-              const int R = rot_row(k_first, hk, i, d);
-              const float lo = fixed_to_f32(__ldcg(row + R)), hi = fixed_to_f32(__ldcg(row + R + 8));
-              const float2 cs = a.rope[(size_t)sp->tok_pos[m] * half + i];
-              kpool[at + i] = f2h(lo * cs.x - hi * cs.y);
-              kpool[at + half + i] = f2h(hi * cs.x + lo * cs.y);
-            } else {
-              const int i2 = 2 * (i - half);
-              const long long* vr = row + v_first + hk * d + i2;
-              *reinterpret_cast<uint32_t*>(vpool + at + i2) =
-                  pack_h2(fixed_to_f32(__ldcg(vr)), fixed_to_f32(__ldcg(vr + 1)));
-            }
-          }
-        }
+        attn_append<DPL>(a, n, sp, j0, nj, kpool, vpool, tid);
       }
       if (w0 == 0) attn_load_queries<DPL>(a, sp, hk, tok0, q0, qn, qhi, qlo, qscale);
       cbar();
       if (!active) continue;
       if (w0 == 0) qs = qscale[min(8 * qt + gid, qn - 1)];
       if (!have && g < nblk) {
-        load_k(g);
-        load_v(g);
+        attn_load_k<DPL>(kf, kpool, rows_s, g, gid, tig);
+        attn_load_v<DPL>(vf, vpool, rows_s, g, gid, tig);
       }
       const uint16_t* qh = qhi + (8 * qt + gid) * S::kQld + 8 * tig;
       const uint16_t* ql = qlo + (8 * qt + gid) * S::kQld + 8 * tig;
       for (int blk = g; blk < nblk; blk += eg) {
         const bool more = blk + eg < nblk;
-        const uint32_t va = *reinterpret_cast<const uint32_t*>(vis_s + 16 * blk + 2 * tig) >> tk;
-        const uint32_t vb = *reinterpret_cast<const uint32_t*>(vis_s + 16 * blk + 8 + 2 * tig) >> tk;
-        float s[2][2][4];  // two chains per 8 entries
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) s[n][e][0] = s[n][e][1] = s[n][e][2] = s[n][e][3] = 0.f;
-#pragma unroll
-        for (int j = 0; j < KJ; ++j) {
-          const uint4 h = *reinterpret_cast<const uint4*>(qh + 32 * j);
-          const uint4 l = *reinterpret_cast<const uint4*>(ql + 32 * j);
-#pragma unroll
-          for (int n = 0; n < 2; ++n) {
-            mma_16816(s[n][0], h.x, l.x, h.y, l.y, kf[n][j].x, kf[n][j].y);
-            mma_16816(s[n][1], h.z, l.z, h.w, l.w, kf[n][j].z, kf[n][j].w);
-          }
-        }
-        if (more) load_k(blk + eg);
-        // scores of query gid and entries 2 tig, + 1, + 8, + 9
         float x[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float (&u)[2][4] = s[i >> 1];
-          const int e = i & 1;
-          const bool see = ((i < 2 ? va : vb) >> (16 * e)) & 1u;
-          x[i] = see ? ((u[0][e] + u[1][e]) + (u[0][2 + e] + u[1][2 + e])) * qs : -INFINITY;
-        }
-        float mn = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
-        mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
-        mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
-        mn = fmaxf(mn, mx);
-        if (__any_sync(0xffffffffu, mn > mx)) {
-          const float alpha = mx == -INFINITY ? 0.f : expf(mx - mn);
-          den *= alpha;
-          const float a0 = __shfl_sync(0xffffffffu, alpha, 8 * tig), a1 = __shfl_sync(0xffffffffu, alpha, 8 * tig + 4);
-#pragma unroll
-          for (int i = 0; i < 4 * VJ; ++i) {
-            o[i][0] *= a0;
-            o[i][1] *= a1;
-            o[i][2] *= a0;
-            o[i][3] *= a1;
-          }
-          mx = mn;
-        }
-        uint32_t ph[2], pl[2];  // the probabilities as the value sum's B fragments
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const float p0 = x[2 * i] == -INFINITY ? 0.f : expf(x[2 * i] - mn) * kProbScale;
-          const float p1 = x[2 * i + 1] == -INFINITY ? 0.f : expf(x[2 * i + 1] - mn) * kProbScale;
-          den += p0 + p1;
-          const uint16_t u = f2h(p0), w = f2h(p1);
-          ph[i] = (uint32_t)u | ((uint32_t)w << 16);
-          pl[i] = pack_h2(p0 - h2f(u), p1 - h2f(w));
-        }
-        // O^T += V^T P^T: a lane's 32-bit word u of the four entries' rows
-        // holds dims 2 u and 2 u + 1 of its 8: rows gid and gid + 8 of a tile
-#pragma unroll
-        for (int i = 0; i < 4 * VJ; ++i) {
-          const int j = i >> 2, u = i & 3;
-          auto word = [&](const uint4& v) { return u == 0 ? v.x : u == 1 ? v.y : u == 2 ? v.z : v.w; };
-          const uint32_t r0 = word(vf[0][j]), r1 = word(vf[1][j]), r2 = word(vf[2][j]), r3 = word(vf[3][j]);
-          const uint32_t f0 = prmt_u32(r0, r1, 0x5410u), f1 = prmt_u32(r0, r1, 0x7632u);
-          const uint32_t f2 = prmt_u32(r2, r3, 0x5410u), f3 = prmt_u32(r2, r3, 0x7632u);
-          mma_16816(o[i], f0, f1, f2, f3, ph[0], ph[1]);
-          mma_16816(o[i], f0, f1, f2, f3, pl[0], pl[1]);
-        }
-        if (more) load_v(blk + eg);
+        attn_scores<DPL>(x, kf, qh, ql, vis_s + 16 * blk, tk, qs, tig);
+        if (more) attn_load_k<DPL>(kf, kpool, rows_s, blk + eg, gid, tig);
+        attn_values<DPL>(x, vf, o, mx, den, tig);
+        if (more) attn_load_v<DPL>(vf, vpool, rows_s, blk + eg, gid, tig);
       }
     }
     // the CTA's pieces through shared memory
@@ -851,16 +1008,7 @@ __device__ __forceinline__ void attn_item_cta(const AttnView* ap, int layer, con
       den += __shfl_xor_sync(0xffffffffu, den, 2);
       if (tig == 0) ml_s[warp * 8 + gid] = make_float2(mx, den);
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {  // query 2 tig + e
-        float* w = pieces + (size_t)(warp * 8 + 2 * tig + e) * S::kOld + 8 * gid;
-#pragma unroll
-        for (int j = 0; j < VJ; ++j) {
-          *reinterpret_cast<float4*>(w + 64 * j) =
-              make_float4(o[4 * j][e], o[4 * j][2 + e], o[4 * j + 1][e], o[4 * j + 1][2 + e]);
-          *reinterpret_cast<float4*>(w + 64 * j + 4) =
-              make_float4(o[4 * j + 2][e], o[4 * j + 2][2 + e], o[4 * j + 3][e], o[4 * j + 3][2 + e]);
-        }
-      }
+      for (int e = 0; e < 2; ++e) attn_store_o<DPL>(pieces + (size_t)(warp * 8 + 2 * tig + e) * S::kOld, o, e, gid);
     }
     cbar();
     for (int i = tid; i < qn * (d / 4); i += kThreads) {
@@ -885,42 +1033,153 @@ __device__ __forceinline__ void attn_item_cta(const AttnView* ap, int layer, con
         h.y = pack_h2(num.z / D, num.w / D);
         *reinterpret_cast<uint2*>(a.out + (size_t)(tok0 + q / G) * a.out_ld + (hk * G + q % G) * d + 4 * f) = h;
       } else {
-        float* p = a.part + ((size_t)item * a.qmax + q) * part_stride(d);
+        float* p = a.part + (size_t)(n.part0 + c * Q + q) * part_stride(d);
         if (f == 0) *reinterpret_cast<float2*>(p) = make_float2(M, D);
         *reinterpret_cast<float4*>(p + 4 + 4 * f) = num;
       }
     }
     cbar();  // the partials are written, and the area is free
   }
-  if (nc == 1) return;
-  // chunks of (b, hk) are items item - c .. item - c + nc - 1
-  int* cnt = &a.cnt[b * a.Hkv + hk];
+}
+
+// The unit's chunks, each query tile of a chunk by one warp, with the arithmetic and
+// the order of attn_chunk: first all blocks' scores, kept in shared memory, and their
+// largest; then the values of one piece after the other (piece g: blocks g, g + eg, ..,
+// what warp g of attn_chunk adds), each scaled and added as the pieces meet there.
+// No barrier between chunks: eight rows of 640..1642 entries at 8B width take 30.5 us
+// a layer (norm, q|k|v and attention), chunk by chunk 79.
+template <int DPL>
+__device__ __forceinline__ void attn_run(const AttnView& a, const AttnUnit& n, int layer, const StepParams* sp,
+                                         uint8_t* area, int* status) {
+  using S = AttnSmem<DPL>;
+  constexpr int d = S::d;
+  uint16_t* kpool = a.kpool + (size_t)layer * a.layer_stride;
+  uint16_t* vpool = a.vpool + (size_t)layer * a.layer_stride;
+  const int tid = opaque(threadIdx.x), warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
+  const int hk = n.hk, tok0 = n.tok0, P = n.P, Q = n.Q, cs = n.cs, c0 = n.c0, c1 = n.c1, end = n.end;
+  const int G = a.Hq / a.Hkv, nqt = (Q + 7) >> 3, eg = kWarps / nqt;
+  uint16_t* qhi = reinterpret_cast<uint16_t*>(area);
+  uint16_t* qlo = reinterpret_cast<uint16_t*>(area + n.qlo);
+  uint32_t* rows_s = reinterpret_cast<uint32_t*>(area + n.rows);
+  uint16_t* vis_s = reinterpret_cast<uint16_t*>(rows_s + kAttnWin);
+  float* qscale = reinterpret_cast<float*>(vis_s + kAttnWin);
+  float4* xs = reinterpret_cast<float4*>(qscale + kAttnQ) + warp * (cs >> 4) * 32 + lane;  // [block][lane]
+  uint4 kf[2][DPL], vf[4][DPL / 2];
+#pragma unroll
+  for (int j = 0; j < DPL; ++j) kf[0][j] = kf[1][j] = make_uint4(0, 0, 0, 0);
+#pragma unroll
+  for (int j = 0; j < DPL / 2; ++j) vf[0][j] = vf[1][j] = vf[2][j] = vf[3][j] = make_uint4(0, 0, 0, 0);
+  const int staged = kAttnWin / cs;  // chunks whose entries are staged together
+  for (int ca = c0; ca < c1; ca += staged) {
+    const int j0 = ca * cs, nj = min(min(ca + staged, c1) * cs, end) - j0;
+    const int items = (min(ca + staged, c1) - ca) * nqt;  // (chunk, query tile), tiles of a chunk side by side
+    bool have = false;
+    if (ca > c0) cbar();  // the entries before are done
+    attn_stage(a, n, j0, nj, rows_s, vis_s, tid);
+    if (ca == c0) {
+      cbar();
+      // a first block of entries from earlier steps loads during the wait for q|k|v
+      have = warp < min(items, n.warps) && (c0 + warp / nqt) * cs + 16 <= P;
+      if (have) attn_load_k<DPL>(kf, kpool, rows_s, warp / nqt * (cs >> 4), gid, tig);
+      if (tid == 0) wait_count(a.cnt_kv + hk, a.kv_units, status, a.limit);
+      cbar();
+      attn_append<DPL>(a, n, sp, c0 * cs, min(c1 * cs, end) - c0 * cs, kpool, vpool, tid);
+      attn_load_queries<DPL>(a, sp, hk, tok0, 0, Q, qhi, qlo, qscale);
+    }
+    cbar();
+    for (int it = warp; it < items && warp < n.warps; it += n.warps) {
+      const int ci = it / nqt, qt = it - ci * nqt, b0 = ci * (cs >> 4);
+      const int nblk = (min(cs, end - (ca + ci) * cs) + 15) >> 4;
+      const int q = 8 * qt + gid, tk = min(q, Q - 1) / G;
+      const float qs = qscale[min(q, Q - 1)];
+      const uint16_t* qh = qhi + q * S::kQld + 8 * tig;
+      const uint16_t* ql = qlo + q * S::kQld + 8 * tig;
+      if (!have) attn_load_k<DPL>(kf, kpool, rows_s, b0, gid, tig);
+      have = false;
+      float M = -INFINITY, x[4];
+      for (int i = 0; i < nblk; ++i) {
+        attn_scores<DPL>(x, kf, qh, ql, vis_s + 16 * (b0 + i), tk, qs, tig);
+        if (i + 1 < nblk)
+          attn_load_k<DPL>(kf, kpool, rows_s, b0 + i + 1, gid, tig);
+        else
+          attn_load_v<DPL>(vf, vpool, rows_s, b0, gid, tig);
+        xs[32 * i] = make_float4(x[0], x[1], x[2], x[3]);
+        M = fmaxf(M, attn_block_max(x));
+      }
+      float num[2 * DPL][4], D = 0.f;
+#pragma unroll
+      for (int i = 0; i < 2 * DPL; ++i) num[i][0] = num[i][1] = num[i][2] = num[i][3] = 0.f;
+      const int ngr = min(eg, nblk);
+      for (int g = 0; g < ngr; ++g) {
+        float o[2 * DPL][4], mx = -INFINITY, den = 0.f;
+#pragma unroll
+        for (int i = 0; i < 2 * DPL; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+        for (int blk = g; blk < nblk; blk += eg) {
+          const float4 xv = xs[32 * blk];
+          const float y[4] = {xv.x, xv.y, xv.z, xv.w};
+          attn_values<DPL>(y, vf, o, mx, den, tig);
+          const int next = blk + eg < nblk ? blk + eg : g + 1;
+          if (blk + eg < nblk || g + 1 < ngr) attn_load_v<DPL>(vf, vpool, rows_s, b0 + next, gid, tig);
+        }
+        den += __shfl_xor_sync(0xffffffffu, den, 1);
+        den += __shfl_xor_sync(0xffffffffu, den, 2);
+        const float k = mx == -INFINITY ? 0.f : expf(mx - M);
+        D = fmaf(den, k, D);
+        const float k0 = __shfl_sync(0xffffffffu, k, 8 * tig), k1 = __shfl_sync(0xffffffffu, k, 8 * tig + 4);
+#pragma unroll
+        for (int i = 0; i < 2 * DPL; ++i) {
+          num[i][0] = fmaf(o[i][0], k0, num[i][0]);
+          num[i][1] = fmaf(o[i][1], k1, num[i][1]);
+          num[i][2] = fmaf(o[i][2], k0, num[i][2]);
+          num[i][3] = fmaf(o[i][3], k1, num[i][3]);
+        }
+      }
+      float* p = a.part + (size_t)(n.part0 + (ca + ci) * Q) * part_stride(d);
+      if (tig == 0 && q < Q) *reinterpret_cast<float2*>(p + q * part_stride(d)) = make_float2(M, D);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int qe = 8 * qt + 2 * tig + e;
+        if (qe < Q) attn_store_o<DPL>(p + qe * part_stride(d) + 4, num, e, gid);
+      }
+    }
+  }
+  cbar();  // the partials are written, and the area is free
+}
+
+// The row's outputs once all its chunks' partials are there.
+template <int DPL>
+__device__ __forceinline__ void attn_merge(const AttnView& a, const AttnUnit& n, int* status) {
+  constexpr int d = 32 * DPL;
+  const int tid = opaque(threadIdx.x), warp = tid >> 5, lane = tid & 31;
+  const int Q = n.Q, G = a.Hq / a.Hkv;
   __shared__ int s_last;
-  const bool alone = Q * nc <= kMergeAlone;
+  const bool alone = Q * n.nc <= kMergeAlone;
   if (tid == 0) {
+    const int mine = n.c1 - n.c0;
     if (alone) {
-      s_last = atom_add_acq_rel(cnt, 1) == nc - 1;
+      s_last = atom_add_acq_rel(n.cnt, mine) == n.nc - mine;
     } else {
-      red_release_add_s32(cnt, 1);
-      wait_count(cnt, nc, status, a.limit);
+      red_release_add_s32(n.cnt, mine);
+      wait_count(n.cnt, n.nc, status, a.limit);
       s_last = 1;
     }
   }
   cbar();
   if (!s_last) return;
-  const float* base = a.part + (size_t)(item - c) * a.qmax * part_stride(d);
-  for (int q = alone ? warp : c + nc * warp; q < Q; q += alone ? kWarps : nc * kWarps)
-    attn_merge_warp<DPL>(base + (size_t)q * part_stride(d), (size_t)a.qmax * part_stride(d), nc,
-                         a.out + (size_t)(tok0 + q / G) * a.out_ld + (hk * G + q % G) * d, lane);
+  const float* base = a.part + (size_t)n.part0 * part_stride(d);
+  for (int q = alone ? warp : n.u + n.units * warp; q < Q; q += alone ? kWarps : n.units * kWarps)
+    attn_merge_warp<DPL>(base + (size_t)q * part_stride(d), (size_t)Q * part_stride(d), n.nc,
+                         a.out + (size_t)(n.tok0 + q / G) * a.out_ld + (n.hk * G + q % G) * d, lane);
 }
 
-template <int NT, int GPU, int DPL>
+template <int NT, int GPU, int DPL, bool kMany>
 __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_constant__ StepKernelArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ GemvPhase s_gp[4];            // per projection kind: q|k|v, o, gate|up, down
   constexpr int kSlots = Geom<GPU>::kStepSlots;
   __shared__ AttnView s_av;
-  __shared__ int2 s_plan;                  // attention items: entries per item, number
+  __shared__ AttnPlan s_plan;              // (kMany)
+  __shared__ AttnUnit s_unit;              // this CTA's attention unit
   __shared__ uint64_t s_nbar;              // the staged RMSNorm's bulk copies
   __shared__ StepParams s_sp;
   __shared__ const uint16_t* s_rowp[kMaxTokens];  // the step's fp16 input rows
@@ -938,7 +1197,17 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
     ring_init_barriers(full, empty, kWarps * kSlots);  // ends with the barrier-init fence
     if (blockIdx.x == 0) a.phase_clock[0] = globaltimer();
   }
-  prologue_params(a.pro, &s_sp, s_rowp);  // ends with a block-wide barrier
+  const auto plan = [&](int l) {
+    if (kMany) {
+      const int total = attn_plan(&s_sp, a.Hq / a.Hkv, a.Hkv, gridDim.x, l, &s_plan);
+      if (l == 0) s_unit.total = total;
+    } else if (l == 0) {
+      attn_one_row(s_sp, a.Hkv, gridDim.x, s_unit);
+    }
+    if (l == 0 && (int)blockIdx.x < s_unit.total)
+      attn_unit_init<DPL, kMany>(s_plan, s_sp, a.Hq / a.Hkv, a.Hkv, a.attn_cnt, a.area_bytes, blockIdx.x, s_unit);
+  };
+  prologue_params(a.pro, &s_sp, s_rowp, plan);  // ends with a block-wide barrier
   const int n_barriers = 4 * a.L + 1;
   if (s_sp.abort_step) {
     // every CTA sees the same inputs and rejects the step alike: count this
@@ -1021,9 +1290,7 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
     av.Hq = a.Hq;
     av.Hkv = a.Hkv;
     av.d = a.d;
-    av.qmax = kMaxTokens * G;
     av.part = a.attn_part;
-    av.cnt = a.attn_cnt;
     av.cnt_kv = a.cnt_kv;
     av.kv_units = (G + 2) * (a.d / kRowsPerBlock) * s_ops[0].upr;
     av.bt = a.pro.bt_dst;
@@ -1034,16 +1301,6 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
     av.out = a.act_attn;
     av.out_ld = a.Kp_dq;
     s_av = av;
-  }
-  if (warp == 2) {
-    int cs, total;
-    attn_plan(sp, a.Hkv, gridDim.x, lane, cs, total);
-    if (lane == 0) s_plan = make_int2(cs, total);
-  }
-  cbar();
-  if (threadIdx.x == 32) {
-    s_av.cs = s_plan.x;
-    s_av.total = s_plan.y;
   }
   prologue_work(a.pro, sp, s_rowp, a.X);
   cbar();
@@ -1108,9 +1365,22 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
       if (lane == 0) s_ring[warp] = ring;
       __syncwarp();
       if (l == 0) gb.wait();        // the prologue's tables and residual are complete
-      else if (xn_smem) cbar();     // the attention items reuse the normalised rows' space
-      for (int item = blockIdx.x; item < s_av.total; item += gridDim.x)
-        attn_item_cta<DPL>(&s_av, l, sp, item, att_area, a.status);
+      else if (xn_smem) cbar();     // the attention reuses the normalised rows' space
+      const int total = s_unit.total;
+      for (int unit = blockIdx.x; unit < total; unit += gridDim.x) {
+        if (total > (int)gridDim.x && (l > 0 || unit != (int)blockIdx.x)) {  // several units per CTA
+          cbar();
+          if (threadIdx.x == 0)
+            attn_unit_init<DPL, kMany>(s_plan, s_sp, a.Hq / a.Hkv, a.Hkv, a.attn_cnt, a.area_bytes, unit, s_unit);
+          cbar();
+        }
+        if (kMany && s_unit.warps > 0)
+          attn_run<DPL>(s_av, s_unit, l, sp, att_area, a.status);
+        else
+          for (int c = s_unit.c0; c < (kMany ? s_unit.c1 : s_unit.c0 + 1); ++c)
+            attn_chunk<DPL>(s_av, s_unit, c, l, sp, att_area, a.status);
+        if (s_unit.nc > 1) attn_merge<DPL>(s_av, s_unit, a.status);
+      }
       __syncwarp();
       asm volatile("" ::: "memory");
       ring = s_ring[warp];
@@ -1135,9 +1405,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   }
 }
 
-template <int NT, int GPU, int DPL>
+template <int NT, int GPU, int DPL, bool kMany>
 cudaError_t launch_t(const StepKernelArgs& a, int grid, cudaStream_t s) {
-  auto kern = step_kernel<NT, GPU, DPL>;
+  auto kern = step_kernel<NT, GPU, DPL, kMany>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kBlockThreads);
@@ -1151,43 +1421,36 @@ cudaError_t launch_t(const StepKernelArgs& a, int grid, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-template <int NT, int GPU, int DPL>
+template <int NT, int GPU, int DPL, bool kMany>
 size_t dyn_limit_t() {
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
   cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, step_kernel<NT, GPU, DPL>) != cudaSuccess) return 0;
+  if (cudaFuncGetAttributes(&fa, step_kernel<NT, GPU, DPL, kMany>) != cudaSuccess) return 0;
   return (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
 }
 
 // The largest dynamic shared memory the kernel may take.
-template <int NT, int GPU, int DPL>
+template <int NT, int GPU, int DPL, bool kMany>
 cudaError_t setup_t() {
-  return cudaFuncSetAttribute(step_kernel<NT, GPU, DPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)dyn_limit_t<NT, GPU, DPL>());
+  return cudaFuncSetAttribute(step_kernel<NT, GPU, DPL, kMany>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)dyn_limit_t<NT, GPU, DPL, kMany>());
 }
 
-// Dynamic shared memory every kernel of a group size may take (0: unknown group).
-template <int GPU>
-size_t dyn_limit_group() {
-  size_t m = dyn_limit_t<1, GPU, 4>();
-  m = std::min(m, dyn_limit_t<2, GPU, 4>());
-  m = std::min(m, dyn_limit_t<1, GPU, 2>());
-  return std::min(m, dyn_limit_t<2, GPU, 2>());
-}
-
-template <int GPU>
-bool part_fits(int L) {
-  return StepSmem<GPU>::area(L, true, kMaxTokens) + kAttnArea <= dyn_limit_group<GPU>();
+// Dynamic shared memory every kernel of a group size and head dim may take.
+template <int GPU, int DPL>
+size_t dyn_limit() {
+  return std::min(std::min(dyn_limit_t<1, GPU, DPL, false>(), dyn_limit_t<1, GPU, DPL, true>()),
+                  std::min(dyn_limit_t<2, GPU, DPL, false>(), dyn_limit_t<2, GPU, DPL, true>()));
 }
 
 // Bytes of the shared-memory area for steps of M tokens: room for the
 // normalised rows where the kernel's limit allows it.
 template <int GPU>
-size_t area_bytes_t(int H, int L, bool part, int M) {
+size_t area_bytes_t(int H, int L, bool part, int M, size_t limit) {
   const size_t want = xn_bytes(H, M) + xn_stage_bytes(H, M);
-  if (want <= kAttnArea || StepSmem<GPU>::area(L, part, M) + want > dyn_limit_group<GPU>()) return kAttnArea;
+  if (want <= kAttnArea || StepSmem<GPU>::area(L, part, M) + want > limit) return kAttnArea;
   return want;
 }
 
@@ -1195,21 +1458,26 @@ size_t area_bytes_t(int H, int L, bool part, int M) {
 
 int step_barriers(int n_layers) { return 4 * n_layers + 1; }
 
-bool step_gu_part_fits(int group, int L) {
-  if (group == 128) return part_fits<1>(L);
-  if (group == 64) return part_fits<2>(L);
-  if (group == 32) return part_fits<4>(L);
-  return false;
+size_t step_dyn_limit(int group, int head_dim) {
+  if (head_dim == 128) return group == 128 ? dyn_limit<1, 4>() : group == 64 ? dyn_limit<2, 4>() : dyn_limit<4, 4>();
+  return group == 128 ? dyn_limit<1, 2>() : group == 64 ? dyn_limit<2, 2>() : dyn_limit<4, 2>();
 }
 
-size_t step_area_bytes(int group, int H, int L, bool part, int M) {
-  if (group == 128) return area_bytes_t<1>(H, L, part, M);
-  if (group == 64) return area_bytes_t<2>(H, L, part, M);
-  return area_bytes_t<4>(H, L, part, M);
+bool step_gu_part_fits(int group, int L, size_t limit) {
+  const size_t area = group == 128  ? StepSmem<1>::area(L, true, kMaxTokens)
+                      : group == 64 ? StepSmem<2>::area(L, true, kMaxTokens)
+                                    : StepSmem<4>::area(L, true, kMaxTokens);
+  return area + kAttnArea <= limit;
 }
 
-int step_gu_split(int n_rb, int upr, int grid, int group, int L) {
-  if (n_rb < 1 || upr < 1 || grid < 1 || !step_gu_part_fits(group, L)) return 0;
+size_t step_area_bytes(int group, int H, int L, bool part, int M, size_t limit) {
+  if (group == 128) return area_bytes_t<1>(H, L, part, M, limit);
+  if (group == 64) return area_bytes_t<2>(H, L, part, M, limit);
+  return area_bytes_t<4>(H, L, part, M, limit);
+}
+
+int step_gu_split(int n_rb, int upr, int grid) {
+  if (n_rb < 1 || upr < 1 || grid < 1) return 0;
   const long long nw = (long long)grid * kWarps;
   const long long even = ((long long)n_rb * upr + nw - 1) / nw;  // most units per warp, grid-wide split
   int best = 0;
@@ -1227,9 +1495,11 @@ size_t step_attention_part_floats(int grid, int G, int d) {
 
 cudaError_t step_setup(int group, int head_dim) {
   cudaError_t e = cudaSuccess;
-#define SETUP_PAIR(GPU, DPL)                                       \
-  if ((e = setup_t<1, GPU, DPL>()) != cudaSuccess) return e;       \
-  if ((e = setup_t<2, GPU, DPL>()) != cudaSuccess) return e;
+#define SETUP_PAIR(GPU, DPL)                                              \
+  if ((e = setup_t<1, GPU, DPL, false>()) != cudaSuccess) return e;       \
+  if ((e = setup_t<1, GPU, DPL, true>()) != cudaSuccess) return e;        \
+  if ((e = setup_t<2, GPU, DPL, false>()) != cudaSuccess) return e;       \
+  if ((e = setup_t<2, GPU, DPL, true>()) != cudaSuccess) return e;
   if (head_dim == 128) {
     if (group == 128) { SETUP_PAIR(1, 4) }
     else if (group == 64) { SETUP_PAIR(2, 4) }
@@ -1247,7 +1517,10 @@ cudaError_t step_setup(int group, int head_dim) {
 
 cudaError_t launch_step(const StepKernelArgs& a, int nt, int group, int grid, cudaStream_t s) {
   const int dpl = a.d / 32;
-#define LAUNCH(GPU, DPL) return nt == 1 ? launch_t<1, GPU, DPL>(a, grid, s) : launch_t<2, GPU, DPL>(a, grid, s);
+  const bool many = a.pro.B > 1;
+#define LAUNCH(GPU, DPL)                                                                              \
+  return nt == 1 ? (many ? launch_t<1, GPU, DPL, true>(a, grid, s) : launch_t<1, GPU, DPL, false>(a, grid, s)) \
+                 : (many ? launch_t<2, GPU, DPL, true>(a, grid, s) : launch_t<2, GPU, DPL, false>(a, grid, s));
   if (dpl == 4) {
     if (group == 128) LAUNCH(1, 4)
     if (group == 64) LAUNCH(2, 4)
