@@ -807,7 +807,9 @@ __device__ __forceinline__ void attn_scores(float (&x)[4], const uint4 (&kf)[2][
     const float (&u)[2][4] = s[i >> 1];
     const int e = i & 1;
     const bool see = ((i < 2 ? va : vb) >> (16 * e)) & 1u;
-    x[i] = see ? ((u[0][e] + u[1][e]) + (u[0][2 + e] + u[1][2 + e])) * qs : -INFINITY;
+    const float hi = u[0][e] + u[1][e], lo = u[0][2 + e] + u[1][2 + e];
+    // (an infinite key: the remainders' product has a sign of its own, or none)
+    x[i] = see ? (fabsf(hi) < INFINITY ? hi + lo : hi) * qs : -INFINITY;
   }
 }
 

@@ -88,3 +88,33 @@ def test_attention_query_scales(scale):
     q = w.layers[0].matrices[0]
     q.scales[:] = (q.scales.view(np.float16).astype(np.float32) * scale).astype(np.float16).view(np.uint16)
     _run("five-tiles", lambda b, l: np.ones(l), w, shape)
+
+
+@pytest.mark.parametrize("n_new", [1, 3])
+def test_a_key_at_minus_infinity_against_its_queries_has_no_weight(n_new):
+    """A cached key that overflowed to an infinity, of the sign that gives its head's queries a score of minus
+    infinity: the entry has weight 0, as in the oracle, and the outputs stay finite."""
+    shape = synth.ShardShape("inf", 1, 256, 4, 4, 64, 320, 64, 0.06, 0, 1e-5, 10000.0, 8192)
+    w = synth.make_weights(shape, 17)
+    L, entry, dim = 80, 21, 5
+    h16 = synth.hidden_in(shape, 8, 0, 1).repeat(n_new, 0)  # one token's queries at one position: one sign per head
+    pos, mask = np.full(n_new, L, np.int32), np.ones((1, L + n_new), np.uint8)
+    k, v = synth.kv_prefill(shape, 5, 0, L, 0)
+
+    def outputs(state):
+        state.load(0, 0, k, v)
+        return state.step([n_new], pos, mask, hidden_in=h16)
+
+    ref = oracle.OracleShard(shape, w)
+    for head in range(4):
+        for inf in (0x7C00, 0xFC00):
+            k[entry, head, dim] = inf
+            rc, want, _ = outputs(ref.state(1, L + n_new))
+            if rc == 0 and np.isfinite(want.view(np.float16)).all():
+                break
+        else:
+            pytest.fail("no sign of the infinity gives a score of minus infinity")
+    g = GpuShard(shape, w)
+    got = outputs(GpuEngine(g, 1, L + n_new))
+    assert_close(got, want, what="key at minus infinity")
+    g.close()
