@@ -121,8 +121,12 @@ int kv_state_reset(kvstate_t state, int row);
 
 /* Sets one layer of one row to `len` cache entries from host fp16 K and V,
  * each [len][Hkv][d] (a prefilled cache, Section 3.4); the row's length
- * becomes len (load every layer with the same len).  Synchronous.  Errors: EINVAL, ECAPACITY (len > capacity),
- * EUNSUPPORTED (row entries shared through a beam gather; reset first). */
+ * becomes len (load every layer with the same len).  Synchronous.  The copies
+ * go through a staging buffer of up to 32 MiB of device memory that stays with
+ * the shard (shard_step_host uses the same one); with less memory free it is
+ * smaller, with none the load is slower but goes without.  Errors: EINVAL,
+ * ECAPACITY (len > capacity), EUNSUPPORTED (row entries shared through a beam
+ * gather; reset first). */
 int kv_state_load(kvstate_t state, int row, int layer, const uint16_t* k, const uint16_t* v, int len);
 
 /* Copies cache entries [start, start+len) of one row and layer, in the row's

@@ -65,6 +65,11 @@ int shard_debug_gemm_rings(int S, int group, int* tile, int* rings);
  * Synchronises the device. */
 int shard_debug_phase_times(shard_t shard, double* us, int n);
 
+/* Test knob for kv_state_load's staging buffer: gives the present one back and
+ * makes later loads behave as if no more than `bytes` of device memory could be
+ * had for it (0: none, so the load makes strided copies; -1: no limit). */
+int shard_debug_set_load_stage(shard_t shard, long long bytes);
+
 /* Test knob for the step kernel's bounded waits (they must never hang the
  * GPU; the paper has no counterpart): limit = polls before a cross-CTA wait
  * gives up (default 2^22); skip_arrival >= 0 makes CTA 1 leave out its arrival at that grid barrier of every following

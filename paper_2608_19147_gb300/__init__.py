@@ -28,7 +28,7 @@ OP_QKV, OP_O, OP_GU, OP_DOWN = 0, 1, 2, 3
 EXPORTS = ("shard_create", "shard_destroy", "kv_state_alloc", "kv_state_free", "kv_state_reset", "kv_state_load",
            "kv_state_read", "kv_state_length", "kv_trim", "kv_state_export", "kv_state_import", "shard_step", "shard_step_packed", "shard_prefill", "shard_step_host", "shard_sync_status",
            "shard_last_error", "shard_debug_op_info", "shard_debug_unpack", "shard_debug_gemv", "shard_debug_gemm",
-           "shard_debug_gemm_rings", "shard_debug_phase_times", "shard_debug_set_wait", "shard_gemv_noalloc", "head_create", "head_destroy", "head_top1",
+           "shard_debug_gemm_rings", "shard_debug_set_load_stage", "shard_debug_phase_times", "shard_debug_set_wait", "shard_gemv_noalloc", "head_create", "head_destroy", "head_top1",
            "head_top1_host", "head_debug_logits")
 # per layer, between the ends of grid-barrier waits: attention (with the next
 # layer's RMSNorm + q|k|v projection in front of it after the first layer), o,
@@ -110,6 +110,7 @@ def load_library(path: str = LIB_PATH):
         "shard_debug_phase_times": ([vp, ctypes.POINTER(ctypes.c_double), ip], ip),
         "shard_debug_gemm": ([vp, ip, ip, vp, ip, ip, vp, ip, vp], ip),
         "shard_debug_gemm_rings": ([ip, ip, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)], ip),
+        "shard_debug_set_load_stage": ([vp, ctypes.c_longlong], ip),
         "shard_debug_set_wait": ([vp, ctypes.c_uint, ip], ip),
         "head_create": ([ctypes.POINTER(head_config), ctypes.POINTER(head_weights_host), ctypes.POINTER(vp)], ip),
         "head_destroy": ([vp], ip),
@@ -314,6 +315,11 @@ def shard_debug_phase_times(shard: int, n_layers: int):
     if k < 0:
         _check(k)
     return list(buf)[:k]
+
+
+def shard_debug_set_load_stage(shard: int, nbytes: int) -> None:
+    """Test knob of kv_state_load's staging buffer (include/shard_debug.h)."""
+    _check(load_library().shard_debug_set_load_stage(shard, int(nbytes)))
 
 
 def shard_debug_set_wait(shard: int, limit: int, skip_arrival: int = -1) -> None:

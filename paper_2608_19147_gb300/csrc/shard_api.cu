@@ -124,6 +124,7 @@ struct shard_s {
   size_t pin_bytes = 0;
   void* dstage = nullptr;
   size_t dstage_bytes = 0;
+  long long stage_limit = -1;  // test knob (shard_debug_set_load_stage)
   std::vector<kvstate_s*> states;
 };
 
@@ -585,14 +586,32 @@ int kv_state_reset(kvstate_t st, int row) {
 constexpr size_t kLoadStageBytes = 32u << 20;  // staged at a time by kv_state_load
 
 // At least `bytes` of the shard's device staging buffer (no work in flight uses it).
+// One that cannot grow stays as it is.
 static cudaError_t grow_stage(shard_s* sh, size_t bytes) {
   if (sh->dstage_bytes >= bytes) return cudaSuccess;
+  void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // reported by the caller, or done without
+    return e;
+  }
   cudaFree(sh->dstage);
-  sh->dstage = nullptr;
-  sh->dstage_bytes = 0;  // a failed allocation leaves no stale size behind
-  const cudaError_t e = cudaMalloc(&sh->dstage, bytes);
-  if (e == cudaSuccess) sh->dstage_bytes = bytes;
-  return e;
+  sh->dstage = p;
+  sh->dstage_bytes = bytes;
+  return cudaSuccess;
+}
+
+// A staging buffer for pieces of up to `entries` cache entries of `bytes` each:
+// the whole load's, else halves of that while memory is short, else what is there.
+// Returns the entries it holds (0: none).
+static int load_stage(shard_s* sh, int entries, size_t bytes) {
+  int most = (int)std::max<size_t>(1, std::min<size_t>(entries, kLoadStageBytes / bytes));
+  const auto held = [&] { return (int)std::min<size_t>(most, sh->dstage_bytes / bytes); };
+  for (; held() < most; most = (most + 1) / 2) {
+    const bool allowed = sh->stage_limit < 0 || (long long)(bytes * most) <= sh->stage_limit;
+    if ((allowed && grow_stage(sh, bytes * most) == cudaSuccess) || most == 1) break;
+  }
+  return held();
 }
 
 int kv_state_load(kvstate_t st, int row, int layer, const uint16_t* k, const uint16_t* v, int len) {
@@ -608,16 +627,16 @@ int kv_state_load(kvstate_t st, int row, int layer, const uint16_t* k, const uin
   // head-major pool: a strided copy of 256-byte rows per head took 16 calls a
   // layer (8 rows of 128..2048 entries into 4 layers of the 8B shape: 6.5 -> 2.6 ms)
   const size_t per = (size_t)sh->Hkv * sh->d;  // values per entry
-  int most = (int)std::max<size_t>(1, std::min<size_t>(len, kLoadStageBytes / (2 * sizeof(uint16_t) * per)));
-  if (len > 0) {
-    cudaError_t e;
-    while ((e = grow_stage(sh, 2 * sizeof(uint16_t) * per * most)) == cudaErrorMemoryAllocation && most > 1) {
-      cudaGetLastError();  // little memory left: smaller pieces
-      most = (most + 1) / 2;
+  const int most = len > 0 ? load_stage(sh, len, 2 * sizeof(uint16_t) * per) : 0;
+  if (len > 0 && most == 0) {  // not even one entry's worth of memory left
+    const size_t w = sizeof(uint16_t) * sh->d;
+    for (int h = 0; h < sh->Hkv; ++h) {
+      const size_t at = (size_t)layer * st->layer_stride + ((size_t)row * sh->Hkv + h) * st->cap * sh->d;
+      CUDA_TRY(cudaMemcpy2D(st->k + at, w, k + (size_t)h * sh->d, w * sh->Hkv, w, len, cudaMemcpyHostToDevice));
+      CUDA_TRY(cudaMemcpy2D(st->v + at, w, v + (size_t)h * sh->d, w * sh->Hkv, w, len, cudaMemcpyHostToDevice));
     }
-    CUDA_TRY(e);
   }
-  for (int j0 = 0; j0 < len; j0 += most) {
+  for (int j0 = 0; most > 0 && j0 < len; j0 += most) {
     const int n = std::min(most, len - j0);
     uint16_t* in = static_cast<uint16_t*>(sh->dstage);
     const size_t bytes = sizeof(uint16_t) * per * n, off = (size_t)layer * st->layer_stride + (size_t)j0 * sh->d;
@@ -1073,7 +1092,14 @@ int shard_step_host(shard_t sh, kvstate_t st, const uint16_t* hidden_in, const i
     CUDA_TRY(cudaHostAlloc(&sh->pin, need, cudaHostAllocDefault));
     sh->pin_bytes = need;
   }
-  CUDA_TRY(grow_stage(sh, need));
+  cudaError_t staged = grow_stage(sh, need);
+  if (staged == cudaErrorMemoryAllocation && sh->dstage) {  // room may come from the smaller one
+    cudaFree(sh->dstage);
+    sh->dstage = nullptr;
+    sh->dstage_bytes = 0;
+    staged = grow_stage(sh, need);
+  }
+  CUDA_TRY(staged);
   uint8_t* hp = static_cast<uint8_t*>(sh->pin);
   uint8_t* dp = static_cast<uint8_t*>(sh->dstage);
   size_t off = 0;
@@ -1218,6 +1244,17 @@ int shard_debug_gemm_rings(int S, int group, int* tile, int* rings) {
   *tile = gemm_tc_tile(S, group);
   gemm_tc_rings(*tile, group, r);
   std::copy(r, r + 6, rings);
+  return SHARD_OK;
+}
+
+int shard_debug_set_load_stage(shard_t sh, long long bytes) {
+  if (!sh || bytes < -1) return fail(SHARD_EINVAL, "shard_debug_set_load_stage: bad argument");
+  CUDA_TRY(cudaSetDevice(sh->device));
+  CUDA_TRY(cudaDeviceSynchronize());
+  cudaFree(sh->dstage);
+  sh->dstage = nullptr;
+  sh->dstage_bytes = 0;
+  sh->stage_limit = bytes;
   return SHARD_OK;
 }
 
