@@ -31,6 +31,8 @@ CASES = {
     "shared-merge": (16, 2, 128, [4], [2999]),
     "whole-rows": (16, 16, 64, [1] * 10, [1100, 1023, 1024, 1, 17, 900, 64, 1090, 300, 0]),
     "uneven": (8, 2, 128, [3, 1, 5, 2], [700, 3, 129, 2049]),
+    "two-passes-shared-merge": (16, 1, 64, [9], [2500]),
+    "runs": (8, 4, 128, [2, 1, 3, 1], [2100, 1500, 1800, 2600]),
 }
 
 
@@ -73,7 +75,7 @@ def test_attention_edges(name):
     _run(name, lambda b, l: rng.random(l) < 0.8, synth.make_weights(shape, 3), shape)
 
 
-@pytest.mark.parametrize("name", ["item+1", "uneven", "shared-merge", "whole-rows"])
+@pytest.mark.parametrize("name", ["item+1", "uneven", "shared-merge", "whole-rows", "two-passes-shared-merge", "runs"])
 def test_attention_items_nobody_sees(name):
     """Only the last 10 cached entries are visible: whole items contribute nothing."""
     shape = _shape(name)

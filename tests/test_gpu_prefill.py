@@ -2,12 +2,12 @@
 cache by running through the stage) against the fp64 oracle, through the C
 ABI.  The oracle's reference is its decode step with all S prompt tokens as
 the new tokens of one request -- the method's definition; the GPU computes
-it with the projections on the tensor cores (tcgen05), in chunks of 256
+it with the projections on the tensor cores (tcgen05), in chunks of 512
 tokens.  Checked at the fixed bar (relative L2 1e-3, max-abs 2e-2 with one
 fp16 ulp where that is larger):
 
-* the tiny shard: a prompt after a short cache, a prompt of two chunks on an
-  empty row, token-id and hidden-state inputs, a prompt with masked holes in
+* the tiny shard: a prompt after a short cache, prompts of one chunk and of two
+  on an empty row and after a cache, token-id and hidden-state inputs, a prompt with masked holes in
   the row's cache, and a second row of a two-row state;
 * two layers of the Llama-3.1-8B stage: a 200-token prompt on a 72-entry
   cache;
@@ -60,7 +60,8 @@ def tiny():
     sh.close()
 
 
-@pytest.mark.parametrize("P,S,use_tokens", [(10, 37, True), (0, 300, False), (72, 16, False)])
+@pytest.mark.parametrize("P,S,use_tokens", [(10, 37, True), (0, 300, False), (72, 16, False), (5, 530, True),
+                                            (0, 600, False)])
 def test_tiny_prefill_matches_oracle_and_decoding_continues(tiny, P, S, use_tokens):
     w, sh = tiny
     shape = synth.TINY
