@@ -874,8 +874,8 @@ def run_prefill(args, rank: int, world: int):
             pkg.kv_state_reset(st, -1)
     pkg.shard_sync_status(sh, sptr)
     ms = max_over_ranks(ms_total, dist, dev)
-    # the dominant kernel, the tensor-core projection, timed alone per 512-token chunk on layer 0
-    # (with the export's reordering of its input, and all of K in one part)
+    # the dominant kernel, the tensor-core projection, timed alone per 512-token chunk on layer 0:
+    # the launches that the prefill makes (K in as many parts, SwiGLU in gate|up's epilogue)
     chunk = 512
     proj = {}
     flops_chunk, ms_chunk = 0.0, 0.0
@@ -884,20 +884,22 @@ def run_prefill(args, rank: int, world: int):
         ld = (Kin + 127) // 128 * 128
         x = torch.zeros((chunk, ld), dtype=torch.int16, device=dev)
         x[:, :Kin] = torch.from_numpy(synth.hidden_in(dataclasses.replace(shape, hidden=Kin), SEED, 9, chunk).view(np.int16))
-        y = torch.empty((chunk, rows), dtype=torch.float32, device=dev)
+        y = torch.empty((4, chunk, rows), dtype=torch.float32, device=dev)
+        h_ld = (shape.ffn + 127) // 128 * 128
+        outs = dict(h=y.data_ptr(), h_ld=h_ld) if k == pkg.OP_GU else dict(y=y.data_ptr(), y_ld=rows, y_part=chunk * rows)
         for _ in range(3):
-            pkg.shard_debug_gemm(sh, 0, k, x.data_ptr(), ld, chunk, y.data_ptr(), rows, sptr)
+            parts = pkg.shard_debug_gemm_stage(sh, 0, k, x.data_ptr(), ld, chunk, stream=sptr, **outs)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         reps = 20
         torch.cuda.synchronize()
         e0.record(stream)
         for _ in range(reps):
-            pkg.shard_debug_gemm(sh, 0, k, x.data_ptr(), ld, chunk, y.data_ptr(), rows, sptr)
+            pkg.shard_debug_gemm_stage(sh, 0, k, x.data_ptr(), ld, chunk, stream=sptr, **outs)
         e1.record(stream)
         torch.cuda.synchronize()
         t_ms = e0.elapsed_time(e1) / reps
         fl = 2.0 * rows * Kin * chunk
-        proj[name] = {"us_per_call": t_ms * 1e3, "tflops": fl / (t_ms * 1e9)}
+        proj[name] = {"us_per_call": t_ms * 1e3, "tflops": fl / (t_ms * 1e9), "k_parts": parts}
         flops_chunk += fl
         ms_chunk += t_ms
     # the same projection at decode-sized token counts: the decode step's
@@ -975,7 +977,7 @@ def run_prefill(args, rank: int, world: int):
                    "parallelism": "replicas" if world > 1 else "single GPU", "seed": SEED},
         "roofline": {
             "kernel": "gemm_tc (W4A16 projection, tcgen05.mma kind::f16 M=128, N=128 tokens, accumulator in TMEM), "
-                      "one 512-token chunk of each projection of layer 0, timed alone with its input's reordering",
+                      "one 512-token chunk of each projection of layer 0, timed alone as the prefill launches it",
             "bound": "tensor",
             "achieved": flops_chunk / (ms_chunk * 1e9),
             "peak": peak,

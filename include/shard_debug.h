@@ -43,10 +43,24 @@ int shard_debug_gemv(shard_t shard, int layer, int op, const uint16_t* x, int M,
  * [S][x_ld], 16-byte aligned, x_ld a multiple of 128 and >= K rounded up to
  * 128, columns K .. x_ld - 1 zero; y dev fp32 [S][y_ld], y_ld >= rows,
  * natural row order.  Same W4A16 arithmetic as the step's projections (exact
- * q - z, fp32 sums, the fp16 group scale applied in fp32).  Asynchronous on
- * cuda_stream. */
+ * q - z, fp32 sums, the fp16 group scale applied in fp32).  All of K in one
+ * part.  x is first copied into the kernel's order of inputs, in a buffer that the
+ * shard keeps and a first or larger call allocates (not under stream capture).
+ * Asynchronous on cuda_stream. */
 int shard_debug_gemm(shard_t shard, int layer, int op, const uint16_t* x, int x_ld, int S, float* y, int y_ld,
                      void* cuda_stream);
+
+/* The many-token projection as shard_prefill launches it.  x dev fp16 [S][x_ld] as
+ * for shard_debug_gemm, but each block of 32 inputs in the kernel's order: input k
+ * at 16 ((k >> 2) & 1) + 4 ((k >> 3) & 3) + (k & 3).  Either y: dev fp32, K in
+ * `parts` parts (1..4, at most K / 128 rounded up; 0: as many as a prefill of S
+ * tokens takes), part p's sums at y + p * y_part, [S][y_ld], natural rows.  Or h
+ * (op 2, parts 0 or 1): dev fp16 [S][h_ld], silu(gate) * up in the same order of
+ * inputs, h_ld a multiple of 8 and >= F rounded up to 128; values past F are left as
+ * they are.  Nothing is allocated.  Asynchronous on cuda_stream.  Returns the parts
+ * (1..4), or a negative error. */
+int shard_debug_gemm_stage(shard_t shard, int layer, int op, const uint16_t* x, int x_ld, int S, int parts, float* y,
+                           int y_ld, long long y_part, uint16_t* h, int h_ld, void* cuda_stream);
 
 /* The many-token projection's token tile for S tokens and its rings, for a
  * model of its barriers: rings[0..5] = stages of weight units, of token tiles

@@ -28,7 +28,7 @@ OP_QKV, OP_O, OP_GU, OP_DOWN = 0, 1, 2, 3
 EXPORTS = ("shard_create", "shard_destroy", "kv_state_alloc", "kv_state_free", "kv_state_reset", "kv_state_load",
            "kv_state_read", "kv_state_length", "kv_trim", "kv_state_export", "kv_state_import", "shard_step", "shard_step_packed", "shard_prefill", "shard_step_host", "shard_sync_status",
            "shard_last_error", "shard_debug_op_info", "shard_debug_unpack", "shard_debug_gemv", "shard_debug_gemm",
-           "shard_debug_gemm_rings", "shard_debug_set_load_stage", "shard_debug_phase_times", "shard_debug_set_wait", "shard_gemv_noalloc", "head_create", "head_destroy", "head_top1",
+           "shard_debug_gemm_stage", "shard_debug_gemm_rings", "shard_debug_set_load_stage", "shard_debug_phase_times", "shard_debug_set_wait", "shard_gemv_noalloc", "head_create", "head_destroy", "head_top1",
            "head_top1_host", "head_debug_logits")
 # per layer, between the ends of grid-barrier waits: attention (with the next
 # layer's RMSNorm + q|k|v projection in front of it after the first layer), o,
@@ -109,6 +109,7 @@ def load_library(path: str = LIB_PATH):
         "shard_gemv_noalloc": ([vp, ip, ip, vp, ip, vp, ip, vp], ip),
         "shard_debug_phase_times": ([vp, ctypes.POINTER(ctypes.c_double), ip], ip),
         "shard_debug_gemm": ([vp, ip, ip, vp, ip, ip, vp, ip, vp], ip),
+        "shard_debug_gemm_stage": ([vp, ip, ip, vp, ip, ip, ip, vp, ip, ctypes.c_longlong, vp, ip, vp], ip),
         "shard_debug_gemm_rings": ([ip, ip, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)], ip),
         "shard_debug_set_load_stage": ([vp, ctypes.c_longlong], ip),
         "shard_debug_set_wait": ([vp, ctypes.c_uint, ip], ip),
@@ -296,6 +297,14 @@ def shard_debug_gemm(shard: int, layer: int, op: int, x: int, x_ld: int, S: int,
                      stream: int = 0) -> None:
     """Many-token tensor-core projection (device pointers as ints; x padded to x_ld)."""
     _check(load_library().shard_debug_gemm(shard, layer, op, x, x_ld, S, y, y_ld, stream or None))
+
+
+def shard_debug_gemm_stage(shard: int, layer: int, op: int, x: int, x_ld: int, S: int, parts: int = 0,
+                           y: Optional[int] = None, y_ld: int = 0, y_part: int = 0, h: Optional[int] = None, h_ld: int = 0,
+                           stream: int = 0) -> int:
+    """The many-token projection as shard_prefill launches it (x in the kernel's order of inputs); the parts of K."""
+    rc = load_library().shard_debug_gemm_stage(shard, layer, op, x, x_ld, S, parts, y, y_ld, y_part, h, h_ld, stream or None)
+    return rc if rc > 0 else _check(rc)
 
 
 def shard_debug_gemm_rings(S: int, group: int):

@@ -1237,6 +1237,42 @@ int shard_debug_gemm(shard_t sh, int layer, int op, const uint16_t* x, int x_ld,
   return SHARD_OK;
 }
 
+int shard_debug_gemm_stage(shard_t sh, int layer, int op, const uint16_t* x, int x_ld, int S, int parts, float* y,
+                           int y_ld, long long y_part, uint16_t* h, int h_ld, void* cuda_stream) {
+  if (!sh || !x || (y == nullptr) == (h == nullptr) || layer < 0 || layer >= sh->L || op < 0 || op >= N_OPS || S < 1)
+    return fail(SHARD_EINVAL, "shard_debug_gemm_stage: bad argument");
+  const PackedOp& p = sh->ops[(size_t)layer * N_OPS + op];
+  const int nat[N_OPS] = {sh->dq + 2 * sh->dkv, sh->H, 2 * sh->F, sh->H};
+  if (parts == 0) parts = op == OP_GU ? 1 : gemm_tc_parts(p.n_rb, p.upr, S, sh->cfg.group, sh->num_sms);
+  if (parts < 1 || parts > std::min(kGemmMaxParts, p.upr) || (h && (op != OP_GU || parts != 1)))
+    return fail(SHARD_EINVAL, "shard_debug_gemm_stage: %d parts of %d units, or h for another projection", parts, p.upr);
+  if (x_ld < p.Kp || x_ld % kUnitK || reinterpret_cast<uintptr_t>(x) % 16)
+    return fail(SHARD_EINVAL, "shard_debug_gemm_stage: x_ld %d must be a multiple of 128 and >= %d; x 16-byte aligned",
+                x_ld, p.Kp);
+  if (y ? y_ld < nat[op] || y_part < (long long)S * y_ld
+        : h_ld < round_up(sh->F, kUnitK) || h_ld % 8 || reinterpret_cast<uintptr_t>(h) % 16)
+    return fail(SHARD_EINVAL, "shard_debug_gemm_stage: output too small or misaligned");
+  CUDA_TRY(cudaSetDevice(sh->device));
+  GemmArgs g{};
+  g.units = p.units;
+  g.n_rb = p.n_rb;
+  g.upr = p.upr;
+  g.act = x;
+  g.act_ld = x_ld;
+  g.S = S;
+  g.parts = parts;
+  g.y = y;
+  g.y_ld = y_ld;
+  g.y_part = (size_t)y_part;
+  g.h = h;
+  g.h_ld = h_ld;
+  g.F = sh->F;
+  g.dims = p.dims;
+  g.status = sh->status;
+  CUDA_TRY(launch_gemm_tc(g, sh->cfg.group, static_cast<cudaStream_t>(cuda_stream)));
+  return parts;
+}
+
 int shard_debug_gemm_rings(int S, int group, int* tile, int* rings) {
   if (S < 1 || (group != 32 && group != 64 && group != 128) || !tile || !rings)
     return fail(SHARD_EINVAL, "shard_debug_gemm_rings: bad argument");
