@@ -153,8 +153,8 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                : "memory");
 }
 
-// W (8 or 16) consecutive fp32 columns of this thread's tensor-memory lane; the
-// registers are not to be read before tc_ld_wait.
+// 16 consecutive fp32 columns of this thread's tensor-memory lane; the registers
+// are not to be read before tc_ld_wait.
 __device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
@@ -164,17 +164,10 @@ __device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr)
-               : "memory");
-}
-template <int W>
-__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[W]) {
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < W; ++i) asm volatile("" : "+r"(r[i]));  // not read before the wait
+  for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(r[i]));  // not read before the wait
 }
 
 // 2-D tensor copy of one box into shared memory, completion on `bar`.
@@ -201,7 +194,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
   constexpr int G = GPU;                        // quantisation groups per unit
   constexpr int kMmaPerGroup = 8 / GPU;         // K = 16 per instruction
   constexpr int kPer = N / (kEpiWarps / 4);     // token columns per epilogue thread
-  constexpr int kLd = kPer < 16 ? kPer : 16;    // of them, columns per load
+  constexpr int kLd = 16;                       // of them, columns per load
   constexpr int kDStages = L::kDStages;
   constexpr uint32_t kHalfB = N * 128;          // bytes per 64-input half
   static_assert(kPer % kLd == 0, "columns per epilogue thread");

@@ -1,7 +1,7 @@
 // Standalone launch of one W4A16 projection (the test export
 // shard_debug_gemv, the allocation-free entry point and the LM head use it).
 // The device code is the warp-level projection of gemv_core.cuh, the same
-// code the whole-step kernel runs: kGemvWarps consumer warps per CTA, one CTA
+// code the whole-step kernel runs: kGemvWarps warps per CTA, one CTA
 // per SM.
 #include <algorithm>
 
@@ -12,13 +12,13 @@ namespace {
 
 constexpr int kCtasPerSm = 1;
 
-constexpr int kW = kGemvWarps;  // consumer warps per CTA
-constexpr int kBlock = (kW + (kSelfRefill ? 0 : 1)) * 32;
+constexpr int kW = kGemvWarps;  // warps per CTA
+constexpr int kBlock = kW * 32;
 
 template <int GPU>
 constexpr size_t smem_bytes() {
   constexpr int kSlots = Geom<GPU>::kGemvSlots;
-  return (size_t)kW * kSlots * Geom<GPU>::kUnitBytes + (size_t)2 * kW * kSlots * sizeof(uint64_t);
+  return (size_t)kW * kSlots * Geom<GPU>::kUnitBytes + (size_t)kW * kSlots * sizeof(uint64_t);
 }
 
 // 227 KB per CTA, less a margin for the kernel's static shared memory
@@ -34,7 +34,6 @@ __global__ void __launch_bounds__(kBlock, 1) gemv_kernel(const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* rings = smem;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)kW * kSlots * Geom<GPU>::kUnitBytes);
-  uint64_t* empty = full + kW * kSlots;
   if (threadIdx.x == 0) {
     s_op[0] = OpDesc{a.units, a.n_rb, a.upr, 0};
     GemvPhase p{};
@@ -44,22 +43,16 @@ __global__ void __launch_bounds__(kBlock, 1) gemv_kernel(const __grid_constant__
     p.status = a.status;
     p.ep = a.ep;
     s_gp = p;
-    ring_init_barriers(full, empty, kW * kSlots);
+    ring_init_barriers(full, kW * kSlots);
   }
   __syncthreads();
-  if (!kSelfRefill && warp == kW) {
-    // the weights do not depend on the preceding kernel: start streaming them
-    ring_producer<GPU, kSlots>(s_op, 1, blockIdx.x, gridDim.x, kW, rings, full, empty, a.status, 1u << 22, lane);
-    return;
-  }
   const int g = blockIdx.x * kW + warp, nw = gridDim.x * kW;
   WarpRing<GPU, kSlots> ring;
   ring.ring = rings + (size_t)warp * kSlots * Geom<GPU>::kUnitBytes;
   ring.full = full + warp * kSlots;
-  ring.empty = empty + warp * kSlots;
   ring.n_used = 0;
   ring.timed_out = false;
-  if (kSelfRefill) ring.start(s_op, 1, g, nw, lane);  // the weights do not depend on the preceding kernel
+  ring.start(s_op, 1, g, nw, lane);  // the weights do not depend on the preceding kernel
   pdl_wait();
   gemv_run<NT, GPU, kSlots>(ring, &s_op[0], &s_gp, g, nw, lane);
   // a dependent kernel may take the SMs that run out of work (not earlier: its

@@ -2,20 +2,19 @@
 // kernel and the standalone projection kernel.
 //
 // Work split.  The unit stream of a projection (n_rb row-blocks x upr units,
-// see kernels.h) is cut into contiguous runs, one per consumer warp of the
+// see kernels.h) is cut into contiguous runs, one per warp of the
 // grid (warp g = cta * warps per CTA + warp), so every warp streams the same
 // number of bytes and keeps its sums in registers for as long as its run
 // stays inside one row-block.
 //
-// Weight streaming.  Every consumer warp owns a ring of shared-memory slots,
+// Weight streaming.  Every warp owns a ring of shared-memory slots,
 // filled with one bulk copy (TMA, non-tensor) per unit, completion signalled
 // on the slot's "full" mbarrier.  The warp's stream is its run of every
 // projection of the launch, in order; because the weights never depend on
-// earlier work, the rings run ahead across projections: while consumers wait
+// earlier work, the rings run ahead across projections: while warps wait
 // at a barrier or work on norms and attention, their next projection's first
-// units are already arriving.  The slot a warp has consumed is refilled
-// either by the warp's own lane 0 at once (kSelfRefill) or by a producer warp
-// that watches the slots' "empty" mbarriers.
+// units are already arriving.  The warp's own lane 0 refills
+// the slot that the warp has consumed, at once.
 //
 // Per unit, a lane turns each 32-bit code word into the four registers of its
 // m16n8k16 A fragment with one AND per register (the codes as fp16
@@ -37,18 +36,12 @@
 
 namespace shard {
 
-// Weight streaming: with kSelfRefill, each consumer warp's lane 0 refills the
-// slot the warp has just consumed with its next unit; otherwise a producer
-// warp per CTA fills every consumer's ring.  Consumer warps per CTA: 12
-// (3 per SM sub-partition), or 11 beside the producer (the sub-partition's
-// register file caps 4 warps at 128 registers each).
-constexpr bool kSelfRefill = true;
-constexpr int kRingSlots = 2;  // step kernel: units in flight per consumer warp (a deeper ring takes the L1 that the norm and attention loads use)
-constexpr int kCtaWarps = kSelfRefill ? 12 : 11;   // consumer warps per CTA of the step kernel
-// Consumer warps per CTA of the standalone projection kernel, whose loop fits 128
+constexpr int kRingSlots = 2;  // step kernel: units in flight per warp (a deeper ring takes the L1 that the norm and attention loads use)
+constexpr int kCtaWarps = 12;  // warps per CTA of the step kernel (3 per SM sub-partition: 168 registers a thread)
+// Warps per CTA of the standalone projection kernel, whose loop fits 128
 // registers (a warp's unit is a chain of latencies: 128256 x 4096 lm_head, 1
 // token 58.5 -> 53.4 us, 5 tokens 67 -> 60, 8 tokens 72 -> 63 against 12 warps).
-constexpr int kGemvWarps = kSelfRefill ? 16 : 11;
+constexpr int kGemvWarps = 16;
 
 template <int GPU>
 struct Geom {
@@ -201,10 +194,9 @@ struct WarpRing {
   static constexpr int UB = Geom<GPU>::kUnitBytes;
   uint8_t* ring;       // [S][UB]
   uint64_t* full;      // [S]
-  uint64_t* empty;     // [S] (producer mode)
   uint32_t n_used;
   bool timed_out;
-  StreamCursor cur;    // self-refill mode: lane 0's copy drives the refills
+  StreamCursor cur;    // lane 0's copy drives the refills
   uint64_t policy;
 
   __device__ __forceinline__ void issue(uint32_t slot, const uint8_t* src) {
@@ -212,7 +204,7 @@ struct WarpRing {
     // L2 evict-first: each weight byte is read once per launch
     bulk_g2s_hint(ring + (size_t)slot * UB, src, UB, &full[slot], policy);
   }
-  // Self-refill mode: lane 0 fills the first S slots.
+  // Lane 0 fills the first S slots.
   __device__ __forceinline__ void start(const OpDesc* ops, int n_ops, int g, int nw, int lane) {
     cur.init(ops, n_ops, g, nw, UB);
     policy = l2_policy_evict_first();
@@ -237,85 +229,26 @@ struct WarpRing {
     }
     return ring + (size_t)slot * UB;
   }
-  // The unit's fragments are in registers: refill the slot with the warp's
-  // next unit (self-refill), or hand it back to the producer.
+  // The unit's fragments are in registers: refill the slot with the warp's next unit.
   __device__ __forceinline__ void release(int lane) {
     __syncwarp();
     const uint32_t slot = n_used % S;
     if (lane == 0) {
-      if (kSelfRefill) {
-        const uint8_t* src;
-        if (cur.next(src, UB)) {
-          // the warp's generic-proxy reads of the slot come before the copy's writes
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          issue(slot, src);
-        }
-      } else {
-        mbar_arrive(&empty[slot]);
+      const uint8_t* src;
+      if (cur.next(src, UB)) {
+        // the warp's generic-proxy reads of the slot come before the copy's writes
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        issue(slot, src);
       }
     }
     ++n_used;
   }
 };
 
-// Initialises the full/empty barriers of all rings of the CTA (one thread).
-__device__ __forceinline__ void ring_init_barriers(uint64_t* full, uint64_t* empty, int n) {
-  for (int i = 0; i < n; ++i) {
-    mbar_init(&full[i], 1);
-    mbar_init(&empty[i], 1);
-  }
+// Initialises the barriers of all rings of the CTA (one thread).
+__device__ __forceinline__ void ring_init_barriers(uint64_t* full, int n) {
+  for (int i = 0; i < n; ++i) mbar_init(&full[i], 1);
   mbar_fence_init();
-}
-
-// Producer mode: lane w < n_warps fills consumer warp w's ring of S slots
-// with the warp's runs of ops[0 .. n_ops), in order; a slot is refilled once
-// its previous unit was released.  Every lane runs the same loop (ready
-// lanes issue, others wait for the next pass), so no lane's wait holds up
-// another's copy.  Bounded: `limit` passes without any copy set
-// ST_WAIT_TIMEOUT and end the producer (the consumers' own bounded waits
-// then give up too).
-template <int GPU, int S>
-__device__ __noinline__ void ring_producer(const OpDesc* ops, int n_ops, int cta, int n_cta, int n_warps, uint8_t* rings,
-                                           uint64_t* full, uint64_t* empty, int* status, uint32_t limit, int lane) {
-  constexpr int UB = Geom<GPU>::kUnitBytes;
-  const bool mine = lane < n_warps;
-  uint8_t* ring = rings + (size_t)(mine ? lane : 0) * S * UB;
-  uint64_t* f = full + (mine ? lane : 0) * S;
-  uint64_t* e = empty + (mine ? lane : 0) * S;
-  StreamCursor cur;
-  cur.init(ops, mine ? n_ops : 0, cta * n_warps + lane, n_cta * n_warps, UB);
-  const uint64_t policy = l2_policy_evict_first();
-  bool active = mine;
-  const uint8_t* src = nullptr;
-  bool have = false;  // `src` holds the next unit, not yet issued
-  uint32_t n = 0, idle = 0;
-  while (true) {
-    if (active && !have) {
-      have = cur.next(src, UB);
-      active = have;
-    }
-    bool issued = false;
-    if (have) {
-      const uint32_t slot = n % S;
-      if (n < (uint32_t)S || mbar_test_wait(&e[slot], ((n / S) - 1) & 1)) {
-        mbar_arrive_expect_tx(&f[slot], UB);
-        bulk_g2s_hint(ring + (size_t)slot * UB, src, UB, &f[slot], policy);
-        ++n;
-        have = false;
-        issued = true;
-      }
-    }
-    if (!__any_sync(0xffffffffu, active)) break;
-    if (__any_sync(0xffffffffu, issued)) {
-      idle = 0;
-    } else {
-      if (++idle > limit) {
-        if (lane == 0) atomicOr(status, ST_WAIT_TIMEOUT);
-        break;
-      }
-      __nanosleep(20);
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------

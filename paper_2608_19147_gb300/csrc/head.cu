@@ -19,7 +19,7 @@
 #include <vector>
 
 #include "../../include/head.h"
-#include "common.cuh"
+#include "launch.cuh"
 
 namespace shard {
 // Sets the calling thread's last error (shard_api.cu) and returns code.
@@ -331,17 +331,8 @@ int run(head_s* h, const uint16_t* hidden, int M, int32_t* token, float* p_max, 
   if (token) {
     int nc = 0;
     const int chunk = chunk_of(h, M, &nc);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nc, M);
-    cfg.blockDim = dim3(kTopThreads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    HEAD_CUDA_TRY(cudaLaunchKernelEx(&cfg, head_top1_kernel, (const float*)logits, ld, (int)c.vocab, chunk, h->parts, h->done,
-                                     (const int*)h->status, token, p_max));
+    HEAD_CUDA_TRY(launch_behind(head_top1_kernel, dim3(nc, M), kTopThreads, 0, s, (const float*)logits, ld, (int)c.vocab,
+                                chunk, h->parts, h->done, (const int*)h->status, token, p_max));
   }
   return SHARD_OK;
 }

@@ -1,8 +1,8 @@
 // The whole decode step of a shard as one persistent, cooperative kernel.
 //
-// One CTA per SM: kCtaWarps consumer warps and one producer warp that streams
-// the weights into the consumers' rings (gemv_core.cuh).  The step runs as a
-// sequence of phases separated by grid-wide barriers ('|'):
+// One CTA per SM, whose warps stream their weights into rings of their own
+// (gemv_core.cuh).  The step runs as a sequence of phases separated by grid-wide
+// barriers ('|'):
 //   prologue (every CTA: its share of the beam-table gather, the new
 //   entries' slots and the residual) ~ for each layer: RMSNorm + q|k|v
 //   projection -> attention (chunk partials and merges, with RoPE and the K/V
@@ -31,13 +31,8 @@
 namespace shard {
 namespace {
 
-constexpr int kWarps = kCtaWarps;           // consumer warps
-constexpr int kThreads = kWarps * 32;       // consumer threads
-constexpr int kBlockThreads = kThreads + (kSelfRefill ? 0 : 32);  // + the producer warp, if any
-// Polls of a busy slot before the producer gives up: a slot may legitimately
-// stay busy while its consumer works through a whole attention phase, so this
-// bound is fixed and far above any step's length.
-constexpr uint32_t kProducerLimit = 1u << 22;
+constexpr int kWarps = kCtaWarps;
+constexpr int kThreads = kWarps * 32;
 
 // Dynamic shared memory: weight rings, their barriers, the op table (4L
 // entries), gate|up partial sums (when they fit), and the area: an attention
@@ -49,7 +44,7 @@ template <int GPU>
 struct StepSmem {
   static constexpr int kSlots = Geom<GPU>::kStepSlots;
   static constexpr size_t kRing = (size_t)kWarps * kSlots * Geom<GPU>::kUnitBytes;
-  static constexpr size_t kBars = (size_t)2 * kWarps * kSlots * sizeof(uint64_t);
+  static constexpr size_t kBars = (size_t)kWarps * kSlots * sizeof(uint64_t);
   static constexpr size_t kOps = kRing + kBars;
   // gate|up partial sums of the shared-memory reduction (swiglu_cta_write) for M tokens
   __host__ __device__ static size_t part(int M) { return (size_t)kWarps * M * kRowsPerBlock * sizeof(float); }
@@ -76,7 +71,7 @@ __device__ __forceinline__ int opaque(int v) {
   return v;
 }
 
-// Barrier among the consumer warps of a CTA (the producer warp runs on its own).
+// Barrier among the warps of a CTA.
 __device__ __forceinline__ void cbar() { named_bar_sync(1, kThreads); }
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
@@ -108,8 +103,8 @@ __device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned 
 
 // Grid-wide barrier on a monotonically increasing counter, in two halves so
 // that work may sit between arriving and waiting.  `target` is this CTA's
-// running count of expected arrivals.  Called by the consumer warps; the
-// caller has synchronised them (cbar) before grid_arrive.  Lives in shared
+// running count of expected arrivals.  The caller has
+// synchronised the CTA (cbar) before grid_arrive.  Lives in shared
 // memory (only thread 0 uses it), so that it takes no registers of the phases.
 struct GridBarrier {
   unsigned long long* ctr;
@@ -229,7 +224,7 @@ __device__ __noinline__ void prologue_params(const PrologueArgs& a, StepParams* 
   __syncthreads();
 }
 
-// Prologue, part 2 (consumer threads of every CTA, a share each): the beam
+// Prologue, part 2 (the threads of every CTA, a share each): the beam
 // table's gather and appends, and the residual stream X = the fp16 inputs in
 // fixed point (exact).
 __device__ __noinline__ void prologue_work(const PrologueArgs& a, const StepParams* sp, const uint16_t* const* rowp,
@@ -928,7 +923,7 @@ __device__ __forceinline__ void attn_append(const AttnView& a, const AttnUnit& n
   }
 }
 
-// One chunk by the CTA's consumer warps: its partials, or the outputs of a row of
+// One chunk by the CTA: its partials, or the outputs of a row of
 // one chunk.
 template <int DPL>
 __device__ __forceinline__ void attn_chunk(const AttnView& a, const AttnUnit& n, int c, int layer, const StepParams* sp,
@@ -1175,7 +1170,7 @@ __device__ __forceinline__ void attn_merge(const AttnView& a, const AttnUnit& n,
 }
 
 template <int NT, int GPU, int DPL, bool kMany>
-__global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_constant__ StepKernelArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) step_kernel(const __grid_constant__ StepKernelArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ GemvPhase s_gp[4];            // per projection kind: q|k|v, o, gate|up, down
   constexpr int kSlots = Geom<GPU>::kStepSlots;
@@ -1189,14 +1184,13 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* rings = smem;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + SS::kRing);
-  uint64_t* empty = full + kWarps * kSlots;
   uint8_t* att_area = smem + SS::area(a.L, a.gu_part, a.pro.M);
   static_assert(AttnSmem<DPL>::kBytes <= kAttnArea, "attention area too small");
   OpDesc* s_ops = reinterpret_cast<OpDesc*>(smem + SS::kOps);
-  for (int i = threadIdx.x; i < 4 * a.L; i += kBlockThreads) s_ops[i] = a.ops[i];
+  for (int i = threadIdx.x; i < 4 * a.L; i += kThreads) s_ops[i] = a.ops[i];
   if (threadIdx.x == 0) {
     mbar_init(&s_nbar, 1);
-    ring_init_barriers(full, empty, kWarps * kSlots);  // ends with the barrier-init fence
+    ring_init_barriers(full, kWarps * kSlots);  // ends with the barrier-init fence
     if (blockIdx.x == 0) a.phase_clock[0] = globaltimer();
   }
   const auto plan = [&](int l) {
@@ -1223,12 +1217,6 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
     }
     return;
   }
-  if (!kSelfRefill && warp == kWarps) {  // the producer warp
-    ring_producer<GPU, kSlots>(s_ops, 4 * a.L, blockIdx.x, gridDim.x, kWarps, rings, full, empty, a.status,
-                               kProducerLimit, lane);
-    return;
-  }
-  // ---- consumer warps from here on: CTA barriers are cbar() ----
   const StepParams* sp = &s_sp;
   const int M = sp->M;
   __shared__ GridBarrier gb;
@@ -1240,10 +1228,9 @@ __global__ void __launch_bounds__(kBlockThreads, 1) step_kernel(const __grid_con
   WarpRing<GPU, kSlots> ring;
   ring.ring = rings + (size_t)warp * kSlots * Geom<GPU>::kUnitBytes;
   ring.full = full + warp * kSlots;
-  ring.empty = empty + warp * kSlots;
   ring.n_used = 0;
   ring.timed_out = false;
-  if (kSelfRefill) ring.start(s_ops, 4 * a.L, blockIdx.x * kWarps + warp, gridDim.x * kWarps, lane);
+  ring.start(s_ops, 4 * a.L, blockIdx.x * kWarps + warp, gridDim.x * kWarps, lane);
   // The normalised rows: in the area (idle during the q|k|v and gate|up
   // projections) when they fit, else read from act_h.
   const int xn_ld = xn_stride(a.H);
@@ -1412,7 +1399,7 @@ cudaError_t launch_t(const StepKernelArgs& a, int grid, cudaStream_t s) {
   auto kern = step_kernel<NT, GPU, DPL, kMany>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kBlockThreads);
+  cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = StepSmem<GPU>::area(a.L, a.gu_part, a.pro.M) + a.area_bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
