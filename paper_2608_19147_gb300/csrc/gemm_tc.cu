@@ -231,7 +231,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s_tmem;
-  bool ok = true;  // false once a wait gave up: the role skips the rest of its waits
+  // false once a wait gave up: the role skips the rest of its waits. The producer
+  // then copies nothing more and the MMA thread neither multiplies nor signals, so
+  // that nothing they started is under way when the CTA ends: every copy is waited
+  // for by a role whose waits hold, or was made a whole wait's limit ago.
+  bool ok = true;
   // spinning: the suspending try_wait measured 8 % slower over the whole kernel
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     if (!ok) return;
@@ -266,9 +270,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
         const int su = k % kUStages, sb = k % kBStages;
         if (k >= kUStages) {
           wait(&u_empty[su], ((k / kUStages) & 1) ^ 1);
+          if (!ok) break;
           load_units(k);
         }
         if (k >= kBStages) wait_done(k - kBStages, G - 1);
+        if (!ok) break;
         mbar_arrive_expect_tx(&full[sb], N * 256);
         for (int h = 0; h < 2; ++h)  // tokens past S read as zero
           tma_load_2d(B_of(sb) + (size_t)h * kHalfB, &P.act_map, (k_begin + k) * kUnitK + h * 64, n0, &full[sb]);
@@ -299,8 +305,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
               tc_mma(tmem + (uint32_t)(sd * N), aBase + 8u * kk, bDesc + (((kk >> 2) * kHalfB + (kk & 3) * 32u) >> 4),
                      instr_desc<N>(), i > 0);
             }
+            tc_commit(&done[sb * G + gq]);
           }
-          if (leader) tc_commit(&done[sb * G + gq]);
           __syncwarp();
         }
       }
