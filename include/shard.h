@@ -188,7 +188,8 @@ int kv_state_import(kvstate_t state, int row, const uint16_t* k, const uint16_t*
  *   hidden_out   dev fp16 [M][H] output hidden states
  * Semantics: with P_b the row length after the gather, new token i of request
  * b is stored at entry P_b + i and attends to entries j <= P_b + i of row b
- * with mask[b][j] != 0; softmax scale 1/sqrt(d).  Host-side errors: EINVAL,
+ * with mask[b][j] != 0; softmax scale 1/sqrt(d).  A request's outputs and cache
+ * entries have the same bits alone and in any batch.  Host-side errors: EINVAL,
  * ECAPACITY (an append would exceed capacity), EUNSUPPORTED.  Values that
  * live on the device (beam_idx, positions, token ids, the mask) are checked
  * by the device; a violation makes the step write nothing further and is
@@ -220,7 +221,9 @@ int shard_step_packed(shard_t shard, kvstate_t state, const uint16_t* hidden_in,
  * is the one shard_step gives for S tokens of one request -- the same
  * rounding points, causal attention among the new tokens and over the row's
  * entries with mask != 0 -- computed with the projections as dense
- * contractions on the tensor cores, in chunks of up to 512 tokens.
+ * contractions on the tensor cores, in chunks of up to 512 tokens.  How a prompt
+ * is cut into calls moves single roundings: the sums over K and over the cache
+ * are split by the number of tokens in a chunk.
  *   hidden_in / token_ids  as shard_step (exactly one), [S] rows
  *   position_ids           dev int32 [S]
  *   attention_mask         dev uint8 [mask_len], the row's mask, mask_len >=

@@ -30,14 +30,16 @@
 // the order of the inputs: a lane's word holds inputs 8 t + 4 j .. + 3 of a
 // 32-input block (t = lane % 4), so activations are kept with each block's
 // 4-input chunks in the order 0 2 4 6 1 3 5 7 (act_pos).
-// What bounds it is the roles' own chains of barrier polls and short dependent
-// work, ~1150 cycles a step against 512 of tensor time: leaving out, one at a
-// time, the MMAs, the dequantisation's arithmetic, the epilogue's loads or the
-// copies changes a step by 2-6 %. Per launch, 512 tokens at 8B width: gate|up
-// 149 us, o 25, down 70, q|k|v 42; with three commits a step by one thread, one
-// dequantise set and suspending waits (which, with A in shared memory, ran at the
-// same ~1 us a step) and straight-line code for the outputs 225, 73 (o and down)
-// and 61.
+// What bounds it is, in the K loop, the roles' own chains of barrier polls and
+// short dependent work, ~1150 cycles a step against 512 of tensor time: leaving
+// out, one at a time, the MMAs, the dequantisation's arithmetic, the epilogue's
+// loads or the copies changes a step by 2-6 %. Before and behind the loop it is
+// filling the rings and writing the tile out, which nothing overlaps with one CTA
+// per SM: gate|up of 512 tokens at 8B width is 6 rounds of 32 steps, 72 % of its
+// 148 us; o takes 25 us, down 71, q|k|v 42 (with three commits a step by one
+// thread, one dequantise set and suspending waits, which with A in shared memory
+// ran at the same ~1 us a step, and straight-line code for the outputs 225, 73 (o
+// and down) and 61).
 // The token tile sits in the canonical K-major layout with the 128-byte
 // swizzle, as the tensor copy writes it. The
 // arithmetic is the decode projection's: exact (q - z), fp32 sums per group,

@@ -11,7 +11,7 @@
 // '~' is a split barrier: CTAs arrive after their prologue share and wait only
 // before the first attention, so the first norm and q|k|v projection overlap
 // the prologue.  '->' is dataflow: q|k|v contributors count finished units
-// per kv head (release) and an attention item waits (acquire, bounded) only
+// per kv head (release) and an attention unit waits (acquire, bounded) only
 // for its kv head's count.
 //
 // The residual stream and the projections' sums are 64-bit fixed point
@@ -36,7 +36,7 @@ constexpr int kThreads = kWarps * 32;
 
 // Dynamic shared memory: weight rings, their barriers, the op table (4L
 // entries), gate|up partial sums (when they fit), and the area: an attention
-// item's (AttnSmem), which between attentions holds the normalised rows when
+// unit's (AttnSmem), which between attentions holds the normalised rows when
 // they fit.  The host sizes the area for the step's token count.
 constexpr size_t kAttnArea = 51 * 1024;  // at least: AttnSmem at head_dim 128, checked in the kernel
 
@@ -440,10 +440,10 @@ __device__ __forceinline__ void rmsnorm_staged(const long long* X, int H, const 
 // registers and code made every step 2 to 4 % slower.
 //
 // First layer's attention phase, against the CUDA-core version before it (a warp
-// per query over 64-entry tiles in shared memory, a CTA's items one after
-// another): 70B width, 4096 entries, 1 token 38 -> 18 us, 5 tokens 113 -> 32;
-// 8B width, 8 requests of 128..2048 entries 69 -> 23, 16 packed tokens over
-// 1024 entries 73 -> 28, 5 tokens over 512 entries 20 -> 15, 1 token over 72..327
+// per query over 64-entry tiles in shared memory, a CTA's tiles one after
+// another): 70B width, 4096 entries, 1 token 38 -> 16 us, 5 tokens 113 -> 29;
+// 8B width, 8 requests of 640..1642 entries 69 -> 23, 16 packed tokens over
+// 1024 entries 73 -> 26, 5 tokens over 512 entries 20 -> 13, 1 token over 72..327
 // entries 9 -> 9 (there it is the latency of the waits).
 // ---------------------------------------------------------------------------
 // A partial is (max, sum of exp, 2 unused, unnormalised output[d]): the
@@ -562,7 +562,7 @@ __device__ __forceinline__ int rot_row(int first, int h, int i, int d) {
   return first + 16 * (h * (d >> 4) + (i >> 3)) + (i & 7);
 }
 
-// Queries q0 .. q0 + qn of an item into shared memory: a warp per query reads
+// Queries q0 .. q0 + qn of a unit into shared memory: a warp per query reads
 // the fixed-point q sums of the query's head and token, rotates them by the
 // token's position (RoPE, pairs (i, i + d/2)), scales the row by a power of
 // two and splits it into fp16 and the fp16 of what that left out.
