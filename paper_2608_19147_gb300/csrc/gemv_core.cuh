@@ -40,7 +40,7 @@ constexpr int kRingSlots = 2;  // step kernel: units in flight per warp (a deepe
 constexpr int kCtaWarps = 12;  // warps per CTA of the step kernel (3 per SM sub-partition: 168 registers a thread)
 // Warps per CTA of the standalone projection kernel, whose loop fits 128
 // registers (a warp's unit is a chain of latencies: 128256 x 4096 lm_head, 1
-// token 58.5 -> 53.4 us, 5 tokens 67 -> 60, 8 tokens 72 -> 63 against 12 warps).
+// token 58.8 -> 51.5 us, 5 tokens 67 -> 60, 8 tokens 72 -> 63 against 12 warps).
 constexpr int kGemvWarps = 16;
 
 template <int GPU>

@@ -1,8 +1,8 @@
 """GPU parity of the step's attention at the edges of its work split, against
 the oracle at the fixed bar: cache lengths around the 16-entry blocks and the
-64-entry items, query tiles of 8 (one, several, more than one pass of 64),
-rows cut into many items (merged by one CTA or shared out), whole rows as
-items (more request-head pairs than CTAs, more entries than one staged
+64-entry chunks, query tiles of 8 (one, several, more than one pass of 64),
+rows cut into many chunks (merged by one CTA or shared out; one per CTA or in
+runs), whole rows as units (more request-head pairs than CTAs, more entries than one staged
 window), entries that no query sees for a whole item, and large or tiny
 queries (their rows are scaled before they are split)."""
 import numpy as np
