@@ -371,7 +371,7 @@ int shard_create(const shard_config* cfg, const shard_weights_host* w, shard_t* 
     }
     DevBuf<uint8_t> src;
     DevBuf<int> rowmap;
-    CUDA_TRY(src.alloc(max_src + 3 * 256));
+    CUDA_TRY(src.alloc(max_src + 9 * 256));  // up to nine arrays, each at a multiple of 256
     CUDA_TRY(rowmap.alloc((size_t)sh->max_rb * kRowsPerBlock));
     for (int l = 0; l < sh->L; ++l) {
       const shard_layer_host& lw = w->layers[l];
